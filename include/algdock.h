@@ -368,7 +368,9 @@ algdock_status algdock_reduced_energies(algdock_ctx* ctx, int64_t N, const float
  * form from f = 0, with gauge f_0 = 0:
  *   f_i <- -ln sum_n exp(-u_in) / sum_k N_k exp(f_k - u_kn)
  * until max_i |change| < tol or max_iter iterations.  u_kn [K][N] double (device), N_k [K] int64
- * (host).  precision_mode 0: FP64 throughout; 1: exponentials in FP32 of FP64 arguments, sums in
+ * (host).  precision_mode 0: FP64 throughout (with every N_k > 0 and K <= 256 the iteration runs on
+ * stored weights, K*N*8 bytes of scratch where at most half of the free memory, kept with the context
+ * up to 4 GiB); 1: exponentials in FP32 of FP64 arguments, sums in
  * FP64; 2: each sample's column shifted by its minimum (FP64, exact in the result) and stored as
  * FP32, then FP32 arguments, exponentials and Kahan-compensated sums, FP64 only where partial sums
  * meet (K <= 16384; extra scratch K*N*4 bytes).  K <= 65535 in every mode.  tol = 0, max_iter = 0
@@ -682,8 +684,8 @@ algdock_status algdock_checkpoint_load(algdock_ctx* ctx, const char* path, uint6
 /* MBAR without any device allocation.  The paper has no counterpart: this is a service of this
  * library for callers that cannot call cudaMalloc - for example a host framework whose caching
  * allocator owns all device memory and forbids direct allocations, or a service that reserves its
- * whole memory budget at start-up.  Same arguments, arithmetic and results as algdock_mbar for
- * precision modes 0 and 1, but the solver's scratch is a fixed 8 MiB array in the library's own
+ * whole memory budget at start-up.  Same arguments and results (to FP64 rounding) as algdock_mbar for
+ * precision modes 0 and 1, always in log-sum-exp form, but the solver's scratch is a fixed 8 MiB array in the library's own
  * device memory (every GPU that loads the library holds it until the process exits); the call
  * itself allocates nothing and does not use the context's own MBAR scratch.
  *  - precision_mode 2 is rejected (ALGDOCK_E_INVALID with its own message): its FP32 copy of

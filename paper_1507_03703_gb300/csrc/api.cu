@@ -23,7 +23,11 @@ size_t mbar_pairs_scratch_bytes(int K, int64_t N);
 cudaError_t mbar_local_pairs(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn,
                              const int64_t* Nk_host, const double* f_host, int mode, double* pairs_host);
 int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn, const int64_t* Nk_host,
-             double tol, int max_iter, int mode, double* f_host, int* iters, int* h_flag, cudaError_t* err);
+             double tol, int max_iter, int mode, bool weights, double* f_host, int* iters, int* h_flag,
+             cudaError_t* err);
+bool mbar_takes_weights(int K, const int64_t* Nk_host);
+size_t mbar_weights_bytes(int K, int64_t N);
+size_t mbar_scratch_bytes_weights(int K, int64_t N);
 }  // namespace algdock
 
 using namespace algdock;
@@ -850,7 +854,7 @@ algdock_status algdock_create(int device, uint64_t seed, const algdock_params* p
     coherent = mappable = 0;
   }
   c->host_coherent = coherent && mappable;
-  if (cudaMallocHost(&c->h_flag, sizeof(int)) != cudaSuccess) {
+  if (cudaMallocHost(&c->h_flag, kMbarFlagBytes) != cudaSuccess) {
     delete c;
     return ALGDOCK_E_CUDA;
   }
@@ -1864,7 +1868,15 @@ algdock_status algdock_mbar(algdock_ctx* c, int32_t K, int64_t N, const double* 
   }
   if (total != N) return fail(c, ALGDOCK_E_INVALID, "mbar: sum of N_k must equal N");
   Device g(c->device);
-  const size_t need = mbar_scratch_bytes_mode(K, N, precision_mode);
+  size_t need = mbar_scratch_bytes_mode(K, N, precision_mode);
+  // FP64 mode on stored weights (K N doubles) where they take at most half of the free memory
+  bool weights = precision_mode == 0 && mbar_takes_weights(K, N_k);
+  const size_t with_weights = weights ? mbar_scratch_bytes_weights(K, N) : 0;
+  if (with_weights > c->mbar_bytes) {
+    size_t free_b = 0, total_b = 0;
+    weights = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && mbar_weights_bytes(K, N) <= free_b / 2;
+  }
+  if (weights) need = with_weights;
   if (need > c->mbar_bytes) {
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "mbar");
@@ -1872,13 +1884,24 @@ algdock_status algdock_mbar(algdock_ctx* c, int32_t K, int64_t N, const double* 
     c->d_mbar = nullptr;
     c->mbar_bytes = 0;
     e = cudaMalloc(&c->d_mbar, need);
+    if (e == cudaErrorMemoryAllocation && weights) {  // fragmented or taken meanwhile: without the weights
+      cudaGetLastError();
+      weights = false;
+      need = mbar_scratch_bytes_mode(K, N, precision_mode);
+      e = cudaMalloc(&c->d_mbar, need);
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "mbar");
     c->mbar_bytes = need;
   }
   cudaError_t err = cudaSuccess;
   int it = 0;
-  const int r = mbar_run(c->stream, c->d_mbar, K, N, u_kn, N_k, tol, max_iter, precision_mode, f_k, &it, c->h_flag,
-                         &err);
+  const int r = mbar_run(c->stream, c->d_mbar, K, N, u_kn, N_k, tol, max_iter, precision_mode, weights, f_k, &it,
+                         c->h_flag, &err);
+  if (weights && c->mbar_bytes > kMbarKeepBytes) {  // the weights of a very large solve are given back
+    cudaFree(c->d_mbar);
+    c->d_mbar = nullptr;
+    c->mbar_bytes = 0;
+  }
   *iters = it;
   if (r < 0) return cuda_fail(c, err, "mbar");
   if (r == 1) return fail(c, ALGDOCK_E_NOT_CONVERGED, "mbar: max_iter reached");

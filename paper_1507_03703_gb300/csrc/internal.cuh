@@ -32,6 +32,8 @@ constexpr double kRepulsiveMinDist = 0.01;         // A
 constexpr double kAttractiveMinDist = 2.0;         // A
 constexpr int kMaxAtoms = 96;                      // 3 atoms per lane of one warp
 constexpr int kMaxLadder = 1024;
+constexpr size_t kMbarFlagBytes = 16;              // pinned words a context polls device flags in
+constexpr size_t kMbarKeepBytes = (size_t)4 << 30;  // MBAR scratch with stored weights kept between solves
 constexpr int kMbarMaxStates = 65535;             // MBAR's state_partials grid has one y-index per state
 
 // Two FP32 values in one 64-bit register pair, for the paired FP32 instructions of sm_100-class
@@ -255,7 +257,7 @@ struct algdock_ctx {
   // scratch owned by the MBAR solver, grown on demand
   void* d_mbar = nullptr;
   size_t mbar_bytes = 0;
-  // pinned host word for convergence polling
+  // pinned host words for convergence polling (kMbarFlagBytes)
   int* h_flag = nullptr;
   // work counter of the single-ligand HMC launch (replicas handed out to warps; zeroed per launch)
   unsigned long long* d_work = nullptr;

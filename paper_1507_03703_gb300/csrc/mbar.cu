@@ -8,8 +8,13 @@
 //   4. finalize:         gauge f_0 = 0, convergence flag                             (one block)
 // Every kernel returns at once when the device flag says the iteration has converged, so the host
 // can enqueue iterations in batches and poll the flag between batches.
+//
+// algdock_mbar's FP64 mode runs the same iteration on stored weights (see "FP64 on stored weights"
+// below): the exponentials are formed once per solve instead of twice per iteration.
+#include <limits.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -31,7 +36,8 @@ inline int64_t mbar_chunk(int K, int64_t N) {
 struct MbarState {
   int converged;
   int iters;
-  int _pad[2];
+  int trip;    // weights path: the iteration left the range the stored weights are exact in
+  int ticket;  // weights path: blocks of weight_update that have finished
 };
 
 // Online log-sum-exp accumulator: value = m + log(s).
@@ -325,10 +331,241 @@ __global__ void init_state(int K, const int64_t* Nk, double* logNk, double* f, M
   if (threadIdx.x == 0) {
     st->converged = 0;
     st->iters = 0;
+    st->trip = 0;
+    st->ticket = 0;
   }
 }
 
+// ---------------------------------------------------------------- FP64 on stored weights
+// With W_kn = exp(g_k - u_kn - c_n) stored once, an iteration of f needs no exponential per
+// element: with a_k = N_k exp(f_k - g_k),
+//   D'_n = sum_k a_k W_kn,   f_k <- g_k - ln sum_n W_kn / D'_n
+// (the shifts c_n cancel, and so does a factor common to all a_k).  Two FP64 multiply-adds per
+// element and iteration remain, which is what bounds it: GB300 issues 2 FP64 lanes per clock and
+// SM, so K = 128, N = 102400 cannot take less than 42 us an iteration (its 105 MB of weights take
+// 15 us from HBM).  Measured: a solve of 43 iterations at that size 88.5 -> 3.94 ms (two log-sum-exp
+// passes with an FP64 exponential per element take 1455 us an iteration), and 25.9 -> 1.58 ms an
+// iteration, the forming of the weights included, at K = 256, N = 1e6.
+//
+// Range.  c_n is the column's maximum (to 2^-20 relative), so the largest weight of a column is 1
+// and only weights below 1e-308 of it are lost.  While the spread of f - g stays within kMaxSpread,
+// D'_n >= N_k exp(-200) and the lost terms are below 1e-120 of any sum of at least kMinSum.  An
+// iteration outside these limits is not applied (trip): the host then runs one log-sum-exp
+// iteration from the same f, takes g = f and forms the weights again.  A ladder whose reduced
+// energies span several hundred kT takes this turn once, at the start from f = 0.
+constexpr int kWTile = 32;             // samples of a tile: W is stored [tile][K][32], zero past N
+constexpr int kWStates = 32;           // states per warp at most
+constexpr int kWMaxStates = 256;       // eight warps
+constexpr double kMaxSpread = 200.0;   // of f - g
+constexpr double kMinSum = 1e-150;     // of sum_n W_kn / D'_n
+
+// One block per tile: lane = sample, each warp every eighth state.
+__global__ void __launch_bounds__(256) build_weights(int K, int64_t N, const double* __restrict__ u,
+                                                     const double* __restrict__ g, double* __restrict__ W) {
+  __shared__ int s_key[8][kWTile];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t n = (int64_t)blockIdx.x * kWTile + lane;
+  const bool in = n < N;
+  const double* col = u + (in ? n : N - 1);
+  // the maximum from the high words alone: as signed integers, with the lower 31 bits of a
+  // negative one inverted, they order as the doubles do
+  int key = INT_MIN;
+  for (int k = warp; k < K; k += 8) {
+    const int hi = __double2hiint(g[k] - __ldg(col + (int64_t)k * N));
+    key = max(key, hi ^ ((hi >> 31) & 0x7fffffff));
+  }
+  s_key[warp][lane] = key;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) key = max(key, s_key[w][lane]);
+  const double c = __hiloint2double(key ^ ((key >> 31) & 0x7fffffff), 0);
+  double* out = W + (int64_t)blockIdx.x * K * kWTile + lane;
+  for (int k = warp; k < K; k += 8)
+    out[(int64_t)k * kWTile] = in ? exp((g[k] - __ldg(col + (int64_t)k * N)) - c) : 0.0;
+}
+
+// The sums of one iteration.  A block takes tiles blockIdx.x, + gridDim.x, ...: the tile goes to
+// shared memory once and serves both passes, D'_n (each warp its states, then one warp adds the
+// warps' parts) and the state sums, which stay in registers (lane = sample) over all the block's
+// tiles.  Several blocks per SM, so that one loads while another computes.  The reduction of the 32
+// accumulators over the lanes halves their number at each step (31 FP64 additions instead of 160:
+// at 2 lanes per clock these count).  part[k][block].
+template <int NW>
+__global__ void __launch_bounds__(32 * NW) weight_pass(int K, int64_t N, const double* __restrict__ W,
+                                                       const double* __restrict__ a, double* __restrict__ part,
+                                                       const MbarState* st) {
+  if (st->converged || st->trip) return;
+  extern __shared__ __align__(16) double s_w[];  // [K][32], then a [K]
+  __shared__ double s_part[NW][kWTile];
+  __shared__ double s_r[kWTile];
+  double* s_a = s_w + K * kWTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (K + NW - 1) / NW;  // <= kWStates
+  const int k0 = warp * per, kn = max(0, min(per, K - k0));
+  for (int k = threadIdx.x; k < K; k += 32 * NW) s_a[k] = a[k];
+  double acc[kWStates];
+#pragma unroll
+  for (int j = 0; j < kWStates; ++j) acc[j] = 0.0;
+  const int64_t tiles = (N + kWTile - 1) / kWTile;
+  const double* mine = s_w + k0 * kWTile + lane;
+  const double* my_a = s_a + k0;
+  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const char* src = (const char*)(W + t * K * kWTile);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_w);
+    for (int i = threadIdx.x; i < K * kWTile / 2; i += 32 * NW)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 16 * i) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+    for (int j = 0; j < kWStates; j += 2) {
+      if (j < kn) d0 = fma(my_a[j], mine[j * kWTile], d0);
+      if (j + 1 < kn) d1 = fma(my_a[j + 1], mine[(j + 1) * kWTile], d1);
+    }
+    s_part[warp][lane] = d0 + d1;
+    __syncthreads();
+    if (warp == (int)(t % NW)) {
+      double d = s_part[0][lane];
+#pragma unroll
+      for (int w = 1; w < NW; ++w) d += s_part[w][lane];
+      s_r[lane] = t * kWTile + lane < N ? 1.0 / d : 0.0;
+    }
+    __syncthreads();
+    const double r = s_r[lane];
+#pragma unroll
+    for (int j = 0; j < kWStates; ++j)
+      if (j < kn) acc[j] = fma(mine[j * kWTile], r, acc[j]);
+    __syncthreads();  // the tile and s_r are free again
+  }
+  // lane l ends with the sum of accumulator l over all lanes
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      const double give = up ? acc[j] : acc[j + o], keep = up ? acc[j + o] : acc[j];
+      acc[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  if (lane < kn) part[(int64_t)(k0 + lane) * gridDim.x + blockIdx.x] = acc[0];
+}
+
+// Each state's block sums added by one warp; the last block to finish applies the gauge f_0 = 0, the
+// limits above, the convergence test, and the factors a of the next iteration.
+__global__ void __launch_bounds__(128) weight_update(int K, int n_part, const double* __restrict__ part,
+                                                     const int64_t* __restrict__ Nk, const double* __restrict__ g,
+                                                     double* f, double* fnew, double* a, MbarState* st, double tol,
+                                                     int max_iter) {
+  if (st->converged || st->trip) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k = blockIdx.x * 4 + warp;
+  if (k < K) {
+    const double* p = part + (int64_t)k * n_part;
+    double s = 0.0;
+    for (int b = lane; b < n_part; b += 32) s += p[b];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    // a sum outside the limits (or NaN) becomes a NaN that trips below
+    if (lane == 0) fnew[k] = s >= kMinSum && s <= 1.0 / kMinSum ? g[k] - log(s) : NAN;
+  }
+  __shared__ bool s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&st->ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // thread t holds states t and t + 128
+  __shared__ double s_max[4], s_top[4], s_bot[4];
+  const double f0 = __ldcg(fnew);
+  double v[2], x[2], delta = 0.0, top = -INFINITY, bot = INFINITY;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int i = threadIdx.x + 128 * j;
+    v[j] = x[j] = 0.0;
+    if (i >= K) continue;
+    v[j] = __ldcg(fnew + i) - f0;
+    x[j] = v[j] - g[i];
+    const double d = fabs(v[j] - f[i]);
+    delta = (d > delta || isnan(d)) ? d : delta;
+    top = fmax(top, x[j]);
+    bot = fmin(bot, x[j]);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double d = __shfl_xor_sync(0xffffffffu, delta, o);
+    delta = (d > delta || isnan(d)) ? d : delta;
+    top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    bot = fmin(bot, __shfl_xor_sync(0xffffffffu, bot, o));
+  }
+  if (lane == 0) {
+    s_max[warp] = delta;
+    s_top[warp] = top;
+    s_bot[warp] = bot;
+  }
+  __syncthreads();
+  for (int w = 0; w < 4; ++w) {
+    delta = (s_max[w] > delta || isnan(s_max[w])) ? s_max[w] : delta;
+    top = fmax(top, s_top[w]);
+    bot = fmin(bot, s_bot[w]);
+  }
+  const bool good = isfinite(delta) && top - bot <= kMaxSpread;
+  if (good) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int i = threadIdx.x + 128 * j;
+      if (i >= K) continue;
+      f[i] = v[j];
+      a[i] = (double)Nk[i] * exp(x[j] - top);
+    }
+  }
+  if (threadIdx.x == 0) {
+    st->ticket = 0;
+    if (!good) {
+      st->trip = 1;
+    } else {
+      st->iters += 1;
+      if (delta < tol) st->converged = 1;
+      else if (st->iters >= max_iter) st->converged = 2;
+    }
+  }
+}
+
+// g = f (or 0 at the start, where f is 0) and the factors that go with it; the trip is cleared.
+__global__ void weight_base(int K, const int64_t* __restrict__ Nk, const double* __restrict__ f, double* g, double* a,
+                            MbarState* st) {
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    g[k] = f[k];
+    a[k] = (double)Nk[k];
+  }
+  if (threadIdx.x == 0) st->trip = 0;
+}
+
+// Blocks of a weight_pass launch: three per SM of four warps (two of eight), no more than tiles.
+int weight_blocks(int K, int64_t N) {
+  const int64_t tiles = (N + kWTile - 1) / kWTile;
+  return (int)std::min<int64_t>(tiles, 152 * (K <= 128 ? 3 : 2));
+}
+
+size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
+
 }  // namespace
+
+// The weights path takes every state sampled (an unsampled state's weights have no bound) and up to
+// 256 states.
+bool mbar_takes_weights(int K, const int64_t* Nk_host) {
+  if (K > kWMaxStates) return false;
+  for (int k = 0; k < K; ++k)
+    if (Nk_host[k] <= 0) return false;
+  return true;
+}
+// Scratch of the weights path: the log-sum-exp solver's, then g[K] | a[K] | part[K][blocks] | W.
+size_t mbar_weights_bytes(int K, int64_t N) {
+  return (size_t)((N + kWTile - 1) / kWTile) * K * kWTile * sizeof(double);
+}
+size_t mbar_scratch_bytes(int K, int64_t N);
+size_t mbar_scratch_bytes_weights(int K, int64_t N) {
+  return align256(mbar_scratch_bytes(K, N)) + align256(16 * (size_t)K) +
+         align256((size_t)K * weight_blocks(K, N) * sizeof(double)) + mbar_weights_bytes(K, N);
+}
 
 // Scratch layout (bytes): MbarState | logNk[K] | f[K] | fnew[K] | Nk[K] (int64) | part[K][n_chunks] | logD[N]
 // (double; float in mode 2), then in mode 2 the shifted FP32 copy w[K][N] (256-byte aligned).
@@ -377,10 +614,14 @@ cudaError_t mbar_local_pairs(cudaStream_t s, void* scratch, int K, int64_t N, co
 }
 
 // Runs the solver on caller-provided scratch (mbar_scratch_bytes(K, N) bytes, 256-byte aligned).
-// h_flag: pinned host int used to poll the device flag.  Returns 0 converged, 1 not converged,
-// -1 on a CUDA error (then *err is set).
+// h_flag: kMbarFlagBytes of pinned host memory used to poll the device state.  weights: iterate on
+// stored weights (mode 0, mbar_takes_weights; scratch mbar_scratch_bytes_weights).  Returns 0
+// converged, 1 not converged, -1 on a CUDA error (then *err is set).
 int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn, const int64_t* Nk_host,
-             double tol, int max_iter, int mode, double* f_host, int* iters, int* h_flag, cudaError_t* err) {
+             double tol, int max_iter, int mode, bool weights, double* f_host, int* iters, int* h_flag,
+             cudaError_t* err) {
+  static_assert(sizeof(MbarState) <= kMbarFlagBytes, "the polled state fits the pinned words");
+  MbarState* h_state = (MbarState*)h_flag;
   const int64_t chunk_len = mbar_chunk(K, N);
   const int64_t n_chunks = (N + chunk_len - 1) / chunk_len;
   char* p = (char*)scratch;
@@ -406,31 +647,74 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
                              (int)(K * sizeof(float)));
     if (e != cudaSuccess) { *err = e; return -1; }
   }
+  auto iterate = [&] {  // one log-sum-exp iteration
+    if (mode == 2) {
+      log_denominators_f32<<<blocks_n, threads, K * sizeof(float), s>>>(K, N, w32, logNk, f, (float*)logD, st);
+      state_partials_f32<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, w32, (const float*)logD, part, (int)n_chunks,
+                                                            st);
+    } else {
+      log_denominators<<<blocks_n, threads, 0, s>>>(K, N, u_kn, logNk, f, logD, st, mode);
+      state_partials<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, u_kn, logD, part, (int)n_chunks, st, mode);
+    }
+    const unsigned merge_blocks = (unsigned)((K * 32 + 255) / 256);
+    if (mode == 2)
+      merge_chunks<true><<<merge_blocks, 256, 0, s>>>(K, (int)n_chunks, part, fnew, st);
+    else
+      merge_chunks<false><<<merge_blocks, 256, 0, s>>>(K, (int)n_chunks, part, fnew, st);
+    finalize<<<1, 256, 0, s>>>(K, f, fnew, st, tol, max_iter);
+  };
+  auto poll = [&] {  // the device state into h_state
+    cudaError_t q = cudaGetLastError();
+    if (q == cudaSuccess) q = cudaMemcpyAsync(h_state, st, sizeof(MbarState), cudaMemcpyDeviceToHost, s);
+    if (q == cudaSuccess) q = cudaStreamSynchronize(s);
+    return q;
+  };
   int done = 0;
   int issued = 0;
   int batch = 4;
-  while (!done) {
-    for (int b = 0; b < batch && issued < max_iter; ++b, ++issued) {
-      if (mode == 2) {
-        log_denominators_f32<<<blocks_n, threads, K * sizeof(float), s>>>(K, N, w32, logNk, f, (float*)logD, st);
-        state_partials_f32<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, w32, (const float*)logD, part,
-                                                              (int)n_chunks, st);
-      } else {
-        log_denominators<<<blocks_n, threads, 0, s>>>(K, N, u_kn, logNk, f, logD, st, mode);
-        state_partials<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, u_kn, logD, part, (int)n_chunks, st, mode);
-      }
-      const unsigned merge_blocks = (unsigned)((K * 32 + 255) / 256);
-      if (mode == 2)
-        merge_chunks<true><<<merge_blocks, 256, 0, s>>>(K, (int)n_chunks, part, fnew, st);
-      else
-        merge_chunks<false><<<merge_blocks, 256, 0, s>>>(K, (int)n_chunks, part, fnew, st);
-      finalize<<<1, 256, 0, s>>>(K, f, fnew, st, tol, max_iter);
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_flag, &st->converged, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (weights) {
+    char* q = p + align256(mbar_scratch_bytes(K, N));
+    double* g = (double*)q;
+    double* a = g + K;
+    double* wpart = (double*)(q + align256(16 * (size_t)K));
+    const int blocks = weight_blocks(K, N);
+    double* W = (double*)((char*)wpart + align256((size_t)K * blocks * sizeof(double)));
+    const size_t smem = (size_t)K * (kWTile + 1) * sizeof(double);
+    const bool wide = K > 128;
+    e = cudaFuncSetAttribute(wide ? weight_pass<8> : weight_pass<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
     if (e != cudaSuccess) { *err = e; return -1; }
-    done = (*h_flag != 0) || issued >= max_iter;
+    while (!done) {
+      const int applied = issued;  // iterations applied when the weights were last formed
+      weight_base<<<1, 256, 0, s>>>(K, Nk, f, g, a, st);
+      build_weights<<<(unsigned)((N + kWTile - 1) / kWTile), 256, 0, s>>>(K, N, u_kn, g, W);
+      for (bool trip = false; !done && !trip;) {
+        for (int b = 0; b < batch && issued < max_iter; ++b, ++issued) {
+          if (wide) weight_pass<8><<<blocks, 256, smem, s>>>(K, N, W, a, wpart, st);
+          else weight_pass<4><<<blocks, 128, smem, s>>>(K, N, W, a, wpart, st);
+          weight_update<<<(unsigned)((K + 3) / 4), 128, 0, s>>>(K, blocks, wpart, Nk, g, f, fnew, a, st, tol, max_iter);
+        }
+        e = poll();
+        if (e != cudaSuccess) { *err = e; return -1; }
+        trip = h_state->trip != 0;
+        issued = trip ? h_state->iters : issued;
+        done = h_state->converged != 0 || issued >= max_iter;
+        if (batch < 64) batch *= 2;
+      }
+      if (done) break;
+      const bool moved = issued > applied;
+      iterate();
+      ++issued;
+      if (issued >= max_iter) done = 1;
+      if (!moved && applied > 0) break;  // tripped twice in a row
+    }
+    batch = 4;
+  }
+  while (!done) {
+    for (int b = 0; b < batch && issued < max_iter; ++b, ++issued) iterate();
+    e = poll();
+    if (e != cudaSuccess) { *err = e; return -1; }
+    done = h_state->converged != 0 || issued >= max_iter;
     if (batch < 64) batch *= 2;
   }
   MbarState hs;
@@ -531,7 +815,7 @@ extern "C" algdock_status algdock_mbar_noalloc(algdock_ctx* c, int32_t K, int64_
     cudaError_t err = cudaSuccess;
     int it = 0;
     int r = -1;
-    if (e == cudaSuccess) r = algdock::mbar_run(c->stream, scratch, K, N, u_kn, N_k, tol, max_iter, precision_mode,
+    if (e == cudaSuccess) r = algdock::mbar_run(c->stream, scratch, K, N, u_kn, N_k, tol, max_iter, precision_mode, false,
                                                 f_k, &it, c->h_flag, &err);
     else err = e;
     if (prev >= 0 && prev != c->device) cudaSetDevice(prev);
