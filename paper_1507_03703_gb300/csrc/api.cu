@@ -709,8 +709,9 @@ algdock_status build_ligand(algdock_ctx* c, const algdock_ligand* L, const algdo
     G.off_bond = 6 * na;
     G.off_ang = G.off_bond + 4 * nb;
     G.off_tor = G.off_ang + 5 * nang;
-    G.off_ptype = G.off_tor + 10 * ntor;
-    G.n_doubles = G.off_ptype + na * na;
+    G.off_pair = G.off_tor + kTor64 * ntor;
+    const int n_pairs = na * (na - 1) / 2;
+    G.n_doubles = G.off_pair + 3 * n_pairs;
     d.assign(G.n_doubles > 0 ? G.n_doubles : 1, 0.0);
     for (int i = 0; i < na; ++i) {
       const double two_r = 2.0 * L->rstar[i];
@@ -722,29 +723,41 @@ algdock_status build_ligand(algdock_ctx* c, const algdock_ligand* L, const algdo
       a[4] = L->rstar[i];
       a[5] = sqrt(L->eps[i]);
     }
-    for (int t = 0; t < nb; ++t) {
-      double* b = &d[G.off_bond + 4 * t];
+    for (int p = 0; p < nb; ++p) {
+      const int t = P.term_at[0][p];
+      double* b = &d[G.off_bond + 4 * p];
       b[0] = L->bonds[2 * t];
       b[1] = L->bonds[2 * t + 1];
       b[2] = L->bond_k[t];
       b[3] = L->bond_r0[t];
     }
-    for (int t = 0; t < nang; ++t) {
-      double* a = &d[G.off_ang + 5 * t];
+    for (int p = 0; p < nang; ++p) {
+      const int t = P.term_at[1][p];
+      double* a = &d[G.off_ang + 5 * p];
       for (int k = 0; k < 3; ++k) a[k] = L->angles[3 * t + k];
       a[3] = L->angle_k[t];
       a[4] = L->angle_theta0[t];
     }
-    for (int t = 0; t < ntor; ++t) {
-      double* q = &d[G.off_tor + 10 * t];
+    for (int p = 0; p < ntor; ++p) {
+      const int t = P.term_at[2][p];
+      double* q = &d[G.off_tor + kTor64 * p];
       for (int k = 0; k < 4; ++k) q[k] = L->torsions[4 * t + k];
       for (int m = 0; m < 3; ++m) {
         q[4 + m] = 0.5 * L->torsion_V[3 * t + m];
-        q[7 + m] = L->torsion_gamma[3 * t + m];
+        q[7 + m] = cos(L->torsion_gamma[3 * t + m]);
+        q[10 + m] = sin(L->torsion_gamma[3 * t + m]);
       }
     }
-    for (int j = 0; j < na; ++j)
-      for (int i = 0; i < na; ++i) d[G.off_ptype + (size_t)j * na + i] = ptype[(size_t)j * na + i];
+    for (int p = 0; p < n_pairs; ++p) {
+      const int i = p % na, j = (i + 1 + p / na) % na;
+      const int ty = ptype[(size_t)j * na + i];
+      const double s_lj = ty == 1 ? 0.5 : 1.0, s_el = ty == 1 ? 1.0 / 1.2 : 1.0;
+      const double R = L->rstar[i] + L->rstar[j];
+      double* q = &d[G.off_pair + p];
+      q[0] = ty == 2 ? -1.0 : R * R;
+      q[n_pairs] = ty == 2 ? 0.0 : 12.0 * s_lj * sqrt(L->eps[i]) * sqrt(L->eps[j]);
+      q[2 * n_pairs] = ty == 2 ? 0.0 : s_el * kCoulomb * L->charge[i] * L->charge[j];
+    }
     double M = 0.0;
     for (int i = 0; i < na; ++i) M += L->mass[i];
     G.total_mass = M;

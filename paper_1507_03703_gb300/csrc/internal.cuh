@@ -174,14 +174,17 @@ struct __align__(16) ReceptorPair {
 };
 
 // The all-FP64 evaluation path (the precision study's FP64 arm): the ligand's parameters in FP64,
-// as offsets (in doubles) into one device buffer, and FP64 lattices.
+// as offsets (in doubles) into one device buffer, and FP64 lattices.  Bonded terms sit at their
+// gather-plan positions, as in the FP32 blob.
+constexpr int kTor64 = 13;
 struct Lig64 {
   int na, nb, nang, ntor;
   int off_atom;   // [na][6]: mass, q, sqrt(A), sqrt(B), R*, sqrt(eps)
   int off_bond;   // [nb][4]: i, j (as doubles), k, r0
   int off_ang;    // [nang][5]: i, j, k, k_theta, theta0
-  int off_tor;    // [ntor][10]: i, j, k, l, V1/2, V2/2, V3/2, gamma1, gamma2, gamma3
-  int off_ptype;  // [na][na] pair types as doubles: 0 nonbonded, 1 1-4, 2 excluded
+  int off_tor;    // [ntor][kTor64]: i, j, k, l, V1/2, V2/2, V3/2, cos(gamma1..3), sin(gamma1..3)
+  int off_pair;   // [3][na (na - 1) / 2]: (R*_i + R*_j)^2 (-1: excluded), 12 eps_ij s_lj, 332 q_i q_j s_el of
+                  // pair p: i = p mod na, j = (i + 1 + p / na) mod na
   int n_doubles;
   double total_mass, site[3], k_rest, d0;
 };

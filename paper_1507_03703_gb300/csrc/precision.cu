@@ -1,15 +1,35 @@
 // The all-FP64 evaluation path: the energy components and forces of stored configurations with
 // every operation in FP64, on FP64 lattices and FP64 parameters.  It is the FP64 arm of the
 // precision study of the FP32 path (grid interaction, "Thermodynamic Cycle"; the ligand force
-// field; the restraint, Eq. (binding_site); the state weights, Eq. (protocol)).  One thread
-// evaluates one configuration; throughput is not its purpose, and GB300's FP64 rate is a small
-// fraction of its FP32 rate.
+// field; the restraint, Eq. (binding_site); the state weights, Eq. (protocol)).
+//
+// GB300 issues 2 FP64 lanes per clock and SM (a warp instruction takes a scheduler 64 cycles), so
+// the kernel is bound by the number of FP64 warp instructions and by nothing else.  One warp per
+// configuration, with every stage laid out so that the lanes are full and each term is computed
+// once:
+//   1. bonded terms, one per lane, their forces to slots that are then added over the balanced
+//      runs of the FP32 kernel's gather schedule;
+//   2. nonbonded pairs, each unordered pair once: pair index p is (i, i + d mod n) with d = 1 + p/n,
+//      i = p mod n, so 32 consecutive pairs have 32 different i and 32 different j, and the forces
+//      on both are added in shared memory without conflict (a ligand of fewer than 32 atoms takes
+//      one d at a time);
+//   3. per atom: the five interpolated channels, edge differences along x, then y, then z.
+// Reciprocal square roots take the place of square roots and divisions (the pair loop's from an
+// FP32 seed by one third-order step), torsions the multiple-angle polynomials of cos(phi), sin(phi).
+// 8192 configurations of 48 atoms take 1.25 ms with the FP64 pipe 86 % busy.  With one thread per
+// configuration (64 blocks, square roots, divisions, atan2, sincos, and forces added in global
+// memory) they took 5.67 ms.  Two configurations per block or four make no difference at that size;
+// two leave more blocks to a small one.
 #include <math.h>
 
 #include "internal.cuh"
 
 namespace algdock {
 namespace {
+
+constexpr int kWarps64 = 2;  // configurations per block, fewer where their shared memory does not fit
+constexpr size_t kMaxSmem64 = 227 * 1024;
+constexpr unsigned kFull = 0xffffffffu;
 
 struct V3 {
   double x, y, z;
@@ -20,19 +40,46 @@ __device__ inline V3 operator*(double s, V3 a) { return V3{s * a.x, s * a.y, s *
 __device__ inline double dot3(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ inline V3 cross3(V3 a, V3 b) { return V3{a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x}; }
 
-// Per-configuration views: positions (converted once to FP64 in the force array's slot) and the
-// force accumulator, both [na][3] in global memory owned by this thread.
-struct Conf {
-  const float* x;
-  double* f;  // may be null (energies only)
-  __device__ V3 pos(int i) const { return V3{(double)x[3 * i], (double)x[3 * i + 1], (double)x[3 * i + 2]}; }
-  __device__ void add(int i, V3 v) const {
-    if (!f) return;
-    f[3 * i] += v.x;
-    f[3 * i + 1] += v.y;
-    f[3 * i + 2] += v.z;
+__device__ inline double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+// 1 / sqrt(v) from an FP32 seed y (error e = 1 - v y^2 about 2^-22) by the third-order step
+// y (1 + e/2 + 3 e^2/8), whose error 5 e^3/16 is below FP64 rounding.
+__device__ inline double rsqrt_step(double v) {
+  const double y = (double)rsqrtf((float)v);
+  const double e = fma(-(v * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// A warp's shared memory: positions [3][na], forces [3][na], bonded slots [3][n_slots + 1] (the last
+// one zero).  A topology with more slots than fit (9000 and more; s null) adds its bonded forces
+// by shared-memory atomics instead.
+struct Warp64 {
+  double *x, *f, *s;
+  int na, ns;
+  __device__ V3 pos(int i) const { return V3{x[i], x[na + i], x[2 * na + i]}; }
+  __device__ V3 slot(int i) const { return V3{s[i], s[ns + i], s[2 * ns + i]}; }
+  __device__ void put(int i, V3 v) const {
+    s[i] = v.x;
+    s[ns + i] = v.y;
+    s[2 * ns + i] = v.z;
+  }
+  // the force of a bonded term's slot i on an atom
+  __device__ void put(int i, int atom, V3 v) const {
+    if (s) {
+      put(i, v);
+    } else {
+      atomicAdd(f + atom, v.x);
+      atomicAdd(f + na + atom, v.y);
+      atomicAdd(f + 2 * na + atom, v.z);
+    }
   }
 };
+__host__ __device__ inline int warp64_doubles(int na, int n_slots, bool slots) {
+  return 6 * na + (slots ? 3 * (n_slots + 1) : 0);
+}
 
 // Trilinear value and gradient of lattice channel ch at p; coordinates outside the lattice are
 // clamped to it, and the gradient along a clamped axis is zero.
@@ -66,158 +113,270 @@ __device__ inline Interp locate(const GridDev64& G, V3 p) {
   return I;
 }
 
-template <typename Get>
-__device__ inline double trilinear(const GridDev64& G, const Interp& I, Get get, V3* grad) {
-  const int64_t sy = G.nx, sz = (int64_t)G.nx * G.ny;
-  double v = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-  for (int e = 0; e < 2; ++e)
-    for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 2; ++a) {
-        const double node = get(I.b + e * sz + b * sy + a);
-        const double wx = a ? I.t[0] : 1.0 - I.t[0], wy = b ? I.t[1] : 1.0 - I.t[1],
-                     wz = e ? I.t[2] : 1.0 - I.t[2];
-        const double dx = a ? 1.0 : -1.0, dy = b ? 1.0 : -1.0, dz = e ? 1.0 : -1.0;
-        v += wx * wy * wz * node;
-        gx += dx * wy * wz * node;
-        gy += wx * dy * wz * node;
-        gz += wx * wy * dz * node;
-      }
-  *grad = V3{I.in[0] ? gx / G.h : 0.0, I.in[1] ? gy / G.h : 0.0, I.in[2] ? gz / G.h : 0.0};
-  return v;
+// a (1 - t) + b t with both products, so that a large corner value far away in t leaves no error of
+// its own size.
+__device__ inline double lerp64(double a, double b, double t) { return fma(t, b, fma(-t, a, a)); }
+
+// Value and gradient in lattice units from the corner values c[z][y][x].
+__device__ inline double trilinear(const double (&c)[8], const double (&t)[3], V3& g) {
+  const double d0 = c[1] - c[0], d1 = c[3] - c[2], d2 = c[5] - c[4], d3 = c[7] - c[6];
+  const double a0 = lerp64(c[0], c[1], t[0]), a1 = lerp64(c[2], c[3], t[0]);
+  const double a2 = lerp64(c[4], c[5], t[0]), a3 = lerp64(c[6], c[7], t[0]);
+  const double y0 = a1 - a0, y1 = a3 - a2;
+  const double b0 = lerp64(a0, a1, t[1]), b1 = lerp64(a2, a3, t[1]);
+  const double x0 = fma(t[1], d1 - d0, d0), x1 = fma(t[1], d3 - d2, d2);
+  g.z = b1 - b0;
+  g.x = fma(t[2], x1 - x0, x0);
+  g.y = fma(t[2], y1 - y0, y0);
+  return lerp64(b0, b1, t[2]);
 }
 
-__global__ void __launch_bounds__(128) eval64_kernel(int64_t N, Lig64 L, const double* __restrict__ P, GridDev64 G,
-                                                    const StateDev* __restrict__ states, int n_states,
-                                                    const int32_t* __restrict__ state_of, const float* __restrict__ x,
-                                                    double* force, double* comps) {
-  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  const int na = L.na;
+struct Eval64Args {
+  int64_t N;
+  Lig64 L;
+  const double* P;        // the ligand's FP64 tables
+  LigandLayout LL;        // of the FP32 blob, for its gather schedule
+  const uint32_t* blob;
+  GridDev64 G;
+  const StateDev* states;
+  int n_states;
+  const int32_t* state_of;
+  const float* x;
+  double* force;
+  double* comps;
+  bool slots;             // the bonded slots are in shared memory
+};
+
+template <bool FORCES>
+__global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args A) {
+  extern __shared__ double smem64[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t n = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  if (n >= A.N) return;
+  const Lig64& L = A.L;
+  const int na = L.na, nb = L.nb, nang = L.nang, ntor = L.ntor, n_slots = A.LL.n_slots;
+  Warp64 W;
+  W.x = smem64 + (size_t)warp * warp64_doubles(na, n_slots, A.slots);
+  W.f = W.x + 3 * na;
+  W.s = A.slots ? W.f + 3 * na : nullptr;
+  W.na = na;
+  W.ns = n_slots + 1;
   double w_sg = 0.0, w_g = 0.0;
-  if (state_of) {
-    const int k = state_of[n];
-    if ((unsigned)k < (unsigned)n_states) {
-      w_sg = states[k].w_sg;
-      w_g = states[k].w_g;
+  if (A.state_of) {
+    const int k = A.state_of[n];
+    if ((unsigned)k < (unsigned)A.n_states) {
+      w_sg = A.states[k].w_sg;
+      w_g = A.states[k].w_g;
     }
   }
-  Conf cf{x + n * na * 3, force ? force + n * na * 3 : nullptr};
-  if (cf.f)
-    for (int i = 0; i < 3 * na; ++i) cf.f[i] = 0.0;
-  const double* atom = P + L.off_atom;
+  const float* xin = A.x + n * na * 3;
+  for (int i = lane; i < na; i += 32)
+    for (int d = 0; d < 3; ++d) {
+      W.x[d * na + i] = (double)xin[3 * i + d];
+      if (FORCES) W.f[d * na + i] = 0.0;
+    }
+  if (FORCES && A.slots && lane == 0) W.put(n_slots, V3{0.0, 0.0, 0.0});
+  __syncwarp();
   double e_lig = 0.0;
   // bonds: k (r - r0)^2
-  for (int t = 0; t < L.nb; ++t) {
-    const double* b = P + L.off_bond + 4 * t;
+  for (int t = lane; t < nb; t += 32) {
+    const double* b = A.P + L.off_bond + 4 * t;
     const int i = (int)b[0], j = (int)b[1];
-    const V3 d = cf.pos(i) - cf.pos(j);
-    const double r = sqrt(dot3(d, d));
-    const double dr = r - b[3];
+    const V3 d = W.pos(i) - W.pos(j);
+    const double r2 = dot3(d, d), inv_r = rsqrt(r2);
+    const double dr = (r2 > 0.0 ? r2 * inv_r : r2) - b[3];
     e_lig += b[2] * dr * dr;
-    const V3 fi = (-2.0 * b[2] * dr / r) * d;
-    cf.add(i, fi);
-    cf.add(j, -1.0 * fi);
+    if (FORCES) {
+      const V3 f = (-2.0 * b[2] * dr * inv_r) * d;
+      W.put(t, i, f);
+      W.put(nb + t, j, V3{-f.x, -f.y, -f.z});
+    }
   }
   // angles: k (theta - theta0)^2, theta at the middle atom
-  for (int t = 0; t < L.nang; ++t) {
-    const double* a = P + L.off_ang + 5 * t;
+  const int ab = 2 * nb;
+  for (int t = lane; t < nang; t += 32) {
+    const double* a = A.P + L.off_ang + 5 * t;
     const int i = (int)a[0], j = (int)a[1], k = (int)a[2];
-    const V3 u = cf.pos(i) - cf.pos(j), w = cf.pos(k) - cf.pos(j);
-    const double lu2 = dot3(u, u), lw2 = dot3(w, w), luw = sqrt(lu2 * lw2);
-    const double c = fmin(1.0, fmax(-1.0, dot3(u, w) / luw));
+    const V3 c0 = W.pos(j), u = W.pos(i) - c0, w = W.pos(k) - c0;
+    const double lu2 = dot3(u, u), lw2 = dot3(w, w), inv_luw = rsqrt(lu2 * lw2);
+    const double c = fmin(1.0, fmax(-1.0, dot3(u, w) * inv_luw));
     const double dth = acos(c) - a[4];
     e_lig += a[3] * dth * dth;
-    // d theta / d u = -(w / luw - c u / lu2) / sin(theta)
-    const double coef = 2.0 * a[3] * dth / sqrt(fmax(1.0 - c * c, 1e-30));
-    const V3 fi = coef * ((1.0 / luw) * w - (c / lu2) * u);
-    const V3 fk = coef * ((1.0 / luw) * u - (c / lw2) * w);
-    cf.add(i, fi);
-    cf.add(k, fk);
-    cf.add(j, -1.0 * (fi + fk));
+    if (FORCES) {
+      // d theta / d u = -(w / luw - c u / lu2) / sin(theta), 1 / lu2 = lw2 / luw^2
+      const double coef = 2.0 * a[3] * dth * rsqrt(fmax(1.0 - c * c, 1e-30));
+      const double cx = coef * inv_luw, cc = cx * inv_luw * c;
+      const V3 fi = cx * w - (cc * lw2) * u, fk = cx * u - (cc * lu2) * w;
+      W.put(ab + t, i, fi);
+      W.put(ab + nang + t, j, V3{-(fi.x + fk.x), -(fi.y + fk.y), -(fi.z + fk.z)});
+      W.put(ab + 2 * nang + t, k, fk);
+    }
   }
   // torsions: sum_n V_n/2 (1 + cos(n phi - gamma_n))
-  for (int t = 0; t < L.ntor; ++t) {
-    const double* q = P + L.off_tor + 10 * t;
+  const int tb = ab + 3 * nang;
+  for (int t = lane; t < ntor; t += 32) {
+    const double* q = A.P + L.off_tor + kTor64 * t;
     const int i = (int)q[0], j = (int)q[1], k = (int)q[2], l = (int)q[3];
-    const V3 b1 = cf.pos(j) - cf.pos(i), b2 = cf.pos(k) - cf.pos(j), b3 = cf.pos(l) - cf.pos(k);
+    const V3 pj = W.pos(j), pk = W.pos(k);
+    const V3 b1 = pj - W.pos(i), b2 = pk - pj, b3 = W.pos(l) - pk;
     const V3 n1 = cross3(b1, b2), n2 = cross3(b2, b3);
-    const double lb2 = sqrt(dot3(b2, b2));
-    const double n1s = fmax(dot3(n1, n1), 1e-60), n2s = fmax(dot3(n2, n2), 1e-60);
-    const double phi = atan2(lb2 * dot3(b1, n2), dot3(n1, n2));
-    double dE = 0.0;
-    for (int m = 1; m <= 3; ++m) {
-      const double arg = m * phi - q[6 + m];
-      e_lig += q[3 + m] * (1.0 + cos(arg));
-      dE -= q[3 + m] * m * sin(arg);
+    const double lb22 = dot3(b2, b2), inv_lb2 = rsqrt(lb22), lb2 = lb22 > 0.0 ? lb22 * inv_lb2 : lb22;
+    // (cos phi, sin phi) is (n1.n2, |b2| b1.n2) normalised; collinear bonds have phi = 0
+    const double cx = dot3(n1, n2), sx = lb2 * dot3(b1, n2);
+    const double h2 = cx * cx + sx * sx, inv_h = rsqrt(h2);
+    const double c1 = h2 > 0.0 ? cx * inv_h : 1.0, s1 = h2 > 0.0 ? sx * inv_h : 0.0;
+    const double c2 = 2.0 * c1 * c1 - 1.0, s2 = 2.0 * s1 * c1;
+    const double c3 = c1 * (2.0 * c2 - 1.0), s3 = s1 * (2.0 * c2 + 1.0);
+    const double *V = q + 4, *cg = q + 7, *sg = q + 10;
+    e_lig += V[0] * (1.0 + c1 * cg[0] + s1 * sg[0]) + V[1] * (1.0 + c2 * cg[1] + s2 * sg[1]) +
+             V[2] * (1.0 + c3 * cg[2] + s3 * sg[2]);
+    if (FORCES) {
+      const double dE = V[0] * (c1 * sg[0] - s1 * cg[0]) + 2.0 * V[1] * (c2 * sg[1] - s2 * cg[1]) +
+                        3.0 * V[2] * (c3 * sg[2] - s3 * cg[2]);
+      // forces: F_i = (dE lb2 / |n1|^2) n1, F_l = -(dE lb2 / |n2|^2) n2, and the middle atoms keep
+      // the total force and torque zero
+      const double i1 = rsqrt(fmax(dot3(n1, n1), 1e-60)), i2 = rsqrt(fmax(dot3(n2, n2), 1e-60));
+      const double el = dE * lb2, inv_lb22 = inv_lb2 * inv_lb2;
+      const V3 fi = (el * i1 * i1) * n1, fl = (-el * i2 * i2) * n2;
+      const double p = dot3(b1, b2) * inv_lb22, r = dot3(b3, b2) * inv_lb22;
+      W.put(tb + t, i, fi);
+      W.put(tb + ntor + t, j, (-(1.0 + p)) * fi + r * fl);
+      W.put(tb + 2 * ntor + t, k, p * fi + (-(1.0 + r)) * fl);
+      W.put(tb + 3 * ntor + t, l, fl);
     }
-    // forces: F_i = (dE lb2 / |n1|^2) n1, F_l = -(dE lb2 / |n2|^2) n2, and the middle atoms keep
-    // the total force and torque zero
-    const V3 fi = (dE * lb2 / n1s) * n1, fl = (-dE * lb2 / n2s) * n2;
-    const double p = dot3(b1, b2) / (lb2 * lb2), r = dot3(b3, b2) / (lb2 * lb2);
-    cf.add(i, fi);
-    cf.add(l, fl);
-    cf.add(j, (-(1.0 + p)) * fi + r * fl);
-    cf.add(k, p * fi + (-(1.0 + r)) * fl);
   }
-  // nonbonded pairs beyond 1-3: Lorentz-Berthelot Lennard-Jones and Coulomb, 1-4 scaled
-  for (int i = 0; i < na; ++i)
-    for (int j = i + 1; j < na; ++j) {
-      const int ty = (int)P[L.off_ptype + (int64_t)j * na + i];
-      if (ty == 2) continue;
-      const double s_lj = ty == 1 ? 0.5 : 1.0, s_el = ty == 1 ? 1.0 / 1.2 : 1.0;
-      const double* ai = atom + 6 * i;
-      const double* aj = atom + 6 * j;
-      const V3 d = cf.pos(i) - cf.pos(j);
-      const double r2 = dot3(d, d), r = sqrt(r2);
-      const double R = ai[4] + aj[4], eps = ai[5] * aj[5];
-      const double s2 = R * R / r2, s6 = s2 * s2 * s2;
-      const double elj = s_lj * eps * (s6 * s6 - 2.0 * s6);
-      const double eel = s_el * kCoulomb * ai[1] * aj[1] / r;
-      e_lig += elj + eel;
-      // -dE/dr / r
-      const double fr = (s_lj * eps * 12.0 * (s6 * s6 - s6) + eel) / r2;
-      cf.add(i, fr * d);
-      cf.add(j, (-fr) * d);
+  __syncwarp();
+  if (FORCES && A.slots) {
+    // the slots of every atom over the lanes' balanced runs; each run's partial sums stay in place
+    const uint2* gs = (const uint2*)(A.blob + A.LL.off_gs) + lane;
+    V3 a{0.0, 0.0, 0.0};
+    for (int j = 0; j < A.LL.gs_iters; ++j) {
+      const uint2 w = __ldg(gs + 32 * j);
+      const uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        a = a + W.slot(e[k] & 0x7fffu);
+        if (e[k] & 0x8000u) {
+          W.put(e[k] & 0x7fffu, a);
+          a = V3{0.0, 0.0, 0.0};
+        }
+      }
     }
+    __syncwarp();
+  }
+  // nonbonded pairs beyond 1-3 (excluded ones have R^2 < 0 and zero coefficients)
+  {
+    const int width = min(na, 32), n_pairs = na * (na - 1) / 2;
+    const double* T = A.P + L.off_pair;
+    double e12 = 0.0, e_el = 0.0;
+    for (int p0 = 0; p0 < n_pairs; p0 += width) {
+      const int p = p0 + lane;
+      const bool on = lane < width && p < n_pairs;
+      int i = 0, j = 0;
+      V3 f{0.0, 0.0, 0.0};
+      if (on) {
+        const int d = p / na;
+        i = p - d * na;
+        j = i + d + 1;
+        j = j >= na ? j - na : j;
+        const double R2 = __ldg(T + p), eps12 = __ldg(T + n_pairs + p), qq = __ldg(T + 2 * n_pairs + p);
+        const V3 dx = W.pos(i) - W.pos(j);
+        double y = rsqrt_step(dot3(dx, dx));
+        y = __double2hiint(R2) < 0 ? 0.0 : y;
+        const double y2 = y * y, s2 = R2 * y2, s6 = s2 * s2 * s2;
+        const double A12 = eps12 * s6, eel = qq * y;
+        e12 = fma(A12, s6 - 2.0, e12);
+        e_el += eel;
+        if (FORCES) f = (fma(A12, s6 - 1.0, eel) * y2) * dx;  // -dE/dr / r times the difference
+      }
+      if (FORCES) {
+        if (on) {
+          W.f[i] += f.x;
+          W.f[na + i] += f.y;
+          W.f[2 * na + i] += f.z;
+        }
+        __syncwarp();
+        if (on) {
+          W.f[j] -= f.x;
+          W.f[na + j] -= f.y;
+          W.f[2 * na + j] -= f.z;
+        }
+        __syncwarp();
+      }
+    }
+    e_lig += e12 * (1.0 / 12.0) + e_el;
+  }
   // restraint on the centre of mass
+  const double* atom = A.P + L.off_atom;
   V3 com{0.0, 0.0, 0.0};
-  for (int i = 0; i < na; ++i) com = com + atom[6 * i] * cf.pos(i);
-  com = (1.0 / L.total_mass) * com;
-  const V3 dc = com - V3{L.site[0], L.site[1], L.site[2]};
+  for (int i = lane; i < na; i += 32) com = com + __ldg(atom + 6 * i) * W.pos(i);
+  com = V3{warp_sum(com.x), warp_sum(com.y), warp_sum(com.z)};
+  const double inv_M = 1.0 / L.total_mass;
+  const V3 dc = inv_M * com - V3{L.site[0], L.site[1], L.site[2]};
   const double d = sqrt(dot3(dc, dc));
-  double e_rest = 0.0;
+  double e_rest = 0.0, c_rest = 0.0;
   if (d > L.d0) {
     const double ex = d - L.d0;
     e_rest = 0.5 * L.k_rest * ex * ex;
-    const double c = -L.k_rest * ex / (d * L.total_mass);
-    for (int i = 0; i < na; ++i) cf.add(i, (c * atom[6 * i]) * dc);
+    c_rest = -L.k_rest * ex / d * inv_M;
   } else if (!(d <= L.d0)) {
     e_rest = d;  // NaN centre of mass
   }
   // grid terms: hard Psi_g = sA r^4 + sB a + q e, soft Psi_sg = sA sr^4 + q se
   double psi_g = 0.0, psi_sg = 0.0;
-  for (int i = 0; i < na; ++i) {
+  const double inv_h = 1.0 / A.G.h;
+  const int64_t sy = A.G.nx, sz = (int64_t)A.G.nx * A.G.ny;
+  for (int i = lane; i < na; i += 32) {
     const double* ai = atom + 6 * i;
-    const Interp I = locate(G, cf.pos(i));
-    V3 gr, ga, ge, gsr, gse;
-    const double r = trilinear(G, I, [&](int64_t m) { return G.hard[m].r; }, &gr);
-    const double la = trilinear(G, I, [&](int64_t m) { return G.hard[m].a; }, &ga);
-    const double le = trilinear(G, I, [&](int64_t m) { return G.hard[m].e; }, &ge);
-    const double sr = trilinear(G, I, [&](int64_t m) { return G.soft[m].r; }, &gsr);
-    const double se = trilinear(G, I, [&](int64_t m) { return G.soft[m].e; }, &gse);
-    psi_g += ai[2] * (r * r) * (r * r) + ai[3] * la + ai[1] * le;
-    psi_sg += ai[2] * (sr * sr) * (sr * sr) + ai[1] * se;
-    if (cf.f) {
-      const V3 dg = (4.0 * ai[2] * r * r * r) * gr + ai[3] * ga + ai[1] * ge;
-      const V3 dsg = (4.0 * ai[2] * sr * sr * sr) * gsr + ai[1] * gse;
-      cf.add(i, (-w_g) * dg + (-w_sg) * dsg);
+    const double m = __ldg(ai), q = __ldg(ai + 1), sA = __ldg(ai + 2), sB = __ldg(ai + 3);
+    const Interp I = locate(A.G, W.pos(i));
+    double c[3][8], r, v;
+    V3 g, dg, dsg;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const double2* h = (const double2*)(A.G.hard + I.b + (k >> 2) * sz + ((k >> 1) & 1) * sy + (k & 1));
+      const double2 ra = __ldg(h), e0 = __ldg(h + 1);
+      c[0][k] = ra.x;
+      c[1][k] = ra.y;
+      c[2][k] = e0.x;
+    }
+    r = trilinear(c[0], I.t, g);
+    dg = (4.0 * sA * r * r * r) * g;
+    v = sA * (r * r) * (r * r);
+    v += sB * trilinear(c[1], I.t, g);
+    dg = dg + sB * g;
+    v += q * trilinear(c[2], I.t, g);
+    dg = dg + q * g;
+    psi_g += v;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const double2 s = __ldg((const double2*)(A.G.soft + I.b + (k >> 2) * sz + ((k >> 1) & 1) * sy + (k & 1)));
+      c[0][k] = s.x;
+      c[1][k] = s.y;
+    }
+    r = trilinear(c[0], I.t, g);
+    dsg = (4.0 * sA * r * r * r) * g;
+    v = sA * (r * r) * (r * r);
+    v += q * trilinear(c[1], I.t, g);
+    dsg = dsg + q * g;
+    psi_sg += v;
+    if (FORCES) {
+      const V3 f = (-w_g) * dg + (-w_sg) * dsg;
+      V3 s = V3{W.f[i], W.f[na + i], W.f[2 * na + i]} + (c_rest * m) * dc;
+      if (A.slots) {
+        const uint2 p = __ldg((const uint2*)(A.blob + A.LL.off_gp) + i);
+        s = s + (W.slot(p.x & 0xffffu) + W.slot(p.x >> 16) + W.slot(p.y & 0xffffu) + W.slot(p.y >> 16));
+      }
+      double* out = A.force + (n * na + i) * 3;
+      out[0] = s.x + (I.in[0] ? inv_h * f.x : 0.0);
+      out[1] = s.y + (I.in[1] ? inv_h * f.y : 0.0);
+      out[2] = s.z + (I.in[2] ? inv_h * f.z : 0.0);
     }
   }
-  double* c = comps + 4 * n;
-  c[0] = e_lig;
-  c[1] = e_rest;
-  c[2] = psi_sg;
-  c[3] = psi_g;
+  e_lig = warp_sum(e_lig);
+  psi_sg = warp_sum(psi_sg);
+  psi_g = warp_sum(psi_g);
+  if (lane < 4) A.comps[4 * n + lane] = lane == 0 ? e_lig : (lane == 1 ? e_rest : (lane == 2 ? psi_sg : psi_g));
 }
 
 __global__ void grid_prepare64_kernel(int64_t n, const double* __restrict__ ljr, const double* __restrict__ lja,
@@ -247,9 +406,18 @@ cudaError_t launch_grid_prepare64(cudaStream_t s, size_t n_nodes, const double* 
 cudaError_t launch_eval64(cudaStream_t s, const algdock_ctx& c, int64_t N, const int32_t* state_of, const float* x,
                           double* force, double* comps) {
   if (N == 0) return cudaSuccess;
-  const int threads = 128;
-  eval64_kernel<<<(unsigned)((N + threads - 1) / threads), threads, 0, s>>>(N, c.lig64, c.d_lig64, c.grid64,
-                                                                          c.d_states, c.K, state_of, x, force, comps);
+  const int na = c.lig.na, ns = c.lig.n_slots;
+  const bool slots = force && sizeof(double) * warp64_doubles(na, ns, true) <= kMaxSmem64;
+  const size_t per = sizeof(double) * warp64_doubles(na, ns, slots);
+  int warps = kWarps64;
+  while (warps * per > kMaxSmem64) warps /= 2;
+  const size_t smem = warps * per;
+  const Eval64Args A{N, c.lig64, c.d_lig64, c.lig, c.d_blob, c.grid64, c.d_states, c.K, state_of, x, force, comps,
+                     slots};
+  auto k = force ? eval64_kernel<true> : eval64_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)((N + warps - 1) / warps), warps * 32, smem, s>>>(A);
   return cudaGetLastError();
 }
 
