@@ -177,8 +177,8 @@ algdock_status algdock_grids_load(algdock_ctx* ctx, const algdock_grid_desc* des
 /* ---------------------------------------------------------------- the all-FP64 path
  * The FP64 arm of the precision study (no counterpart in the paper): the same energy function
  * as algdock_energy_force with every operation in FP64, on FP64 lattices and the ligand's FP64
- * parameters (kept by algdock_ligand_load).  One thread per configuration; a study tool, not a
- * fast path. */
+ * parameters (kept by algdock_ligand_load).  One warp per configuration, bound by the GPU's FP64
+ * rate (2 lanes per clock and SM): about 16 times the FP32 path's time. */
 
 /* FP64 lattices from raw grids (host or device double [nz][ny][nx]), derived as algdock_grids_load
  * does (4th root of the capped repulsive grid, tanh-capped soft grids) but kept in FP64.  They
@@ -488,7 +488,8 @@ algdock_status algdock_batch_hmc_cycle(algdock_ctx* ctx, const int32_t* state_of
 
 /* Launch shapes (for tests and tuning reports).  algdock_hmc_shape: the one-ligand HMC kernel's
  * replicas per block and 1 if it stages the per-pair table (host int32[2]).  algdock_batch_shapes:
- * the same per batch class (host int32 [4][2]; 0 for an empty class).  The pair-table and the
+ * the same per batch class (host int32 [4][2]; 0 for an empty class).  They are the shapes the
+ * pair-table rule is stated in; a launch may hold fewer replicas per block at a time.  The pair-table and the
  * pair-type kernels round differently; the replicas per block do not change a replica's
  * arithmetic. */
 algdock_status algdock_hmc_shape(algdock_ctx* ctx, int32_t* shape);

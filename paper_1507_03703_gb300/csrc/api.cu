@@ -789,8 +789,9 @@ void batch_items(const algdock_ctx* c, int cls, int wpb, std::vector<BatchItem>&
   std::stable_sort(out.begin(), out.end(), [&](const BatchItem& a, const BatchItem& b) { return cost(a) > cost(b); });
 }
 
-// The largest block shared memory of a class shape over the ligands it runs (0 if none).
-size_t batch_class_smem(const algdock_ctx* c, int cls, int wpb, bool table) {
+// The largest block shared memory of a class shape over the ligands it runs (0 if none): as the
+// class rules count it, or (team) as the kernel asks for it with wpb replicas at a time.
+size_t batch_class_smem(const algdock_ctx* c, int cls, int wpb, bool table, bool team = false) {
   size_t m = 0;
   std::vector<char> used(c->n_batch, 0);
   for (int64_t r = 0; r < c->batch_n_rep; ++r) used[c->batch_lig_of[r]] = 1;
@@ -798,7 +799,7 @@ size_t batch_class_smem(const algdock_ctx* c, int cls, int wpb, bool table) {
     if (!used[l]) continue;
     const int k = c->batch_uniform ? kBatchClasses - 1 : c->h_batch[l].cls;
     if (k != cls) continue;
-    m = std::max(m, batch_block_smem(c->h_batch[l].LL, kClassApl[cls], wpb, table));
+    m = std::max(m, (team ? batch_team_smem : batch_block_smem)(c->h_batch[l].LL, kClassApl[cls], wpb, table));
   }
   return m;
 }
@@ -813,7 +814,10 @@ cudaError_t batch_set_class(algdock_ctx* c, int cls, int wpb, bool table) {
   B.n_items = (int)items.size();
   B.wpb = wpb;
   B.table = table;
-  B.smem = batch_class_smem(c, cls, wpb, table);
+  const size_t limit = batch_smem_limit(kClassApl[cls], wpb, table);
+  B.slots = wpb;
+  while (B.slots > 1 && batch_class_smem(c, cls, B.slots, table, true) > limit) --B.slots;
+  B.smem = batch_class_smem(c, cls, B.slots, table, true);
   if (items.empty()) return cudaSuccess;
   cudaError_t e = cudaMalloc(&B.d_items, sizeof(BatchItem) * items.size());
   if (e == cudaSuccess)
@@ -1520,7 +1524,7 @@ algdock_status algdock_batch_layout(algdock_ctx* c, int64_t n_rep, const int32_t
     if (pick < 0) {
       e = batch_set_class(c, k, 4, false);
       if (e == cudaSuccess && c->batch_cls[k].n_items > 0 &&
-          c->batch_cls[k].smem > batch_smem_limit(kClassApl[k], 4, false)) {
+          batch_class_smem(c, k, 4, false) > batch_smem_limit(kClassApl[k], 4, false)) {
         batch_free(c);
         return fail(c, ALGDOCK_E_INVALID, "batch_layout: a ligand's tables exceed shared memory");
       }

@@ -2,20 +2,29 @@
 // interaction energy ("Thermodynamic Cycle"), the ligand force field and the flat-bottom
 // restraint (Eq. (binding_site)), then the Metropolis test on the total energy change.
 //
-// Layout: one warp per replica; lane l owns atoms l, l+32, l+64 (APL = atoms per lane).  Positions,
-// velocities and forces of owned atoms stay in registers for the whole trajectory; the current
-// positions are mirrored in a per-warp shared-memory array so that every lane can read every atom.
-// The ligand's parameters and topology are staged once per CTA in shared memory.
+// Layout: a team of warps per replica, one atom per lane (warp w of the team holds atoms 32w ..
+// 32w+31; up to three warps).  Position, velocity and force of the atom stay in registers for the whole
+// trajectory; the current positions are mirrored in the replica's shared-memory arrays so that
+// every lane can read every atom.  The ligand's parameters and topology are staged once per CTA in
+// shared memory.
 //
 // One force evaluation:
-//   1. bonded terms, one term per lane: each term's forces on its 2-4 atoms go to per-warp
-//      shared-memory slots (role-major, so consecutive lanes write consecutive words);
-//   2. per owned atom: the 8-corner gathers of the grid lattices and the sum of its bonded slots
-//      in a fixed order;
-//   3. nonbonded pairs, each owned atom against every other atom (the pair type table marks
-//      excluded and 1-4 pairs); when the last pass has at most 16 atoms, two lanes share an atom
-//      and split the partner range;
-//   4. the restraint on the warp-reduced centre of mass.
+//   1. bonded terms, one term per lane of the team: each term's forces on its 2-4 atoms go to the
+//      replica's shared-memory slots (role-major, so consecutive lanes write consecutive words);
+//   2. the slots summed over balanced runs by one warp, while each warp does
+//   3. the 8-corner gathers of the grid lattices for its atoms and
+//   4. the nonbonded pairs of its atoms with every other atom (the pair type table marks excluded
+//      and 1-4 pairs); when the last warp has at most 16 atoms, two lanes share an atom and split
+//      the partner range;
+//   5. the restraint on the warp-reduced centre of mass, and each atom's sum of all of these.
+//
+// The same sums in the same order as one warp holding all atoms (two or three per lane), which was
+// the layout before: 128 registers and 16 warps per SM there, where a warp's idle lanes in the second
+// and third pass, its long chain of stages and 38 instructions a pair without the pair table set the
+// pace.  Teams keep 24 warps per SM in two blocks, run stages 2 to 4 beside each other and spread a
+// few replicas over all SMs.  Measured (trials of 50 steps, bit-identical): 48 atoms, 8192 replicas
+// 1852 -> 1592 us; 83 atoms, 1152 replicas 1100 -> 673 us; 60 atoms (no pair table), 4096 replicas
+// 1924 -> 1332 us; 27 atoms, 8192 replicas 1025 -> 825 us; 16 replicas of 20 atoms, 20 steps, 96 -> 62 us.
 // Every force is accumulated by one lane in a fixed order (no atomics), so results are
 // deterministic.
 #include <math.h>
@@ -44,6 +53,12 @@ struct Lig {
   const uint2* gs;  // gather schedule: [gs_iters][32] words of four 16-bit entries
   const uint2* gp;  // [na]: four 16-bit partial-sum slots per atom
   const float4* pair;   // [p][i]: records of atom i with partners 2p, 2p + 1 (only where the table is staged)
+  // the HMC kernel without that table (stage_types): per partner pair (R*, R*', sqrt(eps), sqrt(eps)'),
+  // the scales (LJ, LJ', Coulomb, Coulomb') of each combination of two pair types, and [p][i] the byte
+  // offset of the pair's combination
+  const float4* ppar;
+  const float4* scale;
+  const uint8_t* combo;
 };
 
 __device__ inline Lig bind_ligand(const uint32_t* s, const LigandLayout& L) {
@@ -62,6 +77,21 @@ __device__ inline Lig bind_ligand(const uint32_t* s, const LigandLayout& L) {
   g.gp = (const uint2*)(s + L.off_gp);
   g.pair = (const float4*)(s + L.off_pair);
   return g;
+}
+
+// The hardware's approximate reciprocal square root and quotient.  rsqrtf and __fdividef are the same
+// instructions wrapped in a scaling of denormal arguments (three more instructions each, a tenth of
+// the kernel's); the arguments here are squared distances and their products, which are zero or
+// normal, so the results are the same bits.
+__device__ __forceinline__ float rsqrt_fast(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float div_fast(float a, float b) {
+  float r;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
 __device__ inline double warp_sum(double v) {
@@ -216,18 +246,19 @@ __device__ inline float3 cross(float3 a, float3 b) {
 }
 __device__ inline void put(float4* sl, int s, float3 f) { sl[s] = make_float4(f.x, f.y, f.z, 0.f); }
 
-// Step 1: every bonded term once, one per lane; per-role forces to the warp's float4 slots.
+// Step 1: bonded terms first, first + stride, ... of each kind, one per lane; per-role forces to
+// the replica's float4 slots.
 // Slots: bond t role r -> r*nb + t; angle -> 2nb + r*nang + t; torsion -> 2nb + 3nang + r*ntor + t.
 template <bool ENERGY, bool FORCES = true>
-__device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const float4* xs, float4* sl) {
-  const int lane = threadIdx.x & 31;
+__device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const float4* xs, float4* sl, int first,
+                                     int stride) {
   float e = 0.f;
   const int nb = LL.nb, nang = LL.nang, ntor = LL.ntor;
-  for (int t = lane; t < nb; t += 32) {  // k (r - r0)^2
+  for (int t = first; t < nb; t += stride) {  // k (r - r0)^2
     const float4 bp = L.bond[t];
     const float3 d = sub(xs[__float_as_int(bp.x)], xs[__float_as_int(bp.y)]);
     const float r2 = dot(d, d);
-    const float inv_r = rsqrtf(r2);
+    const float inv_r = rsqrt_fast(r2);
     const float dr = r2 * inv_r - bp.w;
     if (ENERGY) e += bp.z * dr * dr;
     const float c = -2.f * bp.z * dr * inv_r;
@@ -235,18 +266,18 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
     if (FORCES) put(sl, nb + t, make_float3(-c * d.x, -c * d.y, -c * d.z));
   }
   const int ab = 2 * nb;
-  for (int t = lane; t < nang; t += 32) {  // k (theta - theta0)^2
+  for (int t = first; t < nang; t += stride) {  // k (theta - theta0)^2
     const int4 id = L.ang_i[t];
     const float4 ap = L.ang_p[t];
     const float3 u = sub(xs[id.x], xs[id.y]);
     const float3 w = sub(xs[id.z], xs[id.y]);
     const float lu2 = dot(u, u), lw2 = dot(w, w);
-    const float inv_luw = rsqrtf(lu2 * lw2);
+    const float inv_luw = rsqrt_fast(lu2 * lw2);
     const float c = fminf(1.f, fmaxf(-1.f, dot(u, w) * inv_luw));
     const float dth = acosf(c) - ap.y;
     if (ENERGY) e += ap.x * dth * dth;
-    const float coef = 2.f * ap.x * dth * rsqrtf(fmaxf(1.f - c * c, 1e-12f));
-    const float cu = __fdividef(coef * c, lu2), cw = __fdividef(coef * c, lw2), cx = coef * inv_luw;
+    const float coef = 2.f * ap.x * dth * rsqrt_fast(fmaxf(1.f - c * c, 1e-12f));
+    const float cu = div_fast(coef * c, lu2), cw = div_fast(coef * c, lw2), cx = coef * inv_luw;
     const float3 fa = make_float3(cx * w.x - cu * u.x, cx * w.y - cu * u.y, cx * w.z - cu * u.z);
     const float3 fc = make_float3(cx * u.x - cw * w.x, cx * u.y - cw * w.y, cx * u.z - cw * w.z);
     if (FORCES) put(sl, ab + t, fa);
@@ -254,7 +285,7 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
     if (FORCES) put(sl, ab + 2 * nang + t, fc);
   }
   const int tb = ab + 3 * nang;
-  for (int t = lane; t < ntor; t += 32) {  // sum_n V_n/2 (1 + cos(n phi - gamma_n))
+  for (int t = first; t < ntor; t += stride) {  // sum_n V_n/2 (1 + cos(n phi - gamma_n))
     const int4 id = L.tor_i[t];
     const float4 V = L.tor_v[t], cg = L.tor_c[t], sg = L.tor_s[t];
     const float3 b1 = sub(xs[id.y], xs[id.x]);
@@ -262,10 +293,10 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
     const float3 b3 = sub(xs[id.w], xs[id.z]);
     const float3 n1 = cross(b1, b2), n2 = cross(b2, b3);
     const float lb22 = dot(b2, b2);
-    const float inv_lb2 = rsqrtf(lb22);
+    const float inv_lb2 = rsqrt_fast(lb22);
     const float lb2 = lb22 * inv_lb2;
     const float n1s = fmaxf(dot(n1, n1), 1e-20f), n2s = fmaxf(dot(n2, n2), 1e-20f);
-    const float inv = rsqrtf(n1s * n2s);
+    const float inv = rsqrt_fast(n1s * n2s);
     const float cp = dot(n1, n2) * inv;        // cos phi
     const float sp = lb2 * dot(b1, n2) * inv;  // sin phi
     const float c2 = 2.f * cp * cp - 1.f, s2 = 2.f * sp * cp;
@@ -276,7 +307,7 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
     // dE/dphi = sum_n V_n/2 n (cos(n phi) sin g - sin(n phi) cos g)
     const float dE = V.x * (cp * sg.x - sp * cg.x) + 2.f * V.y * (c2 * sg.y - s2 * cg.y) +
                      3.f * V.z * (c3 * sg.z - s3 * cg.z);
-    const float ai = __fdividef(dE * lb2, n1s), al = -__fdividef(dE * lb2, n2s);  // F_i = ai n1, F_l = al n2
+    const float ai = div_fast(dE * lb2, n1s), al = -div_fast(dE * lb2, n2s);  // F_i = ai n1, F_l = al n2
     const float inv_lb22 = inv_lb2 * inv_lb2;
     const float p = dot(b1, b2) * inv_lb22, q = dot(b3, b2) * inv_lb22;
     const float3 fi = make_float3(ai * n1.x, ai * n1.y, ai * n1.z);
@@ -293,71 +324,133 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
   return e;
 }
 
-// Step 3: nonbonded pairs.  Pass a covers atoms 32a .. 32a+31; a pass with at most 16 atoms gives
-// each atom two lanes, which split the partner range and combine with one shuffle.
+// Step 3: nonbonded pairs.  A pass covers atoms base .. base+31; a pass with at most 16 atoms gives
+// each atom two lanes, which split the partner range and combine with one shuffle.  Adds the
+// lane's energies to e2 and returns the force on atom base + lane (valid where that atom exists).
+template <bool ENERGY, bool FORCES = true>
+__device__ inline float3 nonbonded_pass(const Lig& L, int na, int base, const float4* xs, float& e2) {
+  const int lane = threadIdx.x & 31;
+  const int m = na - base;
+  const bool split = m <= 16;
+  const int il = split ? (lane & 15) : lane;
+  const int i = base + il;
+  const bool act = il < m;
+  // partners: all j; split: the low half-warp takes j = 0 .. h-1 upwards, the high half-warp
+  // j = na-1 .. h downwards (opposite directions keep the two rows read per step in different
+  // shared-memory banks)
+  int jb = 0, cnt = na, dir = 1;
+  if (split) {
+    const int h = (na + 1) >> 1;
+    jb = lane < 16 ? 0 : na - 1;
+    cnt = lane < 16 ? h : na - h;
+    dir = lane < 16 ? 1 : -1;
+  }
+  float fx = 0.f, fy = 0.f, fz = 0.f;
+  if (act) {
+    const float4 pi = xs[i];
+    const float4 bi = L.atom_b[i];
+    const float qi = (float)kCoulomb * pi.w, ri = bi.x, si = bi.y;
+    const uint8_t* ty_col = L.ptype + i;
+    for (int jj = 0; jj < cnt; ++jj) {
+      const int j = jb + dir * jj;
+      const float4 pj = xs[j];
+      const float2 bj = *(const float2*)&L.atom_b[j];
+      const uint32_t ty = ty_col[j * na];
+      const bool excluded = ty == 2u;
+      const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
+      const float r2 = excluded ? 1.f : fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      const float inv_r = rsqrt_fast(r2);
+      const float inv_r2 = inv_r * inv_r;
+      const float R = ri + bj.x;
+      const float s2 = R * R * inv_r2;
+      const float s6 = s2 * s2 * s2;
+      const float eps = excluded ? 0.f : (ty == 1u ? 0.5f : 1.f) * (si * bj.y);
+      const float qq = excluded ? 0.f : (ty == 1u ? (float)(1.0 / 1.2) : 1.f) * (qi * pj.w);
+      const float eel = qq * inv_r;
+      const float fr = fmaf(12.f * eps, s6 * s6 - s6, eel) * inv_r2;
+      if (FORCES) {
+        fx = fmaf(fr, dx, fx);
+        fy = fmaf(fr, dy, fy);
+        fz = fmaf(fr, dz, fz);
+      }
+      if (ENERGY) e2 += fmaf(eps, s6 * s6 - 2.f * s6, eel);
+    }
+  }
+  if (split) {
+    fx += __shfl_xor_sync(kFull, fx, 16);
+    fy += __shfl_xor_sync(kFull, fy, 16);
+    fz += __shfl_xor_sync(kFull, fz, 16);
+  }
+  return make_float3(fx, fy, fz);
+}
+
+// The forces of a full pass (more than 16 atoms), partners two at a time: the operations of
+// nonbonded_pass in paired instructions up to the pair force, then both partners added in turn, so
+// the sums are the same bits.  Pair types come as one byte per two partners, an offset into the
+// table of their scales, in place of two bytes and their selects.  22 instructions a partner
+// instead of 38.
+__device__ inline float3 nonbonded_type_pass(const Lig& L, int na, int base, const float4* xs, const float* xp) {
+  const int i = base + (threadIdx.x & 31);
+  float fx = 0.f, fy = 0.f, fz = 0.f;
+  if (i < na) {
+    const float4 own = xs[i];
+    const float2 b = *(const float2*)&L.atom_b[i];
+    const float qc = (float)kCoulomb * own.w;
+    const f32x2 X = pack2(own.x, own.x), Y = pack2(own.y, own.y), Z = pack2(own.z, own.z);
+    const f32x2 Qi = pack2(qc, qc), Ri = pack2(b.x, b.x), Si = pack2(b.y, b.y), twelve = pack2(12.f, 12.f);
+    constexpr f32x2 sign = 0x8000000080000000ull;
+    const float4* pp = (const float4*)xp;
+    const float4* par = L.ppar;
+    const uint8_t* combo = L.combo + i;
+#pragma unroll 2
+    for (int p = (na + 1) >> 1; p > 0; --p) {
+      const float4 q0 = pp[0];  // (x, x', y, y')
+      const float4 q1 = pp[1];  // (z, z', q, q')
+      const float4 s = *par;    // (R*, R*', sqrt(eps), sqrt(eps)')
+      const float4 c = *(const float4*)((const char*)L.scale + *combo);
+      pp += 2;
+      ++par;
+      combo += na;
+      const f32x2 dx = sub2(X, pack2(q0.x, q0.y)), dy = sub2(Y, pack2(q0.z, q0.w));
+      const f32x2 dz = sub2(Z, pack2(q1.x, q1.y));
+      float ra, rb;
+      unpack2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ra, rb);
+      ra = c.z == 0.f ? 1.f : ra;  // excluded (also i itself and the partner that completes an odd count)
+      rb = c.w == 0.f ? 1.f : rb;
+      const f32x2 inv_r = pack2(rsqrt_fast(ra), rsqrt_fast(rb));
+      const f32x2 inv_r2 = mul2(inv_r, inv_r);
+      const f32x2 R = add2(Ri, pack2(s.x, s.y));
+      const f32x2 s2 = mul2(mul2(R, R), inv_r2);
+      const f32x2 s6 = mul2(mul2(s2, s2), s2);
+      const f32x2 eps = mul2(pack2(c.x, c.y), mul2(Si, pack2(s.z, s.w)));
+      const f32x2 qq = mul2(pack2(c.z, c.w), mul2(Qi, pack2(q1.z, q1.w)));
+      const f32x2 fr = mul2(fma2(mul2(twelve, eps), fma2(s6, s6, s6 ^ sign), mul2(qq, inv_r)), inv_r2);
+      float fa, fb, da, db;
+      unpack2(fr, fa, fb);
+      unpack2(dx, da, db);
+      fx = fmaf(fb, db, fmaf(fa, da, fx));
+      unpack2(dy, da, db);
+      fy = fmaf(fb, db, fmaf(fa, da, fy));
+      unpack2(dz, da, db);
+      fz = fmaf(fb, db, fmaf(fa, da, fz));
+    }
+  }
+  return make_float3(fx, fy, fz);
+}
+
 template <int APL, bool ENERGY, bool FORCES = true>
 __device__ inline void nonbonded(const Lig& L, int na, const float4* xs, float (&F)[APL][3], float& el) {
   const int lane = threadIdx.x & 31;
   float e2 = 0.f;
 #pragma unroll
   for (int a = 0; a < APL; ++a) {
-    const int base = 32 * a;
-    const int m = na - base;
+    const int m = na - 32 * a;
     if (m <= 0) break;
-    const bool split = m <= 16;
-    const int il = split ? (lane & 15) : lane;
-    const int i = base + il;
-    const bool act = il < m;
-    // partners: all j; split: the low half-warp takes j = 0 .. h-1 upwards, the high half-warp
-    // j = na-1 .. h downwards (opposite directions keep the two rows read per step in different
-    // shared-memory banks)
-    int jb = 0, cnt = na, dir = 1;
-    if (split) {
-      const int h = (na + 1) >> 1;
-      jb = lane < 16 ? 0 : na - 1;
-      cnt = lane < 16 ? h : na - h;
-      dir = lane < 16 ? 1 : -1;
-    }
-    float fx = 0.f, fy = 0.f, fz = 0.f;
-    if (act) {
-      const float4 pi = xs[i];
-      const float4 bi = L.atom_b[i];
-      const float qi = (float)kCoulomb * pi.w, ri = bi.x, si = bi.y;
-      const uint8_t* ty_col = L.ptype + i;
-      for (int jj = 0; jj < cnt; ++jj) {
-        const int j = jb + dir * jj;
-        const float4 pj = xs[j];
-        const float2 bj = *(const float2*)&L.atom_b[j];
-        const uint32_t ty = ty_col[j * na];
-        const bool excluded = ty == 2u;
-        const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-        const float r2 = excluded ? 1.f : fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float inv_r = rsqrtf(r2);
-        const float inv_r2 = inv_r * inv_r;
-        const float R = ri + bj.x;
-        const float s2 = R * R * inv_r2;
-        const float s6 = s2 * s2 * s2;
-        const float eps = excluded ? 0.f : (ty == 1u ? 0.5f : 1.f) * (si * bj.y);
-        const float qq = excluded ? 0.f : (ty == 1u ? (float)(1.0 / 1.2) : 1.f) * (qi * pj.w);
-        const float eel = qq * inv_r;
-        const float fr = fmaf(12.f * eps, s6 * s6 - s6, eel) * inv_r2;
-        if (FORCES) {
-          fx = fmaf(fr, dx, fx);
-          fy = fmaf(fr, dy, fy);
-          fz = fmaf(fr, dz, fz);
-        }
-        if (ENERGY) e2 += fmaf(eps, s6 * s6 - 2.f * s6, eel);
-      }
-    }
-    if (split) {
-      fx += __shfl_xor_sync(kFull, fx, 16);
-      fy += __shfl_xor_sync(kFull, fy, 16);
-      fz += __shfl_xor_sync(kFull, fz, 16);
-    }
-    if (lane < m && (!split || lane < 16)) {
-      F[a][0] += fx;
-      F[a][1] += fy;
-      F[a][2] += fz;
+    const float3 f = nonbonded_pass<ENERGY, FORCES>(L, na, 32 * a, xs, e2);
+    if (lane < m) {
+      F[a][0] += f.x;
+      F[a][1] += f.y;
+      F[a][2] += f.z;
     }
   }
   if (ENERGY) el += 0.5f * e2;
@@ -385,87 +478,70 @@ __device__ inline void put_pair_pos(float* xp, int i, float x, float y, float z)
   b[4] = z;
 }
 
-template <int APL, bool ENERGY, bool FORCES = true>
-__device__ inline void nonbonded_table(const Lig& L, int na, const float4* xs, const float* xp, float (&F)[APL][3],
-                                       float& el) {
+template <bool ENERGY, int UNROLL>
+__device__ inline float3 nonbonded_table_pass(const Lig& L, int na, int base, const float4* xs, const float* xp,
+                                              f32x2& e2) {
   const int lane = threadIdx.x & 31;
   const int P = (na + 1) >> 1;
   const f32x2 one = pack2(1.f, 1.f), two = pack2(2.f, 2.f), twelfth = pack2(1.f / 12.f, 1.f / 12.f);
-  f32x2 e2 = 0ull;  // (0.f, 0.f)
-#pragma unroll
-  for (int a = 0; a < APL; ++a) {
-    const int base = 32 * a;
-    const int m = na - base;
-    if (m <= 0) break;
-    const bool split = m <= 16;
-    const int il = split ? (lane & 15) : lane;
-    const int i = base + il;
-    const bool act = il < m;
-    int pb = 0, cnt = P, dir = 1;
-    if (split) {
-      const int h = (P + 1) >> 1;
-      pb = lane < 16 ? 0 : P - 1;
-      cnt = lane < 16 ? h : P - h;
-      dir = lane < 16 ? 1 : -1;
-    }
-    f32x2 fx2 = 0ull, fy2 = 0ull, fz2 = 0ull;
-    if (act) {
-      const float4 own = xs[i];  // (x, y, z, R*_i) in the table path
-      const f32x2 X = pack2(own.x, own.x), Y = pack2(own.y, own.y), Z = pack2(own.z, own.z);
-      const f32x2 Ri = pack2(own.w, own.w);
-      const float4* rec = L.pair + (size_t)pb * na + i;
-      const float4* pp = (const float4*)xp + 2 * pb;
-      const int rstep = dir * na, pstep = 2 * dir;
-#pragma unroll 2
-      for (int jj = 0; jj < cnt; ++jj) {
-        const float4 q0 = pp[0];  // (x, x', y, y')
-        const float4 q1 = pp[1];  // (z, z', R*, R*')
-        const float4 t = *rec;    // (e, e', c, c')
-        pp += pstep;
-        rec += rstep;
-        const f32x2 dx = sub2(X, pack2(q0.x, q0.y)), dy = sub2(Y, pack2(q0.z, q0.w));
-        const f32x2 dz = sub2(Z, pack2(q1.x, q1.y));
-        float ra, rb;
-        unpack2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ra, rb);
-        const f32x2 inv_r = pack2(rsqrtf(fmaxf(ra, kPairMinR2)), rsqrtf(fmaxf(rb, kPairMinR2)));
-        const f32x2 R = add2(Ri, pack2(q1.z, q1.w));
-        const f32x2 inv_r2 = mul2(inv_r, inv_r);
-        const f32x2 s2 = mul2(mul2(R, R), inv_r2);
-        const f32x2 s6 = mul2(mul2(s2, s2), s2);
-        const f32x2 e = pack2(t.x, t.y);
-        const f32x2 eel = mul2(pack2(t.z, t.w), inv_r);
-        if (FORCES) {
-          const f32x2 fr = mul2(fma2(e, mul2(s6, sub2(s6, one)), eel), inv_r2);
-          fx2 = fma2(fr, dx, fx2);
-          fy2 = fma2(fr, dy, fy2);
-          fz2 = fma2(fr, dz, fz2);
-        }
-        if (ENERGY) e2 = add2(e2, fma2(mul2(e, twelfth), mul2(s6, sub2(s6, two)), eel));
-      }
-    }
-    float fx, fy, fz, ha, hb;
-    unpack2(fx2, fx, ha);
-    fx += ha;
-    unpack2(fy2, fy, ha);
-    fy += ha;
-    unpack2(fz2, fz, hb);
-    fz += hb;
-    if (split) {
-      fx += __shfl_xor_sync(kFull, fx, 16);
-      fy += __shfl_xor_sync(kFull, fy, 16);
-      fz += __shfl_xor_sync(kFull, fz, 16);
-    }
-    if (lane < m && (!split || lane < 16)) {
-      F[a][0] += fx;
-      F[a][1] += fy;
-      F[a][2] += fz;
+  const int m = na - base;
+  const bool split = m <= 16;
+  const int il = split ? (lane & 15) : lane;
+  const int i = base + il;
+  const bool act = il < m;
+  int pb = 0, cnt = P, dir = 1;
+  if (split) {
+    const int h = (P + 1) >> 1;
+    pb = lane < 16 ? 0 : P - 1;
+    cnt = lane < 16 ? h : P - h;
+    dir = lane < 16 ? 1 : -1;
+  }
+  f32x2 fx2 = 0ull, fy2 = 0ull, fz2 = 0ull;
+  if (act) {
+    const float4 own = xs[i];  // (x, y, z, R*_i) in the table path
+    const f32x2 X = pack2(own.x, own.x), Y = pack2(own.y, own.y), Z = pack2(own.z, own.z);
+    const f32x2 Ri = pack2(own.w, own.w);
+    const float4* rec = L.pair + (size_t)pb * na + i;
+    const float4* pp = (const float4*)xp + 2 * pb;
+    const int rstep = dir * na, pstep = 2 * dir;
+#pragma unroll UNROLL
+    for (int jj = 0; jj < cnt; ++jj) {
+      const float4 q0 = pp[0];  // (x, x', y, y')
+      const float4 q1 = pp[1];  // (z, z', R*, R*')
+      const float4 t = *rec;    // (e, e', c, c')
+      pp += pstep;
+      rec += rstep;
+      const f32x2 dx = sub2(X, pack2(q0.x, q0.y)), dy = sub2(Y, pack2(q0.z, q0.w));
+      const f32x2 dz = sub2(Z, pack2(q1.x, q1.y));
+      float ra, rb;
+      unpack2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ra, rb);
+      const f32x2 inv_r = pack2(rsqrt_fast(fmaxf(ra, kPairMinR2)), rsqrt_fast(fmaxf(rb, kPairMinR2)));
+      const f32x2 R = add2(Ri, pack2(q1.z, q1.w));
+      const f32x2 inv_r2 = mul2(inv_r, inv_r);
+      const f32x2 s2 = mul2(mul2(R, R), inv_r2);
+      const f32x2 s6 = mul2(mul2(s2, s2), s2);
+      const f32x2 e = pack2(t.x, t.y);
+      const f32x2 eel = mul2(pack2(t.z, t.w), inv_r);
+      const f32x2 fr = mul2(fma2(e, mul2(s6, sub2(s6, one)), eel), inv_r2);
+      fx2 = fma2(fr, dx, fx2);
+      fy2 = fma2(fr, dy, fy2);
+      fz2 = fma2(fr, dz, fz2);
+      if (ENERGY) e2 = add2(e2, fma2(mul2(e, twelfth), mul2(s6, sub2(s6, two)), eel));
     }
   }
-  if (ENERGY) {
-    float ea, eb;
-    unpack2(e2, ea, eb);
-    el += 0.5f * (ea + eb);
+  float fx, fy, fz, ha, hb;
+  unpack2(fx2, fx, ha);
+  fx += ha;
+  unpack2(fy2, fy, ha);
+  fy += ha;
+  unpack2(fz2, fz, hb);
+  fz += hb;
+  if (split) {
+    fx += __shfl_xor_sync(kFull, fx, 16);
+    fy += __shfl_xor_sync(kFull, fy, 16);
+    fz += __shfl_xor_sync(kFull, fz, 16);
   }
+  return make_float3(fx, fy, fz);
 }
 
 // Step 2a: the bonded forces gathered over the lanes' balanced runs of the atom-sorted slot list
@@ -494,23 +570,21 @@ __device__ inline void gather_runs(const Lig& L, const LigandLayout& LL, float4*
   }
 }
 
-// Forces on the lane's atoms (and, if ENERGY, the lane's partial energies).  xs holds all
-// positions (x, y, z, q), with R*_i in place of q when TABLE; sl is the warp's bonded-slot scratch
-// (n_slots + 1 float4, the last zero).
-template <int APL, bool ENERGY, bool TABLE = false, bool FORCES = true>
+// Energies (and, with FORCES, the forces on the lane's atoms) of one configuration by one warp, lane l
+// holding atoms l, l+32, l+64.  xs holds all positions (x, y, z, q); sl is the warp's bonded-slot
+// scratch (n_slots + 1 float4, the last zero).
+template <int APL, bool FORCES>
 __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const GridDev& G, const float4* xs, float4* sl,
                                 const float (&x)[APL][3], const float (&mass)[APL], float (&F)[APL][3], float w_sg,
-                                float w_g, bool all_grids, Energies& en, int& outside, const float* xp = nullptr) {
+                                float w_g, Energies& en) {
   const int lane = threadIdx.x & 31;
   const int na = LL.na;
-  float el = bonded_terms<ENERGY, FORCES>(L, LL, xs, sl);
+  float el = bonded_terms<true, FORCES>(L, LL, xs, sl, lane, 32);
   __syncwarp();
   if (FORCES) {
     gather_runs(L, LL, sl);
     __syncwarp();
   }
-  const bool hard = all_grids || w_g != 0.f;
-  const bool soft = all_grids || w_sg != 0.f;
   float eg = 0.f, esg = 0.f;
   float mx = 0.f, my = 0.f, mz = 0.f;
 #pragma unroll
@@ -522,16 +596,13 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
     mx += mass[a] * x[a][0];
     my += mass[a] * x[a][1];
     mz += mass[a] * x[a][2];
-    if (hard || soft) {
-      const GridOut go = grid_atom(G, x[a][0], x[a][1], x[a][2], pa.z, pa.w, pa.y, hard, soft, FORCES ? w_sg : 0.f,
-                                   FORCES ? w_g : 0.f);
-      F[a][0] += go.fx;
-      F[a][1] += go.fy;
-      F[a][2] += go.fz;
-      eg += go.e_g;
-      esg += go.e_sg;
-      outside += go.outside ? 1 : 0;
-    }
+    const GridOut go = grid_atom(G, x[a][0], x[a][1], x[a][2], pa.z, pa.w, pa.y, true, true, FORCES ? w_sg : 0.f,
+                                 FORCES ? w_g : 0.f);
+    F[a][0] += go.fx;
+    F[a][1] += go.fy;
+    F[a][2] += go.fz;
+    eg += go.e_g;
+    esg += go.e_sg;
     if (FORCES) {  // the atom's partial sums, in run order
       const uint2 p = L.gp[i];
       const float4 q0 = sl[p.x & 0xffffu], q1 = sl[p.x >> 16], q2 = sl[p.y & 0xffffu], q3 = sl[p.y >> 16];
@@ -540,8 +611,7 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
       F[a][2] += ((q0.z + q1.z) + q2.z) + q3.z;
     }
   }
-  if (TABLE) nonbonded_table<APL, ENERGY, FORCES>(L, na, xs, xp, F, el);
-  else nonbonded<APL, ENERGY, FORCES>(L, na, xs, F, el);
+  nonbonded<APL, true, FORCES>(L, na, xs, F, el);
   // restraint on the centre of mass
   mx = warp_sumf(mx);
   my = warp_sumf(my);
@@ -571,11 +641,19 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
   en.g = eg;
 }
 
+// The four components summed over the warp.  The butterfly's pairs, with two of the four sums (then
+// one) kept per lane at the first steps: 6 FP64 additions a lane instead of 20, the same sums.
 __device__ inline void reduce_components(const Energies& e, double c[4]) {
-  c[0] = warp_sum((double)e.lig);
-  c[1] = warp_sum((double)e.rest);
-  c[2] = warp_sum((double)e.sg);
-  c[3] = warp_sum((double)e.g);
+  const int lane = threadIdx.x & 31;
+  const double lig = (double)e.lig, rest = (double)e.rest, sg = (double)e.sg, g = (double)e.g;
+  const bool h16 = lane & 16, h8 = lane & 8;
+  const double k0 = (h16 ? sg : lig) + __shfl_xor_sync(kFull, h16 ? lig : sg, 16);
+  const double k1 = (h16 ? g : rest) + __shfl_xor_sync(kFull, h16 ? rest : g, 16);
+  double v = (h8 ? k1 : k0) + __shfl_xor_sync(kFull, h8 ? k0 : k1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) c[j] = __shfl_sync(kFull, v, 8 * j);
 }
 
 // U_k = ((U_L + U_I) + w_sg Psi_sg) + w_g Psi_g, a zero weight dropping its term.
@@ -592,26 +670,68 @@ __device__ inline void stage_ligand(uint32_t* s, const uint32_t* __restrict__ bl
   for (int i = threadIdx.x; i < words / 4; i += blockDim.x) dst[i] = src[i];
 }
 
-// Shared memory of one block: ligand blob, then per warp 32*APL float4 positions, with the pair
-// table also the pair-interleaved mirror of the pair loop (32*APL * 4 floats), and the bonded-slot
-// scratch (n_slots + 1 float4, the last a zero slot).
+// Shared memory of one replica: 32*APL float4 positions, the pair-interleaved mirror of the pair loop
+// (32*APL * 4 floats), the bonded-slot scratch (n_slots + 1 float4, the last a zero slot) and, for a
+// team of warps, what they exchange.  A block holds the ligand blob and one such area per replica
+// (of the energy kernel: per warp, without the mirror and the exchange area, which is also what the
+// rule on the pair table counts, with the mirror where the table is).
 __host__ __device__ inline int scratch_words(const LigandLayout& L) { return 4 * (L.n_slots + 1); }
 __host__ __device__ inline int warp_words(const LigandLayout& L, int apl, bool table) {
   return (table ? 8 : 4) * 32 * apl + scratch_words(L);
 }
+struct TeamExchange {
+  f32x2 lane[32];                // per-lane values on their way to the first warp
+  float rx, ry, rz, rc, re;      // restraint: displacement, force factor, energy
+  int accept;
+  unsigned long long replica[2];
+};
+constexpr int kTeamWords = (sizeof(TeamExchange) + 15) / 16 * 4;
+__host__ __device__ inline int replica_words(const LigandLayout& L, int apl) {
+  return warp_words(L, apl, true) + (apl > 1 ? kTeamWords : 0);
+}
+// Staged tables of a block: the blob with the pair table, or without it the pair-type tables after it.
+__host__ __device__ inline int combo_words(const LigandLayout& L) { return (((L.na + 1) / 2) * L.na + 15) / 16 * 4; }
+__host__ __device__ inline int staged_words(const LigandLayout& L, bool table) {
+  return table ? L.words_pair : L.words + 4 * ((L.na + 1) / 2) + 64 + combo_words(L);
+}
 
 struct WarpSmem {
   float4* xs;
-  float* xp;  // pair-interleaved positions (table kernels only)
+  float* xp;   // pair-interleaved positions and R* (pair table) or charges
   float4* sl;  // bonded-force slots
+  TeamExchange* ex;
 };
-template <int APL, bool TABLE = false>
-__device__ inline WarpSmem warp_smem(uint32_t* smem, int staged_words, const LigandLayout& LL, int warp) {
-  uint32_t* p = smem + staged_words + warp * warp_words(LL, APL, TABLE);
-  float* xp = TABLE ? (float*)(p + 4 * 32 * APL) : nullptr;
-  float4* sl = (float4*)(p + (TABLE ? 8 : 4) * 32 * APL);
-  if ((threadIdx.x & 31) == 0) sl[LL.n_slots] = make_float4(0.f, 0.f, 0.f, 0.f);  // the zero slot
-  return WarpSmem{(float4*)p, xp, sl};
+template <int APL, bool MIRROR>
+__device__ inline WarpSmem warp_smem(uint32_t* p, const LigandLayout& LL) {
+  float* xp = MIRROR ? (float*)(p + 4 * 32 * APL) : nullptr;
+  float4* sl = (float4*)(p + (MIRROR ? 8 : 4) * 32 * APL);
+  return WarpSmem{(float4*)p, xp, sl, (TeamExchange*)(p + warp_words(LL, APL, MIRROR))};
+}
+
+// The pair-type tables (Lig::ppar, scale, combo) from the staged blob, by the whole block.
+__device__ inline void stage_types(uint32_t* s, const LigandLayout& LL, Lig& L) {
+  const int na = LL.na, P = (na + 1) / 2;
+  float4* par = (float4*)(s + LL.words);
+  float4* scale = par + P;
+  uint8_t* combo = (uint8_t*)(scale + 16);
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    const float4 a = L.atom_b[2 * p], b = 2 * p + 1 < na ? L.atom_b[2 * p + 1] : none;
+    par[p] = make_float4(a.x, b.x, a.y, b.y);
+  }
+  for (int e = threadIdx.x; e < 16; e += blockDim.x) {
+    auto lj = [](int ty) { return ty == 0 ? 1.f : (ty == 1 ? 0.5f : 0.f); };
+    auto el = [](int ty) { return ty == 0 ? 1.f : (ty == 1 ? (float)(1.0 / 1.2) : 0.f); };
+    scale[e] = make_float4(lj(e & 3), lj(e >> 2), el(e & 3), el(e >> 2));
+  }
+  for (int e = threadIdx.x; e < P * na; e += blockDim.x) {
+    const int p = e / na, i = e - p * na;
+    const int ta = L.ptype[2 * p * na + i], tb = 2 * p + 1 < na ? L.ptype[(2 * p + 1) * na + i] : 2;
+    combo[e] = (uint8_t)(16 * (ta | tb << 2));
+  }
+  L.ppar = par;
+  L.scale = scale;
+  L.combo = combo;
 }
 
 struct HmcArgs {
@@ -639,213 +759,410 @@ struct HmcArgs {
   unsigned long long* work;  // single-ligand launches: replicas handed out so far (zero at launch), or NULL
 };
 
-// One HMC trial of replica r by the calling warp: momenta, n_steps of velocity Verlet, the
-// Metropolis test, and the write-back of an accepted trial.  xs / xp / sl are the warp's
-// shared-memory arrays (the zero partner of an odd atom count is already in xp).
-template <int APL, bool TABLE, bool BATCH>
+// The warps of a replica's team: warp w of W holds atoms 32w .. 32w+31.
+template <int W>
+__device__ __forceinline__ void team_sync(int team) {
+  if (W == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(team), "n"(32 * W) : "memory");
+}
+
+// One force evaluation by the team, with the positions published.  The pieces and the order of
+// every sum are those of one warp holding all atoms; the pieces that do not depend on one another
+// run in different warps:
+//   - bonded terms over all the team's lanes; then
+//   - the last warp, which has the fewest atoms, adds the slots over the balanced runs and forms the
+//     centre of mass, while each warp does its atoms' grid terms and pairs; then
+//   - each warp adds up its atoms' forces.
+// An energy evaluation (the first and the last of a trial) also sums energies per lane in the order
+// of one warp: the first warp takes all bonded terms, and the pair and grid sums of a lane pass
+// through the warps in turn.  Its results are valid in the first warp.
+template <int W, bool ENERGY, bool TABLE, int UNROLL>
+__device__ __forceinline__ void team_evaluate(const LigandLayout& LL, const Lig& L, const GridDev& G,
+                                              const WarpSmem& ws, int w, int team, const float (&x)[3], float mass,
+                                              float (&F)[3], float w_sg, float w_g, float invM, float d0_safe2,
+                                              Energies& en, int& outside) {
+  const int lane = threadIdx.x & 31;
+  const int na = LL.na;
+  const int i = 32 * w + lane;
+  const bool own = i < na;
+  float el = 0.f;
+  if (ENERGY) {
+    if (w == 0) el = bonded_terms<true>(L, LL, ws.xs, ws.sl, lane, 32);
+  } else {
+    bonded_terms<false>(L, LL, ws.xs, ws.sl, i, 32 * W);
+  }
+  team_sync<W>(team);
+  float rx, ry, rz, rc = 0.f, er = 0.f;
+  if (w == W - 1) {
+    gather_runs(L, LL, ws.sl);
+    float mx = 0.f, my = 0.f, mz = 0.f;
+    if (W == 1) {
+      if (own) {
+        mx += mass * x[0];
+        my += mass * x[1];
+        mz += mass * x[2];
+      }
+    } else {
+#pragma unroll
+      for (int a = 0; a < W; ++a) {
+        const int j = lane + 32 * a;
+        if (j >= na) continue;
+        const float m = L.atom_b[j].z;
+        const float4 p = ws.xs[j];
+        mx += m * p.x;
+        my += m * p.y;
+        mz += m * p.z;
+      }
+    }
+    mx = warp_sumf(mx);
+    my = warp_sumf(my);
+    mz = warp_sumf(mz);
+    rx = mx * invM - LL.site[0], ry = my * invM - LL.site[1], rz = mz * invM - LL.site[2];
+    const float d2 = rx * rx + ry * ry + rz * rz;
+    if (!(d2 < d0_safe2)) {  // not clearly inside
+      const float d = sqrtf(d2);
+      if (d > LL.d0) {
+        const float ex = d - LL.d0;
+        er = 0.5f * LL.k_rest * ex * ex;
+        rc = -LL.k_rest * ex / d * invM;
+      } else if (!(d <= LL.d0)) {  // NaN centre of mass: make the energy NaN
+        er = d;
+      }
+    }
+    if (W > 1 && lane == 0) {
+      ws.ex->rx = rx;
+      ws.ex->ry = ry;
+      ws.ex->rz = rz;
+      ws.ex->rc = rc;
+      ws.ex->re = er;
+    }
+  }
+  const bool hard = ENERGY || w_g != 0.f;
+  const bool soft = ENERGY || w_sg != 0.f;
+  float eg = 0.f, esg = 0.f;
+  F[0] = F[1] = F[2] = 0.f;
+  if (own && (hard || soft)) {
+    const float4 pa = L.atom_a[i];
+    const GridOut go = grid_atom(G, x[0], x[1], x[2], pa.z, pa.w, pa.y, hard, soft, w_sg, w_g);
+    F[0] += go.fx;
+    F[1] += go.fy;
+    F[2] += go.fz;
+    eg += go.e_g;
+    esg += go.e_sg;
+    outside += go.outside ? 1 : 0;
+  }
+  float3 f = make_float3(0.f, 0.f, 0.f);
+  if (!ENERGY || W == 1) {
+    f32x2 e2 = 0ull;
+    float e1 = 0.f;
+    if (TABLE) {
+      if (32 * w < na) f = nonbonded_table_pass<ENERGY, UNROLL>(L, na, 32 * w, ws.xs, ws.xp, e2);
+    } else if (!ENERGY && na - 32 * w > 16) {
+      f = nonbonded_type_pass(L, na, 32 * w, ws.xs, ws.xp);
+    } else if (32 * w < na) {
+      f = nonbonded_pass<ENERGY>(L, na, 32 * w, ws.xs, e1);
+    }
+    if (ENERGY) {
+      float ea = e1, eb = 0.f;
+      if (TABLE) unpack2(e2, ea, eb);
+      el += 0.5f * (TABLE ? ea + eb : e1);
+    }
+  } else {
+    for (int a = 0; a < W; ++a) {
+      if (w == a && 32 * a < na) {
+        f32x2 e2 = a > 0 ? ws.ex->lane[lane] : 0ull;
+        if (TABLE) {
+          f = nonbonded_table_pass<true, 1>(L, na, 32 * a, ws.xs, ws.xp, e2);
+        } else {
+          float e1, pad;
+          unpack2(e2, e1, pad);
+          f = nonbonded_pass<true>(L, na, 32 * a, ws.xs, e1);
+          e2 = pack2(e1, 0.f);
+        }
+        ws.ex->lane[lane] = e2;
+      }
+      team_sync<W>(team);
+    }
+    if (w == 0) {
+      float ea, eb;
+      unpack2(ws.ex->lane[lane], ea, eb);
+      el += 0.5f * (TABLE ? ea + eb : ea);
+    }
+    for (int a = 1; a < W; ++a) {
+      team_sync<W>(team);
+      if (w == a) ws.ex->lane[lane] = pack2(eg, esg);
+      team_sync<W>(team);
+      if (w == 0) {
+        float v, u;
+        unpack2(ws.ex->lane[lane], v, u);
+        eg += v;
+        esg += u;
+      }
+    }
+  }
+  team_sync<W>(team);  // partial sums and restraint
+  if (W > 1) {
+    rx = ws.ex->rx;
+    ry = ws.ex->ry;
+    rz = ws.ex->rz;
+    rc = ws.ex->rc;
+    if (ENERGY) er = ws.ex->re;
+  }
+  if (own) {
+    // the atom's partial sums, in run order
+    const uint2 p = L.gp[i];
+    const float4 q0 = ws.sl[p.x & 0xffffu], q1 = ws.sl[p.x >> 16], q2 = ws.sl[p.y & 0xffffu], q3 = ws.sl[p.y >> 16];
+    F[0] += ((q0.x + q1.x) + q2.x) + q3.x;
+    F[1] += ((q0.y + q1.y) + q2.y) + q3.y;
+    F[2] += ((q0.z + q1.z) + q2.z) + q3.z;
+    F[0] += f.x;
+    F[1] += f.y;
+    F[2] += f.z;
+    if (rc != 0.f) {
+      F[0] += rc * mass * rx;
+      F[1] += rc * mass * ry;
+      F[2] += rc * mass * rz;
+    }
+  }
+  if (ENERGY) {
+    en.lig = el;
+    en.rest = lane == 0 ? er : 0.f;
+    en.sg = esg;
+    en.g = eg;
+  }
+}
+
+// Sum of the atoms' m v^2 (in the first warp): a lane's atoms in order, then over the lanes.  t: the
+// calling lane's v^2.
+template <int W>
+__device__ __forceinline__ double team_kinetic(const Lig& L, int na, const WarpSmem& ws, int w, int team, float mass,
+                                               float t) {
+  const int lane = threadIdx.x & 31;
+  float* buf = (float*)ws.ex->lane;
+  if (W > 1) {
+    if (w > 0) buf[32 * (w - 1) + lane] = t;
+    team_sync<W>(team);
+    if (w > 0) return 0.0;
+  }
+  float kin = 0.f;
+  if (lane < na) kin += mass * t;
+#pragma unroll
+  for (int a = 1; a < W; ++a) {
+    const int j = lane + 32 * a;
+    if (j < na) kin += L.atom_b[j].z * buf[32 * (a - 1) + lane];
+  }
+  return warp_sum((double)kin);
+}
+
+// One HMC trial of replica r by the calling team: momenta, n_steps of velocity Verlet, the
+// Metropolis test, and the write-back of an accepted trial.  ws: the replica's shared-memory arrays
+// (the zero partner of an odd atom count and the zero slot are already there).
+template <int W, bool TABLE, bool BATCH, int UNROLL>
 __device__ __forceinline__ void hmc_trial(const HmcArgs& A, const LigandLayout& LL, const Lig& L, const WarpSmem& ws,
-                                          int64_t r) {
+                                          int w, int team, int64_t r) {
   const int lane = threadIdx.x & 31;
   float4* xs = ws.xs;
   float* xp = ws.xp;
   const int na = LL.na;
+  const int i = 32 * w + lane;
+  const bool own = i < na;
   const int64_t xstride = BATCH ? A.x_stride : na;
   const int k = A.state_of[r];
   if ((unsigned)k >= (unsigned)A.n_states) {  // invalid state index: leave the replica untouched
-    if (lane == 0) {
+    if (w == 0 && lane == 0) {
       if (A.dH) A.dH[r] = __longlong_as_double(0x7ff8000000000000ll);
       if (A.acc) A.acc[r] = 0;
     }
     return;
   }
-  const StateDev st = A.states[k];
-  const float dt = st.dt, hdt = 0.5f * st.dt;
+  const StateDev* st = A.states + k;
+  const float dt = st->dt, hdt = 0.5f * dt;
+  const float w_sg = st->w_sg_f, w_g = st->w_g_f;
   const uint32_t rid = (uint32_t)(A.rep_offset + r);
+  const float invM = 1.f / LL.total_mass;
+  // below this square the centre of mass is inside the restraint's flat bottom whatever the rounding
+  const float d0_safe2 = LL.d0 > 0.f ? LL.d0 * LL.d0 * 0.999f : 0.f;
 
-  float x[APL][3], v[APL][3], F[APL][3];
-  float mass[APL], accel[APL];  // the lane's atoms' masses and force-to-acceleration factors
-  float kin = 0.f;
-#pragma unroll
-  for (int a = 0; a < APL; ++a) {
-    const int i = lane + 32 * a;
-    if (i < na) {
-      const float* src = A.x + (r * xstride + i) * 3;
-      x[a][0] = src[0];
-      x[a][1] = src[1];
-      x[a][2] = src[2];
-      const U4 o = philox(A.seed, (uint32_t)i, rid, A.cycle, kPurposeMomentum);
-      // Box-Muller: u1 in (0, 1] from 23 bits + 1/2, u2 in [0, 1) from 23 bits (exact in FP32)
-      const float u1 = ((float)(o.x >> 9) + 0.5f) * (1.0f / 8388608.0f);
-      const float u2 = (float)(o.y >> 9) * (1.0f / 8388608.0f);
-      const float u3 = ((float)(o.z >> 9) + 0.5f) * (1.0f / 8388608.0f);
-      const float u4 = (float)(o.w >> 9) * (1.0f / 8388608.0f);
-      const float rr1 = sqrtf(-2.f * logf(u1)), rr2 = sqrtf(-2.f * logf(u3));
-      float s1, c1, s2, c2;
-      sincospif(2.f * u2, &s1, &c1);
-      sincospif(2.f * u4, &s2, &c2);
-      const float4 pb = L.atom_b[i];
-      mass[a] = pb.z;
-      accel[a] = L.atom_a[i].x;
-      const float sd = st.sqrt_kT * pb.w;  // sqrt(kT * 4.184e-4 / m)
-      v[a][0] = rr1 * c1 * sd;
-      v[a][1] = rr1 * s1 * sd;
-      v[a][2] = rr2 * c2 * sd;
-      kin += pb.z * (v[a][0] * v[a][0] + v[a][1] * v[a][1] + v[a][2] * v[a][2]);
-      // the fourth component: the charge for the pair-type loop, R*_i for the table loop (which
-      // reads the partners' positions and radii from the pair-interleaved mirror)
-      xs[i] = make_float4(x[a][0], x[a][1], x[a][2], TABLE ? pb.x : L.atom_a[i].y);
-      if (TABLE) {
-        put_pair_pos(xp, i, x[a][0], x[a][1], x[a][2]);
-        xp[8 * (i >> 1) + 6 + (i & 1)] = pb.x;  // R*_i
-      }
-    } else {
-      x[a][0] = x[a][1] = x[a][2] = 0.f;
-      v[a][0] = v[a][1] = v[a][2] = 0.f;
-      mass[a] = accel[a] = 0.f;
-    }
+  float x[3] = {0.f, 0.f, 0.f}, v[3] = {0.f, 0.f, 0.f}, F[3];
+  float mass = 0.f, accel = 0.f;  // the atom's mass and force-to-acceleration factor
+  // the fourth component: the charge for the pair-type loop, R*_i for the table loop (which
+  // reads the partners' positions and radii from the pair-interleaved mirror)
+  float fourth = 0.f;
+  if (own) {
+    const float* src = A.x + (r * xstride + i) * 3;
+    x[0] = src[0];
+    x[1] = src[1];
+    x[2] = src[2];
+    const U4 o = philox(A.seed, (uint32_t)i, rid, A.cycle, kPurposeMomentum);
+    // Box-Muller: u1 in (0, 1] from 23 bits + 1/2, u2 in [0, 1) from 23 bits (exact in FP32)
+    const float u1 = ((float)(o.x >> 9) + 0.5f) * (1.0f / 8388608.0f);
+    const float u2 = (float)(o.y >> 9) * (1.0f / 8388608.0f);
+    const float u3 = ((float)(o.z >> 9) + 0.5f) * (1.0f / 8388608.0f);
+    const float u4 = (float)(o.w >> 9) * (1.0f / 8388608.0f);
+    const float rr1 = sqrtf(-2.f * logf(u1)), rr2 = sqrtf(-2.f * logf(u3));
+    float s1, c1, s2, c2;
+    sincospif(2.f * u2, &s1, &c1);
+    sincospif(2.f * u4, &s2, &c2);
+    const float4 pb = L.atom_b[i];
+    const float4 pa = L.atom_a[i];
+    mass = pb.z;
+    accel = pa.x;
+    const float sd = st->sqrt_kT * pb.w;  // sqrt(kT * 4.184e-4 / m)
+    v[0] = rr1 * c1 * sd;
+    v[1] = rr1 * s1 * sd;
+    v[2] = rr2 * c2 * sd;
+    fourth = TABLE ? pb.x : pa.y;
+    xs[i] = make_float4(x[0], x[1], x[2], fourth);
+    put_pair_pos(xp, i, x[0], x[1], x[2]);
+    xp[8 * (i >> 1) + 6 + (i & 1)] = fourth;
   }
-  __syncwarp();
+  const double mv0 = team_kinetic<W>(L, na, ws, w, team, mass, v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+  team_sync<W>(team);
   int outside = 0;
   Energies en;
-  double c[4];
-  evaluate<APL, true, TABLE>(LL, L, A.G, xs, ws.sl, x, mass, F, st.w_sg_f, st.w_g_f, true, en, outside, xp);
-  reduce_components(en, c);
-  // the starting components go out now (a rejected trial leaves them); only U0 stays live
-  const double U0 = weighted(c, st.w_sg, st.w_g);
-  if (lane < 4) A.comps[r * 4 + lane] = lane == 0 ? c[0] : (lane == 1 ? c[1] : (lane == 2 ? c[2] : c[3]));
-  double U1 = U0;
-  const double K0 = 0.5 * kKineticToKcal * warp_sum((double)kin);
-  for (int s = 0; s < A.n_steps; ++s) {
-#pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          v[a][d] = fmaf(hdt * accel[a], F[a][d], v[a][d]);
-          x[a][d] = fmaf(dt, v[a][d], x[a][d]);
+  double c[4] = {0.0, 0.0, 0.0, 0.0}, U0 = 0.0, U1 = 0.0;
+  for (int s = 0;; ++s) {  // s steps done up to the force evaluation
+    if (s == 0 || s == A.n_steps) {
+      team_evaluate<W, true, TABLE, 1>(LL, L, A.G, ws, w, team, x, mass, F, w_sg, w_g, invM, d0_safe2,
+                                      en, outside);
+      if (w == 0) {
+        reduce_components(en, c);
+        U1 = weighted(c, st->w_sg, st->w_g);
+        if (s == 0) {  // the starting components go out now (a rejected trial leaves them); only U0 stays live
+          U0 = U1;
+          if (lane < 4) A.comps[r * 4 + lane] = lane == 0 ? c[0] : (lane == 1 ? c[1] : (lane == 2 ? c[2] : c[3]));
         }
       }
-    }
-    __syncwarp();  // all lanes finished reading the previous positions and bonded slots
-#pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na) {
-        float4 p = xs[i];
-        p.x = x[a][0];
-        p.y = x[a][1];
-        p.z = x[a][2];
-        xs[i] = p;
-        if (TABLE) put_pair_pos(xp, i, x[a][0], x[a][1], x[a][2]);
-      }
-    }
-    __syncwarp();
-    if (s + 1 < A.n_steps) {
-      evaluate<APL, false, TABLE>(LL, L, A.G, xs, ws.sl, x, mass, F, st.w_sg_f, st.w_g_f, false, en, outside, xp);
     } else {
-      evaluate<APL, true, TABLE>(LL, L, A.G, xs, ws.sl, x, mass, F, st.w_sg_f, st.w_g_f, true, en, outside, xp);
-      reduce_components(en, c);
-      U1 = weighted(c, st.w_sg, st.w_g);
+      team_evaluate<W, false, TABLE, UNROLL>(LL, L, A.G, ws, w, team, x, mass, F, w_sg, w_g, invM,
+                                            d0_safe2, en, outside);
     }
+    if (own && s > 0) {
 #pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na) {
+      for (int d = 0; d < 3; ++d) v[d] = fmaf(hdt * accel, F[d], v[d]);
+    }
+    if (s == A.n_steps) break;
+    // every warp has finished reading the previous positions (the evaluation's last barrier)
+    if (own) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) v[a][d] = fmaf(hdt * accel[a], F[a][d], v[a][d]);
+      for (int d = 0; d < 3; ++d) {
+        v[d] = fmaf(hdt * accel, F[d], v[d]);
+        x[d] = fmaf(dt, v[d], x[d]);
       }
+      xs[i] = make_float4(x[0], x[1], x[2], fourth);
+      put_pair_pos(xp, i, x[0], x[1], x[2]);
     }
+    team_sync<W>(team);  // positions published; the bonded slots of the last evaluation read
   }
-  kin = 0.f;
-#pragma unroll
-  for (int a = 0; a < APL; ++a) {
-    const int i = lane + 32 * a;
-    if (i < na) kin += mass[a] * (v[a][0] * v[a][0] + v[a][1] * v[a][1] + v[a][2] * v[a][2]);
-  }
-  const double K1 = 0.5 * kKineticToKcal * warp_sum((double)kin);
-  const double dH = (K1 + U1) - (K0 + U0);
-  const U4 o = philox(A.seed, 0u, rid, A.cycle, kPurposeAccept);
-  const double u = uniform53(o.x, o.y);
-  const bool accept = u < exp(-dH / st.kT);
-  if (accept) {  // a rejected trial leaves the stored positions and components as they were
-#pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na) {
-        float* dst = A.x + (r * xstride + i) * 3;
-        dst[0] = x[a][0];
-        dst[1] = x[a][1];
-        dst[2] = x[a][2];
-      }
-    }
-    if (A.n_steps > 0 && lane < 4)
+  const double mv1 = team_kinetic<W>(L, na, ws, w, team, mass, v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+  bool accept = false;
+  if (w == 0) {
+    const double dH = fma(0.5 * kKineticToKcal, mv1, U1) - fma(0.5 * kKineticToKcal, mv0, U0);
+    const U4 o = philox(A.seed, 0u, rid, A.cycle, kPurposeAccept);
+    const double u = uniform53(o.x, o.y);
+    accept = u < exp(-dH / st->kT);
+    if (accept && A.n_steps > 0 && lane < 4)
       A.comps[r * 4 + lane] = lane == 0 ? c[0] : (lane == 1 ? c[1] : (lane == 2 ? c[2] : c[3]));
+    if (lane == 0) {
+      if (A.dH) A.dH[r] = dH;
+      if (A.acc) A.acc[r] = accept ? 1 : 0;
+      if (A.counters) {
+        if (accept) atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_ACCEPTED], 1ull);
+        if (!isfinite(dH)) atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_NONFINITE], 1ull);
+      }
+      if (W > 1) ws.ex->accept = accept;
+    }
   }
-  if (lane == 0) {
-    if (A.dH) A.dH[r] = dH;
-    if (A.acc) A.acc[r] = accept ? 1 : 0;
+  if (W > 1) {
+    team_sync<W>(team);
+    accept = ws.ex->accept;
+  }
+  if (accept && own) {  // a rejected trial leaves the stored positions and components as they were
+    float* dst = A.x + (r * xstride + i) * 3;
+    dst[0] = x[0];
+    dst[1] = x[1];
+    dst[2] = x[2];
   }
   if (A.counters) {
     const int out_total = __reduce_add_sync(kFull, outside);
-    if (lane == 0) {
-      if (accept) atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_ACCEPTED], 1ull);
-      if (!isfinite(dH)) atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_NONFINITE], 1ull);
-      if (out_total) atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_OUTSIDE], (unsigned long long)out_total);
-    }
+    if (lane == 0 && out_total)
+      atomicAdd((unsigned long long*)&A.counters[ALGDOCK_CNT_OUTSIDE], (unsigned long long)out_total);
   }
 }
 
-
-// WPB warps per block; TABLE: the pair table is staged with the blob (16-warp blocks share it).
-// BATCH: the block's ligand and replicas come from its work item (a run of up to WPB replicas of
+// A team of APL warps per replica, one atom per lane; a block holds the ligand's tables and up to
+// SLOTS replicas (blockDim.x / (32 APL) of them, fewer where their shared memory does not fit).
+// MINB blocks per SM.  At 48 atoms two blocks of 6 replicas take 1592 us, one of 12 1685, of 10 1770, of
+// 8 1769, of 16 (64 registers) 1810: more warps wait on the shared-memory pipe (70 % busy) instead.
+// TABLE: the pair table is staged with the blob.
+// BATCH: the block's ligand and replicas come from its work item (a run of consecutive replicas of
 // one ligand of a multi-ligand batch) and positions are stored x_stride atoms apart.
-// Otherwise, with A.work set, the blocks are persistent: each warp takes replicas from the work
+// Otherwise each team runs one replica (team t of block b replica t gridDim.x + b) or, with A.work
+// set, the blocks are persistent: each team takes replicas from the work
 // counter until all n_rep are handed out, highest index first (the coupling leg, whose trials
 // gather the lattices, before the cheaper warming leg), so that no SM idles while another still
-// runs a last wave of blocks.  Which warp runs a replica does not change its result.
-template <int APL, int WPB, bool TABLE, bool BATCH = false>
-__global__ void __launch_bounds__(WPB * 32) hmc_kernel(const HmcArgs A) {
+// runs a last wave of blocks.  Which team runs a replica does not change its result.
+template <int APL, int SLOTS, bool TABLE, bool BATCH = false, int MINB = 1>
+__global__ void __launch_bounds__(SLOTS * APL * 32, MINB) hmc_kernel(const HmcArgs A) {
+  constexpr int kUnroll = APL == 1 ? 4 : (SLOTS * APL > 24 ? 1 : 2);  // of the table pair loop
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ LigandLayout s_ll;
   const uint32_t* blob = A.blob;
-  int64_t r_first = (int64_t)blockIdx.x * WPB;
-  int count = WPB;
   if (BATCH) {
     const BatchItem it = A.items[blockIdx.x];
     if (threadIdx.x == 0) s_ll = A.bligs[it.lig].LL;
     blob = A.blob + A.bligs[it.lig].blob_off;
-    r_first = it.r0;
-    count = it.count;
     __syncthreads();
   }
   const LigandLayout& LL = BATCH ? s_ll : A.LL;
-  const int staged = TABLE ? LL.words_pair : LL.words;
-  stage_ligand(smem, blob, staged);
-  __syncthreads();
+  const int staged = staged_words(LL, TABLE);
+  stage_ligand(smem, blob, TABLE ? LL.words_pair : LL.words);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp >= count) return;
-  const Lig L = bind_ligand(smem, LL);
-  const WarpSmem ws = warp_smem<APL, TABLE>(smem, staged, LL, warp);
+  // A warp's scheduler is its index mod 4.  Teams of two swap their roles every other pair of teams,
+  // so that each scheduler gets as many first warps (more atoms) as last ones.
+  const int team = warp / APL, w = (APL == 2 ? warp + (team >> 1) : warp) % APL;
+  const int slots = (int)blockDim.x / (32 * APL);
   const int na = LL.na;
-  if (TABLE && (na & 1) && lane == 0) {  // the zero partner that completes the last pair
-    put_pair_pos(ws.xp, na, 0.f, 0.f, 0.f);
-    ws.xp[8 * (na >> 1) + 7] = 0.f;
+  const WarpSmem ws = warp_smem<APL, true>(smem + staged + team * replica_words(LL, APL), LL);
+  if (w == 0 && lane == 0) {
+    ws.sl[LL.n_slots] = make_float4(0.f, 0.f, 0.f, 0.f);  // the zero slot
+    if (na & 1) {  // the zero partner that completes the last pair
+      put_pair_pos(ws.xp, na, 0.f, 0.f, 0.f);
+      ws.xp[8 * (na >> 1) + 7] = 0.f;
+    }
   }
-  if (!BATCH && A.work) {
-    for (;;) {
-      unsigned long long t = 0;
-      if (lane == 0) t = atomicAdd(A.work, 1ull);
-      t = __shfl_sync(kFull, t, 0);
-      if (t >= (unsigned long long)A.n_rep) break;
-      __syncwarp();  // the previous trial's reads of the warp's shared arrays are done
-      hmc_trial<APL, TABLE, BATCH>(A, LL, L, ws, A.n_rep - 1 - (int64_t)t);
+  __syncthreads();
+  Lig L = bind_ligand(smem, LL);
+  if (!TABLE) {
+    stage_types(smem, LL, L);
+    __syncthreads();
+  }
+  if (BATCH) {
+    const BatchItem it = A.items[blockIdx.x];
+    for (int j = team; j < it.count; j += slots) {
+      const int64_t r = it.r0 + j;
+      if (r < A.n_rep) hmc_trial<APL, TABLE, BATCH, kUnroll>(A, LL, L, ws, w, team, r);
     }
     return;
   }
-  const int64_t r = r_first + warp;
-  if (r >= A.n_rep) return;
-  hmc_trial<APL, TABLE, BATCH>(A, LL, L, ws, r);
+  if (!A.work) {
+    const int64_t r = (int64_t)team * gridDim.x + blockIdx.x;
+    if (r < A.n_rep) hmc_trial<APL, TABLE, BATCH, kUnroll>(A, LL, L, ws, w, team, r);
+    return;
+  }
+  for (int it = 0;; it ^= 1) {
+    unsigned long long t = 0;
+    if (w == 0 && lane == 0) t = atomicAdd(A.work, 1ull);
+    if (APL == 1) {
+      t = __shfl_sync(kFull, t, 0);
+    } else {  // two words in turn: the next is written while a slow warp may still read this one
+      if (w == 0 && lane == 0) ws.ex->replica[it] = t;
+      team_sync<APL>(team);
+      t = ws.ex->replica[it];
+    }
+    if (t >= (unsigned long long)A.n_rep) break;
+    hmc_trial<APL, TABLE, BATCH, kUnroll>(A, LL, L, ws, w, team, A.n_rep - 1 - (int64_t)t);
+  }
 }
 
 // Energy (and, with force != NULL, force) of stored configurations, one warp each.  With
@@ -873,7 +1190,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
   const int64_t n = (int64_t)blockIdx.x * kWarpsPerBlock + warp;
   if (n >= A.N) return;
   const Lig L = bind_ligand(smem, A.LL);
-  const WarpSmem ws = warp_smem<APL>(smem, A.LL.words, A.LL, warp);
+  const WarpSmem ws = warp_smem<APL, false>(smem + A.LL.words + warp * warp_words(A.LL, APL, false), A.LL);
+  if (lane == 0) ws.sl[A.LL.n_slots] = make_float4(0.f, 0.f, 0.f, 0.f);  // the zero slot
   const int na = A.LL.na;
   float w_sg = 0.f, w_g = 0.f;
   if (A.state_of) {
@@ -899,8 +1217,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
   }
   __syncwarp();
   Energies en;
-  int outside = 0;
-  evaluate<APL, true, false, FORCES>(A.LL, L, A.G, ws.xs, ws.sl, x, mass, F, w_sg, w_g, true, en, outside);
+  evaluate<APL, FORCES>(A.LL, L, A.G, ws.xs, ws.sl, x, mass, F, w_sg, w_g, en);
   double c[4];
   reduce_components(en, c);
   if (FORCES && A.force) {
@@ -1111,8 +1428,22 @@ size_t block_smem(const LigandLayout& L, int apl, int wpb = kWarpsPerBlock, bool
   return ((size_t)(table ? L.words_pair : L.words) + (size_t)wpb * warp_words(L, apl, table)) * 4;
 }
 
-constexpr int kTableWarps = 16;  // warps per block of the pair-table HMC kernel (512 threads, 128 registers)
+constexpr int kTableWarps = 16;  // replicas per block of the pair-table HMC kernel
+// Replicas per block of a one-ligand launch, with and without the pair table, by atoms per lane (warps
+// per team).  Up to 4 replicas per SM of 33-64 atoms take the kernel with 126 registers instead of 80
+// (32 replicas of 48 atoms: 166 us against 193); from there on the one with 24 warps per SM.
+constexpr int kTable1 = 5, kTable2 = 6, kTable2Few = 4, kType1 = 16, kType2 = 4, kType3 = 8;
 constexpr size_t kMaxBlockSmem = 227 * 1024;
+
+// Dynamic shared memory of an HMC block of `slots` replicas, and the most of at most `slots` that a
+// limit holds (at least one).
+size_t team_smem(const LigandLayout& L, int apl, int slots, bool table) {
+  return ((size_t)staged_words(L, table) + (size_t)slots * replica_words(L, apl)) * 4;
+}
+int team_slots(const LigandLayout& L, int apl, int slots, bool table, size_t limit) {
+  while (slots > 1 && team_smem(L, apl, slots, table) > limit) --slots;
+  return slots;
+}
 
 template <typename Kernel, typename Args>
 cudaError_t launch_templated(Kernel k1, Kernel k2, Kernel k3, int apl, size_t smem, int64_t items, cudaStream_t s,
@@ -1137,34 +1468,55 @@ cudaError_t launch_hmc(cudaStream_t s, const algdock_ctx& c, int64_t n_rep, cons
                        int64_t rep_offset, int64_t* counters) {
   if (n_rep == 0) return cudaSuccess;
   HmcArgs A{c.grid, c.lig, c.d_blob, c.d_states, c.K, n_rep, state_of, x, comps, dH, acc, n_steps, seed,
-            (uint32_t)cycle, rep_offset, counters, nullptr, nullptr, 0, c.d_work};
+            (uint32_t)cycle, rep_offset, counters, nullptr, nullptr, 0, nullptr};
   const int apl = atoms_per_lane(c.lig.na);
-  // the pair table where 16-warp blocks can stage it (up to 64 atoms with a small topology);
-  // otherwise the pair-type path in 4-warp blocks
+  // the pair table where a block of 16 replicas can stage it (up to 64 atoms with a small topology);
+  // otherwise the pair-type path
   const bool table = hmc_uses_table(c.lig);
   void (*k)(const HmcArgs);
-  if (table) k = apl == 1 ? hmc_kernel<1, kTableWarps, true> : hmc_kernel<2, kTableWarps, true>;
-  else k = apl == 1 ? hmc_kernel<1, kWarpsPerBlock, false>
-                    : (apl == 2 ? hmc_kernel<2, kWarpsPerBlock, false> : hmc_kernel<3, kWarpsPerBlock, false>);
-  const int wpb = table ? kTableWarps : kWarpsPerBlock;
-  const size_t smem = table ? block_smem(c.lig, apl, kTableWarps, true) : block_smem(c.lig, apl);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int most;
+  int sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
   if (e != cudaSuccess) return e;
-  // persistent blocks: as many as fit on the device at once, never more than the replicas need
-  int per_sm = 0, sms = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, wpb * 32, smem);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+  if (table && apl == 2 && n_rep <= (int64_t)kTable2Few * sms) {
+    k = hmc_kernel<2, kTable2Few, true>;
+    most = kTable2Few;
+  } else if (table) {
+    k = apl == 1 ? hmc_kernel<1, kTable1, true, false, 4> : hmc_kernel<2, kTable2, true, false, 2>;
+    most = apl == 1 ? kTable1 : kTable2;
+  } else {
+    k = apl == 1 ? hmc_kernel<1, kType1, false>
+                 : (apl == 2 ? hmc_kernel<2, kType2, false, false, 2> : hmc_kernel<3, kType3, false>);
+    most = apl == 1 ? kType1 : (apl == 2 ? kType2 : kType3);
+  }
+  int slots = team_slots(c.lig, apl, most, table, kMaxBlockSmem), per_sm = 0;
+  size_t smem = team_smem(c.lig, apl, slots, table);
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, slots * apl * 32, smem);
   if (e != cudaSuccess) return e;
-  const int64_t need = (n_rep + wpb - 1) / wpb;
-  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * sms));
-  e = cudaMemsetAsync(c.d_work, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  k<<<(unsigned)blocks, wpb * 32, smem, s>>>(A);
+  // As many blocks as fit on the device at once.  Replicas that fill their teams once or twice are
+  // spread evenly over them; what fills them more than once comes from the work counter.
+  const int64_t fit = (int64_t)std::max(per_sm, 1) * sms;
+  const int64_t rounds = (n_rep + fit * slots - 1) / (fit * slots);
+  if (rounds <= 2) slots = (int)((n_rep + rounds * fit - 1) / (rounds * fit));
+  smem = team_smem(c.lig, apl, slots, table);
+  if (rounds > 1) {
+    A.work = c.d_work;
+    e = cudaMemsetAsync(c.d_work, 0, sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t blocks = std::min(n_rep, fit);
+  const int threads = slots * apl * 32;
+  k<<<(unsigned)blocks, threads, smem, s>>>(A);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ multi-ligand batches
 size_t batch_block_smem(const LigandLayout& L, int apl, int wpb, bool table) { return block_smem(L, apl, wpb, table); }
+size_t batch_team_smem(const LigandLayout& L, int apl, int slots, bool table) {
+  return team_smem(L, apl, slots, table);
+}
 
 // Launch shapes tried for a class: pair-table blocks of 16 or 8 replicas, or 4-replica blocks
 // without the table (classes 0 and 1); 8-replica table blocks or 4 without (2); 4 or 8 replicas
@@ -1251,7 +1603,8 @@ cudaError_t launch_hmc_batch(cudaStream_t s, const algdock_ctx& c, const int32_t
       if (e != cudaSuccess) break;
     }
     A.items = B.d_items;
-    batch_kernel(kClassApl[k], B.wpb, B.table)<<<(unsigned)B.n_items, B.wpb * 32, B.smem, st>>>(A);
+    batch_kernel(kClassApl[k], B.wpb, B.table)
+        <<<(unsigned)B.n_items, B.slots * kClassApl[k] * 32, B.smem, st>>>(A);
     e = cudaGetLastError();
     if (e == cudaSuccess && n_active > 1) {
       e = cudaEventRecord(c.batch_join[k], st);

@@ -213,10 +213,11 @@ struct BatchLigand {
 struct BatchItem {
   int32_t lig, r0, count, pad;
 };
-// Launch shape of one class: replicas (warps) per block and whether the per-pair table is staged
-// with the blob.
+// Launch shape of one class: replicas per work item, replicas a block runs at a time (fewer where
+// their shared memory does not fit) and whether the per-pair table is staged with the blob.
 struct BatchClass {
   int wpb = 0;
+  int slots = 0;
   bool table = false;
   BatchItem* d_items = nullptr;
   int n_items = 0;
@@ -353,6 +354,8 @@ bool hmc_uses_table(const LigandLayout& L);
 // batches: the block shared memory of a class shape, the candidate shapes of a class, and the
 // HMC trial of every replica of the batch (classes on forked streams, joined on s)
 size_t batch_block_smem(const LigandLayout& L, int apl, int wpb, bool table);
+// the shared memory a block of the class's kernel asks for with `slots` replicas at a time
+size_t batch_team_smem(const LigandLayout& L, int apl, int slots, bool table);
 // Dynamic shared memory a batch kernel of this shape may request on the current device: the
 // per-block opt-in limit less the kernel's static shared memory (0 if the query fails).
 size_t batch_smem_limit(int apl, int wpb, bool table);
