@@ -1715,17 +1715,8 @@ algdock_status algdock_reduced_energies(algdock_ctx* c, int64_t N, const float* 
     return fail(c, ALGDOCK_E_INVALID, "reduced_energies: arrays must be device pointers");
   Device g(c->device);
   cudaError_t e = cudaSuccess;
-  double* tmp = nullptr;
-  double* cp = comps;
-  if (x) {
-    if (!cp) {
-      e = cudaMallocAsync(&tmp, (size_t)N * 4 * sizeof(double), c->stream);
-      cp = tmp;
-    }
-    if (e == cudaSuccess) e = launch_evaluate(c->stream, *c, N, x, cp);
-  }
-  if (e == cudaSuccess && u_kn) e = launch_ukn(c->stream, *c, N, cp, k_begin, k_count, u_kn);
-  if (tmp) cudaFreeAsync(tmp, c->stream);
+  if (x) e = launch_evaluate(c->stream, *c, N, x, comps, k_begin, u_kn ? k_count : 0, u_kn);
+  else if (u_kn) e = launch_ukn(c->stream, *c, N, comps, k_begin, k_count, u_kn);
   if (e != cudaSuccess) return cuda_fail(c, e, "reduced_energies");
   return ALGDOCK_OK;
   ALGDOCK_CATCH(c)

@@ -438,6 +438,59 @@ __device__ inline float3 nonbonded_type_pass(const Lig& L, int na, int base, con
   return make_float3(fx, fy, fz);
 }
 
+// The energies of a pass (full or split) for atom base + lane, partners two at a time, as
+// nonbonded_type_pass: the same terms added to e in the same order as nonbonded_pass.
+__device__ inline void nonbonded_energy_pass(const Lig& L, int na, int base, const float4* xs, const float* xp,
+                                             float& e) {
+  const int lane = threadIdx.x & 31;
+  const int m = na - base, P = (na + 1) >> 1;
+  const bool split = m <= 16;
+  const int i = base + (split ? (lane & 15) : lane);
+  // split: the low half-warp takes j = 0 .. h-1 upwards, the high one j = na-1 .. h downwards; an odd
+  // h leaves each half one partner of the middle pair
+  const int h = (na + 1) >> 1;
+  const bool down = split && lane >= 16;
+  const int cnt = !split ? P : (down ? P - h / 2 : (h + 1) / 2);
+  const int middle = split && (h & 1) ? h / 2 : -1;
+  if (i >= na) return;
+  const float4 own = xs[i];
+  const float2 b = *(const float2*)&L.atom_b[i];
+  const float qc = (float)kCoulomb * own.w;
+  const f32x2 X = pack2(own.x, own.x), Y = pack2(own.y, own.y), Z = pack2(own.z, own.z);
+  const f32x2 Qi = pack2(qc, qc), Ri = pack2(b.x, b.x), Si = pack2(b.y, b.y), minus_two = pack2(-2.f, -2.f);
+  int p = down ? P - 1 : 0;
+  const int step = down ? -1 : 1;
+#pragma unroll 2
+  for (int k = 0; k < cnt; ++k, p += step) {
+    const float4 q0 = ((const float4*)xp)[2 * p];      // (x, x', y, y')
+    const float4 q1 = ((const float4*)xp)[2 * p + 1];  // (z, z', q, q')
+    const float4 s = L.ppar[p];                        // (R*, R*', sqrt(eps), sqrt(eps)')
+    const float4 c = *(const float4*)((const char*)L.scale + L.combo[p * na + i]);
+    const f32x2 dx = sub2(X, pack2(q0.x, q0.y)), dy = sub2(Y, pack2(q0.z, q0.w));
+    const f32x2 dz = sub2(Z, pack2(q1.x, q1.y));
+    float ra, rb;
+    unpack2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ra, rb);
+    ra = c.z == 0.f ? 1.f : ra;  // excluded (also i itself and the partner that completes an odd count)
+    rb = c.w == 0.f ? 1.f : rb;
+    const f32x2 inv_r = pack2(rsqrt_fast(ra), rsqrt_fast(rb));
+    const f32x2 inv_r2 = mul2(inv_r, inv_r);
+    const f32x2 R = add2(Ri, pack2(s.x, s.y));
+    const f32x2 s2 = mul2(mul2(R, R), inv_r2);
+    const f32x2 s6 = mul2(mul2(s2, s2), s2);
+    const f32x2 eps = mul2(pack2(c.x, c.y), mul2(Si, pack2(s.z, s.w)));
+    const f32x2 qq = mul2(pack2(c.z, c.w), mul2(Qi, pack2(q1.z, q1.w)));
+    const f32x2 lj = fma2(s6, s6, mul2(minus_two, s6));
+    float ea, eb;
+    unpack2(fma2(eps, lj, mul2(qq, inv_r)), ea, eb);
+    if (p == middle) {  // the other half-warp's partner adds nothing here
+      ea = down ? 0.f : ea;
+      eb = down ? eb : 0.f;
+    }
+    e += down ? eb : ea;
+    e += down ? ea : eb;
+  }
+}
+
 template <int APL, bool ENERGY, bool FORCES = true>
 __device__ inline void nonbonded(const Lig& L, int na, const float4* xs, float (&F)[APL][3], float& el) {
   const int lane = threadIdx.x & 31;
@@ -570,21 +623,31 @@ __device__ inline void gather_runs(const Lig& L, const LigandLayout& LL, float4*
   }
 }
 
-// Energies (and, with FORCES, the forces on the lane's atoms) of one configuration by one warp, lane l
-// holding atoms l, l+32, l+64.  xs holds all positions (x, y, z, q); sl is the warp's bonded-slot
-// scratch (n_slots + 1 float4, the last zero).
-template <int APL, bool FORCES>
+// Restraint energy of the summed m x.
+__device__ inline float restraint_energy(const LigandLayout& LL, float mx, float my, float mz) {
+  const float invM = 1.f / LL.total_mass;
+  const float dx = mx * invM - LL.site[0], dy = my * invM - LL.site[1], dz = mz * invM - LL.site[2];
+  const float d = sqrtf(dx * dx + dy * dy + dz * dz);
+  if (d > LL.d0) {
+    const float ex = d - LL.d0;
+    return 0.5f * LL.k_rest * ex * ex;
+  }
+  return d <= LL.d0 ? 0.f : d;  // NaN centre of mass: make the energy NaN
+}
+
+// Energies and the forces on the lane's atoms of one configuration by one warp, lane l holding atoms l,
+// l+32, l+64.  xs holds all positions (x, y, z, q); sl is the warp's bonded-slot scratch (n_slots + 1
+// float4, the last zero).
+template <int APL>
 __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const GridDev& G, const float4* xs, float4* sl,
                                 const float (&x)[APL][3], const float (&mass)[APL], float (&F)[APL][3], float w_sg,
                                 float w_g, Energies& en) {
   const int lane = threadIdx.x & 31;
   const int na = LL.na;
-  float el = bonded_terms<true, FORCES>(L, LL, xs, sl, lane, 32);
+  float el = bonded_terms<true>(L, LL, xs, sl, lane, 32);
   __syncwarp();
-  if (FORCES) {
-    gather_runs(L, LL, sl);
-    __syncwarp();
-  }
+  gather_runs(L, LL, sl);
+  __syncwarp();
   float eg = 0.f, esg = 0.f;
   float mx = 0.f, my = 0.f, mz = 0.f;
 #pragma unroll
@@ -596,14 +659,13 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
     mx += mass[a] * x[a][0];
     my += mass[a] * x[a][1];
     mz += mass[a] * x[a][2];
-    const GridOut go = grid_atom(G, x[a][0], x[a][1], x[a][2], pa.z, pa.w, pa.y, true, true, FORCES ? w_sg : 0.f,
-                                 FORCES ? w_g : 0.f);
+    const GridOut go = grid_atom(G, x[a][0], x[a][1], x[a][2], pa.z, pa.w, pa.y, true, true, w_sg, w_g);
     F[a][0] += go.fx;
     F[a][1] += go.fy;
     F[a][2] += go.fz;
     eg += go.e_g;
     esg += go.e_sg;
-    if (FORCES) {  // the atom's partial sums, in run order
+    {  // the atom's partial sums, in run order
       const uint2 p = L.gp[i];
       const float4 q0 = sl[p.x & 0xffffu], q1 = sl[p.x >> 16], q2 = sl[p.y & 0xffffu], q3 = sl[p.y >> 16];
       F[a][0] += ((q0.x + q1.x) + q2.x) + q3.x;
@@ -611,7 +673,7 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
       F[a][2] += ((q0.z + q1.z) + q2.z) + q3.z;
     }
   }
-  nonbonded<APL, true, FORCES>(L, na, xs, F, el);
+  nonbonded<APL, true>(L, na, xs, F, el);
   // restraint on the centre of mass
   mx = warp_sumf(mx);
   my = warp_sumf(my);
@@ -1180,8 +1242,7 @@ struct EvalArgs {
   double* comps;
 };
 
-// FORCES = false: energies only (the bonded force slots, grid gradients and pair forces are skipped).
-template <int APL, bool FORCES>
+template <int APL>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArgs A) {
   extern __shared__ __align__(16) uint32_t smem[];
   stage_ligand(smem, A.blob, A.LL.words);
@@ -1217,10 +1278,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
   }
   __syncwarp();
   Energies en;
-  evaluate<APL, FORCES>(A.LL, L, A.G, ws.xs, ws.sl, x, mass, F, w_sg, w_g, en);
+  evaluate<APL>(A.LL, L, A.G, ws.xs, ws.sl, x, mass, F, w_sg, w_g, en);
   double c[4];
   reduce_components(en, c);
-  if (FORCES && A.force) {
+  {
 #pragma unroll
     for (int a = 0; a < APL; ++a) {
       const int i = lane + 32 * a;
@@ -1233,6 +1294,112 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
     }
   }
   if (A.comps && lane < 4) A.comps[n * 4 + lane] = c[lane];
+}
+
+// Energies only: no bonded force slots, grid gradients or pair forces, so a warp's shared memory is its
+// positions (twice) and 32 warps fit an SM (498 us for 102400 configurations of 48 atoms and their u_kn at
+// 128 states; 24 warps 518, 16 warps 567; 791 with one staging of the ligand per four configurations, one
+// partner at a time and u_kn in a launch of its own).  Persistent blocks stage the ligand once.  A block
+// takes tiles of 8 * per consecutive configurations, `per` to a warp, and, with u_kn, forms their reduced
+// energies at k_count states from k_begin while other blocks evaluate: u_kn is FP64 work (5
+// operations an element on a pipe of 2 lanes per clock, 105 us for 128 x 102400), the evaluation FP32.
+constexpr int kEnergyWarps = 8, kEnergyPer = 4;
+struct EnergyArgs {
+  GridDev G;
+  LigandLayout LL;
+  const uint32_t* blob;
+  const StateDev* states;
+  int64_t N;
+  int per;
+  const float* x;
+  double* comps;  // may be NULL with u_kn
+  double* u_kn;   // may be NULL
+  int k_begin, k_count;
+};
+
+template <int APL>
+__global__ void __launch_bounds__(kEnergyWarps * 32, 4) energy_kernel(const EnergyArgs A) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ double s_c[kEnergyWarps * kEnergyPer][4];
+  const LigandLayout& LL = A.LL;
+  const int na = LL.na;
+  stage_ligand(smem, A.blob, LL.words);
+  __syncthreads();
+  Lig L = bind_ligand(smem, LL);
+  stage_types(smem, LL, L);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float4* xs = (float4*)(smem + staged_words(LL, false) + warp * 8 * 32 * APL);
+  float* xp = (float*)(xs + 32 * APL);
+  if ((na & 1) && lane == 0) {  // the zero partner that completes the last pair
+    put_pair_pos(xp, na, 0.f, 0.f, 0.f);
+    xp[8 * (na >> 1) + 7] = 0.f;
+  }
+  __syncthreads();
+  const int tile_n = kEnergyWarps * A.per, shift = 31 - __clz(tile_n);  // a power of two
+  const int64_t tiles = (A.N + tile_n - 1) / tile_n;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    for (int j = 0; j < A.per; ++j) {
+      const int slot = warp * A.per + j;
+      const int64_t n = tile * tile_n + slot;
+      if (n >= A.N) break;
+      __syncwarp();  // the previous configuration's reads are done
+      float mx = 0.f, my = 0.f, mz = 0.f, eg = 0.f, esg = 0.f;
+#pragma unroll
+      for (int a = 0; a < APL; ++a) {
+        const int i = lane + 32 * a;
+        if (i >= na) continue;
+        const float* src = A.x + (n * na + i) * 3;
+        const float x = src[0], y = src[1], z = src[2], q = L.atom_a[i].y;
+        xs[i] = make_float4(x, y, z, q);
+        put_pair_pos(xp, i, x, y, z);
+        xp[8 * (i >> 1) + 6 + (i & 1)] = q;
+      }
+      __syncwarp();
+      float el = bonded_terms<true, false>(L, LL, xs, nullptr, lane, 32);
+#pragma unroll
+      for (int a = 0; a < APL; ++a) {
+        const int i = lane + 32 * a;
+        if (i >= na) continue;
+        const float4 p = xs[i], pa = L.atom_a[i];
+        const float m = L.atom_b[i].z;
+        mx += m * p.x;
+        my += m * p.y;
+        mz += m * p.z;
+        const GridOut go = grid_atom(A.G, p.x, p.y, p.z, pa.z, pa.w, pa.y, true, true, 0.f, 0.f);
+        eg += go.e_g;
+        esg += go.e_sg;
+      }
+      float e2 = 0.f;
+#pragma unroll
+      for (int a = 0; a < APL; ++a)
+        if (32 * a < na) nonbonded_energy_pass(L, na, 32 * a, xs, xp, e2);
+      el += 0.5f * e2;
+      Energies en;
+      en.lig = el;
+      en.sg = esg;
+      en.g = eg;
+      mx = warp_sumf(mx);
+      my = warp_sumf(my);
+      mz = warp_sumf(mz);
+      en.rest = lane == 0 ? restraint_energy(LL, mx, my, mz) : 0.f;
+      double c[4];
+      reduce_components(en, c);
+      if (lane < 4) {
+        const double v = lane == 0 ? c[0] : (lane == 1 ? c[1] : (lane == 2 ? c[2] : c[3]));
+        if (A.comps) A.comps[n * 4 + lane] = v;
+        s_c[slot][lane] = v;
+      }
+    }
+    if (!A.u_kn) continue;
+    __syncthreads();
+    for (int e = threadIdx.x; e < tile_n * A.k_count; e += kEnergyWarps * 32) {
+      const int k = e >> shift, slot = e & (tile_n - 1);
+      const int64_t n = tile * tile_n + slot;
+      const StateDev& st = A.states[A.k_begin + k];
+      if (n < A.N) A.u_kn[(int64_t)k * A.N + n] = __dmul_rn(st.beta, weighted(s_c[slot], st.w_sg, st.w_g));
+    }
+    __syncthreads();
+  }
 }
 
 // External-coordinate moves ("Sampling"): for a replica whose state has alpha < alpha_max, n_moves
@@ -1614,25 +1781,35 @@ cudaError_t launch_hmc_batch(cudaStream_t s, const algdock_ctx& c, const int32_t
   return e;
 }
 
-static cudaError_t launch_eval(cudaStream_t s, const algdock_ctx& c, int64_t N, const int32_t* state_of,
-                               const float* x, float* force, double* comps) {
+// Components of N configurations (comps, or NULL) and, with u_kn, their reduced energies at k_count
+// states from k_begin.
+cudaError_t launch_evaluate(cudaStream_t s, const algdock_ctx& c, int64_t N, const float* x, double* comps, int k_begin,
+                            int k_count, double* u_kn) {
   if (N == 0) return cudaSuccess;
-  EvalArgs A{c.grid, c.lig, c.d_blob, c.d_states, c.K, N, state_of, x, force, comps};
   const int apl = atoms_per_lane(c.lig.na);
-  if (force)
-    return launch_templated(eval_kernel<1, true>, eval_kernel<2, true>, eval_kernel<3, true>, apl,
-                            block_smem(c.lig, apl), N, s, A);
-  return launch_templated(eval_kernel<1, false>, eval_kernel<2, false>, eval_kernel<3, false>, apl,
-                          block_smem(c.lig, apl), N, s, A);
-}
-
-cudaError_t launch_evaluate(cudaStream_t s, const algdock_ctx& c, int64_t N, const float* x, double* comps) {
-  return launch_eval(s, c, N, nullptr, x, nullptr, comps);
+  void (*k)(const EnergyArgs) = apl == 1 ? energy_kernel<1> : (apl == 2 ? energy_kernel<2> : energy_kernel<3>);
+  const size_t smem = 4 * ((size_t)staged_words(c.lig, false) + (size_t)kEnergyWarps * 8 * 32 * apl);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int per_sm = 0, sms = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kEnergyWarps * 32, smem);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+  if (e != cudaSuccess) return e;
+  const int64_t fit = (int64_t)std::max(per_sm, 1) * sms;
+  // several configurations per warp (longer rows of u_kn) once every block still has a few tiles
+  const int per = N >= 4 * fit * kEnergyWarps * kEnergyPer ? kEnergyPer : 1;
+  const int64_t tiles = (N + kEnergyWarps * per - 1) / (kEnergyWarps * per);
+  const EnergyArgs A{c.grid, c.lig, c.d_blob, c.d_states, N, per, x, comps, k_count > 0 ? u_kn : nullptr, k_begin,
+                     k_count};
+  k<<<(unsigned)std::min(tiles, fit), kEnergyWarps * 32, smem, s>>>(A);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_energy_force(cudaStream_t s, const algdock_ctx& c, int64_t N, const int32_t* state_of,
                                 const float* x, float* force, double* comps) {
-  return launch_eval(s, c, N, state_of, x, force, comps);
+  if (N == 0) return cudaSuccess;
+  EvalArgs A{c.grid, c.lig, c.d_blob, c.d_states, c.K, N, state_of, x, force, comps};
+  const int apl = atoms_per_lane(c.lig.na);
+  return launch_templated(eval_kernel<1>, eval_kernel<2>, eval_kernel<3>, apl, block_smem(c.lig, apl), N, s, A);
 }
 
 cudaError_t launch_external(cudaStream_t s, const algdock_ctx& c, int64_t n_rep, const int32_t* state_of, float* x,

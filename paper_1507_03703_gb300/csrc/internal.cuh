@@ -348,7 +348,8 @@ cudaError_t launch_gather_probe(cudaStream_t s, const algdock_ctx& c, int64_t n_
 cudaError_t launch_hmc(cudaStream_t s, const algdock_ctx& c, int64_t n_rep, const int32_t* state_of, float* x,
                        double* comps, double* dH, uint8_t* acc, int n_steps, uint64_t seed, uint64_t cycle,
                        int64_t rep_offset, int64_t* counters);
-cudaError_t launch_evaluate(cudaStream_t s, const algdock_ctx& c, int64_t N, const float* x, double* comps);
+cudaError_t launch_evaluate(cudaStream_t s, const algdock_ctx& c, int64_t N, const float* x, double* comps,
+                            int k_begin = 0, int k_count = 0, double* u_kn = nullptr);
 // the one-ligand HMC launch shape: 16-replica blocks with the pair table staged, else 4 without
 bool hmc_uses_table(const LigandLayout& L);
 // batches: the block shared memory of a class shape, the candidate shapes of a class, and the
