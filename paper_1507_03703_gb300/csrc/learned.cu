@@ -233,8 +233,10 @@ cudaError_t gemm_wgrad(cudaStream_t s, int M, int N, int K, const TA* A, int lda
 // mma.sync m16n8k16 through ldmatrix.  Eight warps split the output columns: 32 each in the hidden
 // layers, 48 in the output layer.  Rounding is that of the layer-by-layer GEMMs: BF16 inputs and
 // hidden activations, FP32 accumulation.
-constexpr int FM = 16;               // rows per CTA
-constexpr int F_MT = FM / 16;        // m16 row tiles per warp
+// MT: m16 row tiles per CTA.  One tile spreads up to 16 x 152 rows over all SMs (one CTA each: the
+// weight ring fills an SM's shared memory); above that two tiles halve the passes over the weights,
+// which is what a CTA waits for.
+constexpr int F_MAX_MT = 2;
 constexpr int FKC = 64;              // input columns per weight chunk
 constexpr int FWS = FKC + 8;         // padded row of a weight chunk (bf16): conflict-free ldmatrix
 constexpr int FHS = NHID + 8;        // padded row of a hidden activation tile
@@ -246,14 +248,16 @@ constexpr int F_CH0 = NFEAT / FKC;   // chunks of the input layer
 constexpr int F_CHH = NHID / FKC;    // chunks of each later layer
 constexpr int F_NCHUNK = F_CH0 + 3 * F_CHH;
 constexpr int F_STAGE_ELEMS = F_NOUT_ROWS * FWS;
-constexpr size_t F_SMEM = (size_t)(F_STAGES * F_STAGE_ELEMS + 2 * FM * FHS + FM * FXS) * sizeof(bf16);
+constexpr size_t f_smem_bytes(int mt) {
+  return (size_t)(F_STAGES * F_STAGE_ELEMS + 2 * 16 * mt * FHS + 16 * mt * FXS) * sizeof(bf16);
+}
 // packed weights: chunks of the three 256-row layers, then the four chunks of the 360-row layer
 constexpr int F_CHUNK_H = NHID * FWS;                // elements of a 256-row chunk
 constexpr int F_CHUNK_O = NOUT * FWS;                // elements of a 360-row chunk
 constexpr int F_NCHUNK_H = F_CH0 + 2 * F_CHH;        // chunks of 256 rows
 constexpr int F_PACKED = F_NCHUNK_H * F_CHUNK_H + F_CHH * F_CHUNK_O;
 static_assert(NFEAT % FKC == 0 && NHID % FKC == 0, "whole chunks");
-static_assert(F_SMEM <= 227 * 1024, "shared memory of one CTA");
+static_assert(f_smem_bytes(F_MAX_MT) <= 227 * 1024, "shared memory of one CTA");
 static_assert((F_CHUNK_H * 2) % 16 == 0 && (F_CHUNK_O * 2) % 16 == 0 && (F_STAGE_ELEMS * 2) % 16 == 0,
               "bulk copies move multiples of 16 bytes between 16-byte aligned addresses");
 constexpr long long kMbarSpinLimit = 1ll << 22;      // bounded waits (well over a second in all)
@@ -336,7 +340,9 @@ __global__ void pack_weights_kernel(const bf16* __restrict__ W, bf16* Wp) {
   Wp[e] = col < FKC ? W[woff + row * k_in + kc * FKC + col] : __float2bfloat16(0.f);
 }
 
+template <int F_MT>
 __global__ void __launch_bounds__(F_WARPS * 32) mlp_fused_kernel(const FusedArgs P) {
+  constexpr int FM = 16 * F_MT;  // rows per CTA
   extern __shared__ __align__(16) unsigned char f_smem[];
   __shared__ __align__(8) uint64_t full[F_STAGES];
   bf16* const Wst = (bf16*)f_smem;
@@ -852,38 +858,49 @@ struct MoveArgs {
   int t_eff;         // moved torsions (<= topo.T); the mixture uses 6 + t_eff dimensions
 };
 
-// Draw d ~ q(. | x), y = Apply(x, d), log q(d | x).  One warp per replica.
+// Draw d ~ q(. | x), y = Apply(x, d), log q(d | x).  One warp per replica; the first warp draws the
+// components of the block's four replicas, eight lanes each, because an FP64 instruction costs the
+// same for four replicas as for one (64 cycles a warp: the draws were a third of this kernel).
 template <int APL>
 __global__ void sample_apply_kernel(const MoveArgs A, const float* __restrict__ x, float* y, float* delta,
                                     double* logq) {
   __shared__ float s_pos[4][96 * 3];
   __shared__ float s_dl[4][DMAX];
+  __shared__ int s_comp[4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * 4 + warp;
-  if (r >= A.n_rep) return;
   const int na = A.P.LL.na, T = A.t_eff, D = 6 + T;
   const float* o = A.out + r * NOUT;
   const uint32_t rid = (uint32_t)(A.rep_offset + r);
-  // component: cumulative softmax in FP64 against a 53-bit uniform, the weights computed one per
-  // lane and summed in component order (every lane walks the same sum)
-  const float m8 = warp8_max(o[lane & 7]);
-  const double w = lane < NCOMP ? exp((double)o[lane] - (double)m8) : 0.0;
-  double z = 0.0;
+  if (warp == 0) {
+    // component: cumulative softmax in FP64 against a 53-bit uniform, the weights computed one per
+    // lane and summed in component order
+    const int j = lane >> 3;
+    const bool in = r + j < A.n_rep;
+    const float v = in ? o[j * NOUT + (lane & 7)] : 0.f;
+    const float m8 = warp8_max(v);
+    const double w = exp((double)v - (double)m8);
+    double z = 0.0;
 #pragma unroll
-  for (int c = 0; c < NCOMP; ++c) z += __shfl_sync(kFull, w, c);
-  const U4 ru = philox(A.seed, 100u, rid, A.ctr, kPurposeLearned);
-  const double u = uniform53(ru.x, ru.y) * z;
-  int comp = NCOMP - 1;
-  bool found = false;
-  double cum = 0.0;
+    for (int c = 0; c < NCOMP; ++c) z += __shfl_sync(kFull, w, 8 * j + c);
+    const U4 ru = philox(A.seed, 100u, rid + j, A.ctr, kPurposeLearned);
+    const double u = uniform53(ru.x, ru.y) * z;
+    int comp = NCOMP - 1;
+    bool found = false;
+    double cum = 0.0;
 #pragma unroll
-  for (int c = 0; c < NCOMP; ++c) {
-    cum += __shfl_sync(kFull, w, c);
-    if (!found && u < cum) {
-      comp = c;
-      found = true;
+    for (int c = 0; c < NCOMP; ++c) {
+      cum += __shfl_sync(kFull, w, 8 * j + c);
+      if (!found && u < cum) {
+        comp = c;
+        found = true;
+      }
     }
+    if ((lane & 7) == 0) s_comp[j] = comp;
   }
+  __syncthreads();
+  if (r >= A.n_rep) return;
+  const int comp = s_comp[warp];
   if (lane < D) {
     const U4 rr = philox(A.seed, (uint32_t)lane, rid, A.ctr, kPurposeLearned);
     const float u1 = ((float)(rr.x >> 9) + 0.5f) * (1.0f / 8388608.0f);
@@ -960,42 +977,56 @@ __device__ inline double weighted_u(const double* c, double w_sg, double w_g) {
   return e;
 }
 
-// log q(-d | x'), the acceptance test, and the copy of accepted moves.  One warp per replica.
+// log q(-d | x'), the acceptance test, and the copy of accepted moves (with the network's outputs at
+// the new pose, out_x, unless it is NULL).  One warp per replica; the block's four FP64 tests run in the
+// lanes of one warp.
 template <int APL>
 __global__ void accept_kernel(const MoveArgs A, const float* __restrict__ y, const double* __restrict__ comps_y,
                               const float* __restrict__ delta, const double* __restrict__ logq_f, float* x,
-                              double* comps, int32_t* accepted, int64_t* counters) {
+                              double* comps, float* out_x, int32_t* accepted, int64_t* counters) {
   __shared__ float s_dl[4][DMAX];
+  __shared__ float s_lq[4];
+  __shared__ int s_acc[4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * 4 + warp;
-  if (r >= A.n_rep) return;
   const int na = A.P.LL.na, D = 6 + A.t_eff;
-  const int k = A.state_of[r];
-  if ((unsigned)k >= (unsigned)A.n_states) return;
-  if (lane < DMAX) s_dl[warp][lane] = -delta[r * DMAX + lane];
-  __syncwarp();
-  const double lqr = (double)mixture_terms(A.out + r * NOUT, D, s_dl[warp], lane).lq;
-  const StateDev st = A.states[k];
-  const double du = st.beta * (weighted_u(comps_y + r * 4, st.w_sg, st.w_g) - weighted_u(comps + r * 4, st.w_sg, st.w_g));
-  const double lr = (lqr - logq_f[r]) - du;
-  const U4 rr = philox(A.seed, 101u, (uint32_t)(A.rep_offset + r), A.ctr, kPurposeLearned);
-  const bool acc = uniform53(rr.x, rr.y) < exp(lr);
-  if (acc) {
+  if (r < A.n_rep) {
+    if (lane < DMAX) s_dl[warp][lane] = -delta[r * DMAX + lane];
+    __syncwarp();
+    const float lq = mixture_terms(A.out + r * NOUT, D, s_dl[warp], lane).lq;
+    if (lane == 0) s_lq[warp] = lq;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    const int64_t q = (int64_t)blockIdx.x * 4 + threadIdx.x;
+    const int k = q < A.n_rep ? A.state_of[q] : -1;
+    bool acc = false;
+    if ((unsigned)k < (unsigned)A.n_states) {
+      const StateDev& st = A.states[k];
+      const double du =
+          st.beta * (weighted_u(comps_y + q * 4, st.w_sg, st.w_g) - weighted_u(comps + q * 4, st.w_sg, st.w_g));
+      const double lr = ((double)s_lq[threadIdx.x] - logq_f[q]) - du;
+      const U4 rr = philox(A.seed, 101u, (uint32_t)(A.rep_offset + q), A.ctr, kPurposeLearned);
+      acc = uniform53(rr.x, rr.y) < exp(lr);
+      if (acc && accepted) accepted[q] += 1;
+      if (counters) {
+        if (acc) atomicAdd((unsigned long long*)&counters[ALGDOCK_CNT_ACCEPTED], 1ull);
+        if (!isfinite(lr)) atomicAdd((unsigned long long*)&counters[ALGDOCK_CNT_NONFINITE], 1ull);
+      }
+    }
+    s_acc[threadIdx.x] = acc;
+  }
+  __syncthreads();
+  if (!s_acc[warp]) return;
 #pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na)
-        for (int d = 0; d < 3; ++d) x[(r * na + i) * 3 + d] = y[(r * na + i) * 3 + d];
-    }
-    if (lane < 4) comps[r * 4 + lane] = comps_y[r * 4 + lane];
+  for (int a = 0; a < APL; ++a) {
+    const int i = lane + 32 * a;
+    if (i < na)
+      for (int d = 0; d < 3; ++d) x[(r * na + i) * 3 + d] = y[(r * na + i) * 3 + d];
   }
-  if (lane == 0) {
-    if (acc && accepted) accepted[r] += 1;
-    if (counters) {
-      if (acc) atomicAdd((unsigned long long*)&counters[ALGDOCK_CNT_ACCEPTED], 1ull);
-      if (!isfinite(lr)) atomicAdd((unsigned long long*)&counters[ALGDOCK_CNT_NONFINITE], 1ull);
-    }
-  }
+  if (lane < 4) comps[r * 4 + lane] = comps_y[r * 4 + lane];
+  if (out_x)
+    for (int c = lane; c < NOUT; c += 32) out_x[r * NOUT + c] = A.out[r * NOUT + c];
 }
 
 PoseArgs pose_args(const algdock_ctx& c) { return PoseArgs{c.lig, c.d_blob, c.ltopo}; }
@@ -1135,7 +1166,10 @@ static bool fused_ready(const float* feat) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
   if (done[dev].load(std::memory_order_acquire) == 1) return true;
-  if (cudaFuncSetAttribute(mlp_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM) != cudaSuccess) {
+  if (cudaFuncSetAttribute(mlp_fused_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f_smem_bytes(1)) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(mlp_fused_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f_smem_bytes(2)) !=
+          cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1150,7 +1184,8 @@ static cudaError_t forward_run(cudaStream_t s, const float* params, const bf16* 
   const int n = (int)N;
   if (fused_ready(feat)) {
     FusedArgs P{params, Wp, n, feat, out, keep ? h1 : nullptr, keep ? h2 : nullptr, keep ? h3 : nullptr};
-    mlp_fused_kernel<<<(unsigned)((N + FM - 1) / FM), F_WARPS * 32, F_SMEM, s>>>(P);
+    if (N > 16 * 152) mlp_fused_kernel<2><<<(unsigned)((N + 31) / 32), F_WARPS * 32, f_smem_bytes(2), s>>>(P);
+    else mlp_fused_kernel<1><<<(unsigned)((N + 15) / 16), F_WARPS * 32, f_smem_bytes(1), s>>>(P);
     return cudaGetLastError();
   }
   cudaError_t e = gemm<float, false, bf16, false, EPI_RELU_BF16>(s, n, NHID, NFEAT, feat, NFEAT, W + WOFF_1, NFEAT, h1,
@@ -1313,11 +1348,11 @@ cudaError_t learned_adam(cudaStream_t s, float* params, uint16_t* wbf16, const f
   return cudaGetLastError();
 }
 
-// Scratch of one learned move: features, packed weights and h1..h3, outputs, y, delta, log q,
-// components of y.
+// Scratch of one learned move: features, packed weights and h1..h3, outputs at x and at y, y, delta,
+// log q, components of y.
 size_t learned_propose_scratch(int64_t R, int na) {
   return align256((size_t)R * NFEAT * sizeof(float)) + learned_forward_scratch(R) +
-         align256((size_t)R * NOUT * sizeof(float)) + align256((size_t)R * na * 3 * sizeof(float)) +
+         2 * align256((size_t)R * NOUT * sizeof(float)) + align256((size_t)R * na * 3 * sizeof(float)) +
          align256((size_t)R * DMAX * sizeof(float)) + align256((size_t)R * sizeof(double)) +
          align256((size_t)R * 4 * sizeof(double));
 }
@@ -1333,7 +1368,9 @@ cudaError_t learned_propose(cudaStream_t s, const algdock_ctx& c, const float* p
   p += align256((size_t)R * NFEAT * sizeof(float));
   void* fwd = p;
   p += learned_forward_scratch(R);
-  float* out = (float*)p;
+  float* out_x = (float*)p;
+  p += align256((size_t)R * NOUT * sizeof(float));
+  float* out_y = (float*)p;
   p += align256((size_t)R * NOUT * sizeof(float));
   float* y = (float*)p;
   p += align256((size_t)R * na * 3 * sizeof(float));
@@ -1344,24 +1381,28 @@ cudaError_t learned_propose(cudaStream_t s, const algdock_ctx& c, const float* p
   double* comps_y = (double*)p;
   const int apl = na <= 32 ? 1 : (na <= 64 ? 2 : 3);
   const unsigned blocks = (unsigned)((R + 3) / 4);
-  cudaError_t e = cudaSuccess;
+  // the network's outputs at the current poses: once, then those at y where a move was accepted
+  cudaError_t e = learned_features(s, c, R, state_of, x, comps, feat);
+  if (e == cudaSuccess) e = forward_scratch(s, params, wbf16, R, feat, out_x, fwd, true);
   for (int mv = 0; mv < n_moves && e == cudaSuccess; ++mv) {
-    MoveArgs A{pose_args(c), c.d_states, c.K, R, state_of, out, seed, (uint32_t)(cycle * (uint64_t)n_moves + mv),
+    MoveArgs A{pose_args(c), c.d_states, c.K, R, state_of, out_x, seed, (uint32_t)(cycle * (uint64_t)n_moves + mv),
                rep_offset, t_eff};
-    e = learned_features(s, c, R, state_of, x, comps, feat);
-    if (e == cudaSuccess) e = forward_scratch(s, params, wbf16, R, feat, out, fwd, mv == 0);
-    if (e != cudaSuccess) break;
     if (apl == 1) sample_apply_kernel<1><<<blocks, 128, 0, s>>>(A, x, y, delta, logq);
     else if (apl == 2) sample_apply_kernel<2><<<blocks, 128, 0, s>>>(A, x, y, delta, logq);
     else sample_apply_kernel<3><<<blocks, 128, 0, s>>>(A, x, y, delta, logq);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_evaluate(s, c, R, y, comps_y);
     if (e == cudaSuccess) e = learned_features(s, c, R, state_of, y, comps_y, feat);
-    if (e == cudaSuccess) e = forward_scratch(s, params, wbf16, R, feat, out, fwd, false);
+    if (e == cudaSuccess) e = forward_scratch(s, params, wbf16, R, feat, out_y, fwd, false);
     if (e != cudaSuccess) break;
-    if (apl == 1) accept_kernel<1><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, accepted, counters);
-    else if (apl == 2) accept_kernel<2><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, accepted, counters);
-    else accept_kernel<3><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, accepted, counters);
+    A.out = out_y;
+    float* keep = mv + 1 < n_moves ? out_x : nullptr;
+    if (apl == 1)
+      accept_kernel<1><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, keep, accepted, counters);
+    else if (apl == 2)
+      accept_kernel<2><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, keep, accepted, counters);
+    else
+      accept_kernel<3><<<blocks, 128, 0, s>>>(A, y, comps_y, delta, logq, x, comps, keep, accepted, counters);
     e = cudaGetLastError();
   }
   return e;
