@@ -1402,6 +1402,18 @@ __global__ void __launch_bounds__(kEnergyWarps * 32, 4) energy_kernel(const Ener
   }
 }
 
+// u < exp(z), decided by an FP32 exponential where it is clear: at |z| <= 40 that is within 1e-5 of
+// exp(z), and an FP64 exponential is some 30 dependent FP64 instructions.
+__device__ inline bool below_exp(double u, double z) {
+  if (z >= 0.0) return u < 1.0 || u < exp(z);
+  if (z > -40.0) {
+    const float e = expf((float)z), v = (float)u;
+    if (v < 0.9999f * e) return true;
+    if (v > 1.0001f * e) return false;
+  }
+  return u < exp(z);
+}
+
 // External-coordinate moves ("Sampling"): for a replica whose state has alpha < alpha_max, n_moves
 // moves, each a uniformly random rotation about the centre of mass (the unit quaternion of three
 // uniforms by Shoemake's construction) and a Gaussian translation of sigma per dimension, accepted
@@ -1465,30 +1477,50 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) external_kernel(const Ext
   const double u0 = weighted(c0, st.w_sg, st.w_g);
   int n_acc = 0, outside = 0;
   double u_cur = u0;
+  // Few replicas take these moves (one of 128 states at paper scale), so a launch waits for one
+  // warp's chain of moves.  Out of that chain: the moves' random numbers (one move per lane, 32 at a
+  // time), the FP64 exponential, the wait for one pass's lattice loads before the next pass's.  20
+  // moves of 64 replicas of 48 atoms: 143 -> 68 us.
+  float rot[9], shift_s[2], shift_c[3];  // rotation; the translation's products sigma r and their cosines
+  double uni = 0.0;                      // accept uniform
   for (int mv = 0; mv < A.n_moves; ++mv) {
-    const uint32_t ctr = (uint32_t)(A.cycle * (uint64_t)A.n_moves + (uint64_t)mv);
-    // rotation
-    const U4 rq = philox(A.seed, 0u, rid, ctr, kPurposeExternal);
-    const float u1 = (float)(rq.x >> 9) * (1.0f / 8388608.0f);
-    const float u2 = (float)(rq.y >> 9) * (1.0f / 8388608.0f);
-    const float u3 = (float)(rq.z >> 9) * (1.0f / 8388608.0f);
-    const float s1 = sqrtf(1.f - u1), s2 = sqrtf(u1);
-    float sn2, cs2, sn3, cs3;
-    sincospif(2.f * u2, &sn2, &cs2);
-    sincospif(2.f * u3, &sn3, &cs3);
-    const float qx = s1 * sn2, qy = s1 * cs2, qz = s2 * sn3, qw = s2 * cs3;
-    const float R00 = 1.f - 2.f * (qy * qy + qz * qz), R01 = 2.f * (qx * qy - qz * qw), R02 = 2.f * (qx * qz + qy * qw);
-    const float R10 = 2.f * (qx * qy + qz * qw), R11 = 1.f - 2.f * (qx * qx + qz * qz), R12 = 2.f * (qy * qz - qx * qw);
-    const float R20 = 2.f * (qx * qz - qy * qw), R21 = 2.f * (qy * qz + qx * qw), R22 = 1.f - 2.f * (qx * qx + qy * qy);
-    // translation: Box-Muller on 23-bit uniforms, as for the momenta
-    const U4 rt = philox(A.seed, 1u, rid, ctr, kPurposeExternal);
-    const float ua = ((float)(rt.x >> 9) + 0.5f) * (1.0f / 8388608.0f), ub = (float)(rt.y >> 9) * (1.0f / 8388608.0f);
-    const float uc = ((float)(rt.z >> 9) + 0.5f) * (1.0f / 8388608.0f), ud = (float)(rt.w >> 9) * (1.0f / 8388608.0f);
-    float sb, cb, sd_, cd;
-    sincospif(2.f * ub, &sb, &cb);
-    sincospif(2.f * ud, &sd_, &cd);
-    const float ra = sqrtf(-2.f * logf(ua)), rc = sqrtf(-2.f * logf(uc));
-    const float tx = A.sigma * ra * cb, ty = A.sigma * ra * sb, tz = A.sigma * rc * cd;
+    if ((mv & 31) == 0 && mv + lane < A.n_moves) {
+      const uint32_t ctr = (uint32_t)(A.cycle * (uint64_t)A.n_moves + (uint64_t)(mv + lane));
+      // rotation
+      const U4 rq = philox(A.seed, 0u, rid, ctr, kPurposeExternal);
+      const float u1 = (float)(rq.x >> 9) * (1.0f / 8388608.0f);
+      const float u2 = (float)(rq.y >> 9) * (1.0f / 8388608.0f);
+      const float u3 = (float)(rq.z >> 9) * (1.0f / 8388608.0f);
+      const float s1 = sqrtf(1.f - u1), s2 = sqrtf(u1);
+      float sn2, cs2, sn3, cs3;
+      sincospif(2.f * u2, &sn2, &cs2);
+      sincospif(2.f * u3, &sn3, &cs3);
+      const float qx = s1 * sn2, qy = s1 * cs2, qz = s2 * sn3, qw = s2 * cs3;
+      rot[0] = 1.f - 2.f * (qy * qy + qz * qz), rot[1] = 2.f * (qx * qy - qz * qw), rot[2] = 2.f * (qx * qz + qy * qw);
+      rot[3] = 2.f * (qx * qy + qz * qw), rot[4] = 1.f - 2.f * (qx * qx + qz * qz), rot[5] = 2.f * (qy * qz - qx * qw);
+      rot[6] = 2.f * (qx * qz - qy * qw), rot[7] = 2.f * (qy * qz + qx * qw), rot[8] = 1.f - 2.f * (qx * qx + qy * qy);
+      // translation: Box-Muller on 23-bit uniforms, as for the momenta
+      const U4 rt = philox(A.seed, 1u, rid, ctr, kPurposeExternal);
+      const float ua = ((float)(rt.x >> 9) + 0.5f) * (1.0f / 8388608.0f), ub = (float)(rt.y >> 9) * (1.0f / 8388608.0f);
+      const float uc = ((float)(rt.z >> 9) + 0.5f) * (1.0f / 8388608.0f), ud = (float)(rt.w >> 9) * (1.0f / 8388608.0f);
+      float sb, cb, sd_, cd;
+      sincospif(2.f * ub, &sb, &cb);
+      sincospif(2.f * ud, &sd_, &cd);
+      shift_s[0] = A.sigma * sqrtf(-2.f * logf(ua)), shift_s[1] = A.sigma * sqrtf(-2.f * logf(uc));
+      shift_c[0] = cb, shift_c[1] = sb, shift_c[2] = cd;
+      const U4 ra4 = philox(A.seed, 2u, rid, ctr, kPurposeExternal);
+      uni = uniform53(ra4.x, ra4.y);
+    }
+    const int src = mv & 31;
+    const float R00 = __shfl_sync(kFull, rot[0], src), R01 = __shfl_sync(kFull, rot[1], src),
+                R02 = __shfl_sync(kFull, rot[2], src), R10 = __shfl_sync(kFull, rot[3], src),
+                R11 = __shfl_sync(kFull, rot[4], src), R12 = __shfl_sync(kFull, rot[5], src),
+                R20 = __shfl_sync(kFull, rot[6], src), R21 = __shfl_sync(kFull, rot[7], src),
+                R22 = __shfl_sync(kFull, rot[8], src);
+    const float sab = __shfl_sync(kFull, shift_s[0], src), scd = __shfl_sync(kFull, shift_s[1], src);
+    const float tx = sab * __shfl_sync(kFull, shift_c[0], src), ty = sab * __shfl_sync(kFull, shift_c[1], src),
+                tz = scd * __shfl_sync(kFull, shift_c[2], src);
+    const double u_acc = __shfl_sync(kFull, uni, src);
     // centre of mass, moved pose, its grid terms and restraint
     float cx = 0.f, cy = 0.f, cz = 0.f;
 #pragma unroll
@@ -1509,15 +1541,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) external_kernel(const Ext
       y[a][0] = cx + (R00 * vx + R01 * vy + R02 * vz) + tx;
       y[a][1] = cy + (R10 * vx + R11 * vy + R12 * vz) + ty;
       y[a][2] = cz + (R20 * vx + R21 * vy + R22 * vz) + tz;
-      if (lane + 32 * a < na) {
-        const GridOut go = grid_atom(A.G, y[a][0], y[a][1], y[a][2], sA[a], sB[a], q[a], true, true, 0.f, 0.f);
-        eg += go.e_g;
-        esg += go.e_sg;
-        out_mv += go.outside ? 1 : 0;
-        mx += m[a] * y[a][0];
-        my += m[a] * y[a][1];
-        mz += m[a] * y[a][2];
-      }
+      // without a branch, so that the lattice loads of all passes are in flight together
+      const bool own = lane + 32 * a < na;
+      const GridOut go = grid_atom(A.G, y[a][0], y[a][1], y[a][2], sA[a], sB[a], q[a], true, true, 0.f, 0.f);
+      eg += own ? go.e_g : 0.f;
+      esg += own ? go.e_sg : 0.f;
+      out_mv += own && go.outside ? 1 : 0;
+      mx += m[a] * y[a][0];
+      my += m[a] * y[a][1];
+      mz += m[a] * y[a][2];
     }
     mx = warp_sumf(mx);
     my = warp_sumf(my);
@@ -1534,11 +1566,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) external_kernel(const Ext
     double c1[4];
     c1[0] = c0[0];
     c1[1] = (double)er;
-    c1[2] = warp_sum((double)esg);
-    c1[3] = warp_sum((double)eg);
+    // both grid sums over the warp: the butterfly's pairs, one of the two sums per lane
+    const bool high = lane & 16;
+    double v = (double)(high ? eg : esg) + __shfl_xor_sync(kFull, (double)(high ? esg : eg), 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    c1[2] = __shfl_sync(kFull, v, 0);
+    c1[3] = __shfl_sync(kFull, v, 16);
     const double u1e = weighted(c1, st.w_sg, st.w_g);
-    const U4 ra4 = philox(A.seed, 2u, rid, ctr, kPurposeExternal);
-    const bool acc = uniform53(ra4.x, ra4.y) < exp(-st.beta * (u1e - u_cur));
+    const bool acc = below_exp(u_acc, -st.beta * (u1e - u_cur));
     outside += out_mv;
     if (acc) {
 #pragma unroll
