@@ -881,6 +881,13 @@ algdock_status algdock_create(int device, uint64_t seed, const algdock_params* p
     delete c;
     return ALGDOCK_E_OOM;
   }
+  if (cudaStreamCreateWithFlags(&c->leg_side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->leg_fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->leg_join, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    algdock_destroy(c);
+    return ALGDOCK_E_CUDA;
+  }
   *out = c;
   return ALGDOCK_OK;
 }
@@ -912,6 +919,9 @@ void algdock_destroy(algdock_ctx* c) {
   cudaFree(c->d_stage);
   cudaFree(c->d_rbuf);
   if (c->cycle_side) cudaStreamDestroy(c->cycle_side);
+  if (c->leg_side) cudaStreamDestroy(c->leg_side);
+  if (c->leg_fork) cudaEventDestroy(c->leg_fork);
+  if (c->leg_join) cudaEventDestroy(c->leg_join);
   if (c->cycle_fork) cudaEventDestroy(c->cycle_fork);
   if (c->cycle_join) cudaEventDestroy(c->cycle_join);
   delete c;
@@ -2044,13 +2054,22 @@ algdock_status algdock_cycle(algdock_ctx* c, const algdock_run_desc* d, uint64_t
   if (e == cudaSuccess && side) e = cudaEventRecord(c->cycle_join, snap_s);
   base = 0;
   NvtxRange rx("algdock_cycle: exchange");
+  // The legs are independent, and the sweeps of one leg are a chain of phases that leaves most of the GPU
+  // idle (one block per ladder): every other leg runs on a second stream.  64 ladders of 32 and of 96
+  // states take 51 and 70 us after one another, 72 beside each other.
+  const bool two = d->n_legs > 1;
+  if (e == cudaSuccess && two) e = cudaEventRecord(c->leg_fork, c->stream);
+  if (e == cudaSuccess && two) e = cudaStreamWaitEvent(c->leg_side, c->leg_fork, 0);
   for (int l = 0; l < d->n_legs && e == cudaSuccess; ++l) {
-    e = launch_exchange(c->stream, *c, d->n_chains, d->K[l], d->state_offset[l], dc + 4 * base, dcfg + cbase,
-                        ds + base, d->n_sweeps, d->max_sep, d->seed, cycle, d->ladder_offset + (int64_t)l * d->n_chains,
-                        nullptr, nullptr);
+    e = launch_exchange(l % 2 ? c->leg_side : c->stream, *c, d->n_chains, d->K[l], d->state_offset[l], dc + 4 * base,
+                        dcfg + cbase, ds + base, d->n_sweeps, d->max_sep, d->seed, cycle,
+                        d->ladder_offset + (int64_t)l * d->n_chains, nullptr, nullptr);
     base += (int64_t)d->n_chains * d->K[l];
     cbase += (int64_t)d->n_chains * d->K[l];
   }
+  if (e == cudaSuccess && two) e = cudaEventRecord(c->leg_join, c->leg_side);
+  if (e == cudaSuccess && two) e = cudaStreamWaitEvent(c->stream, c->leg_join, 0);
+  if (e != cudaSuccess && two) cudaStreamSynchronize(c->leg_side);  // nothing of a failed call stays in flight
   if (e == cudaSuccess && side) e = cudaStreamWaitEvent(c->stream, c->cycle_join, 0);
   const bool checks = c->params.checks != 0;
   if (e == cudaSuccess && checks) {

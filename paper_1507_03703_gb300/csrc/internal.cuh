@@ -275,6 +275,9 @@ struct algdock_ctx {
   bool host_coherent = false;
   cudaStream_t cycle_side = nullptr;
   cudaEvent_t cycle_fork = nullptr, cycle_join = nullptr;
+  // the stream on which algdock_cycle sweeps every other leg's ladders
+  cudaStream_t leg_side = nullptr;
+  cudaEvent_t leg_fork = nullptr, leg_join = nullptr;
   // the context's seed and the method's adjustable arguments (algdock_create, algdock_set_params)
   uint64_t seed = 0;
   algdock_params params{};
