@@ -403,13 +403,34 @@ cudaError_t learned_pose_delta(cudaStream_t s, const algdock_ctx& c, int64_t N, 
 // partial tiles C + z M ldc.  *err (device int) is set if a bounded wait runs out.
 bool umma_supported(int device);
 cudaError_t umma_gemm(cudaStream_t s, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,
-                      int ldc, int epi, const float* bias, const void* mask, int ldm, int n_split, int* err);
+                      int ldc, int epi, const float* bias, const void* mask, int ldm, int n_split, int* err,
+                      void* CT = nullptr, int ldt = 0);
 int umma_split_count(int K, int n_split);
-cudaError_t transpose_to_bf16(cudaStream_t s, int rows, int cols, const void* in, int ld_in, bool in_f32, void* out,
-                              int ld_out);
+// Split products C_z = A_z . B_z^T (FP32 partial products [slices][M][N] each, as umma_gemm's) of one
+// reduction length K in one launch, and BF16 copies (transposed or not) of several matrices in one.
+constexpr int kUmmaGroupMax = 4, kCopyGroupMax = 5;
+struct UmmaProduct {
+  int M, N;
+  const void* A;
+  int lda;
+  const void* B;
+  int ldb;
+  float* C;
+};
+cudaError_t umma_group(cudaStream_t s, int n, const UmmaProduct* p, int K, int n_split, int* err);
+struct CopyTask {
+  const void* in;
+  int rows, cols, ld_in;
+  bool f32, transpose;
+  void* out;
+  int ld_out;
+};
+cudaError_t copy_group(cudaStream_t s, int n, const CopyTask* t);
 // Rows from which the learned network's gradient and forward pass run on tcgen05 (with tc_err set):
-// measured against the mma.sync kernels on one GB300, the gradient ties at 4096 rows and wins from
-// 8192 (2.2x at 65536); the forward ties at 8192 and wins from 16384 (1.6x at 65536).
+// measured against the mma.sync kernels on one GB300, the gradient takes 139 us at 4096 rows (with an
+// Adam step) against about 255 and 1075 at 65536 against 2350 (before its launches were grouped); the
+// forward ties at 8192 and wins from 16384 (1.6x at 65536).  The two paths round differently, so the
+// lines stay where they were set.
 constexpr int64_t kTcMinRowsGrad = 4096;
 constexpr int64_t kTcMinRowsForward = 8192;
 size_t learned_forward_scratch(int64_t N);

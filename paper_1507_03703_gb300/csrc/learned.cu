@@ -498,6 +498,78 @@ cudaError_t colsum(cudaStream_t s, int M, int N, const T* G, float* out, float* 
   return cudaGetLastError();
 }
 
+// The sums that close a gradient on the tensor-core path, of all four layers at once.  First the
+// column sums of the layers' output gradients (as colsum_kernel; block x = kColsumBlocks adds up the
+// loss, as sum_kernel), then the slices of weight products and column sums, in the order of the
+// parameter vector.
+constexpr int kColsumOut = (NOUT + 31) / 32, kColsumHid = NHID / 32, kColsumBlocks = kColsumOut + 3 * kColsumHid;
+struct GradSums {
+  int n, nz;                  // rows, slices of the weight products
+  const float* g4;            // output gradients of layers 4 (FP32), 3, 2, 1
+  const bf16 *g3, *g2, *g1;
+  float *w4, *w3, *w2, *w1;   // weight products [nz][M][N]
+  float* b;                   // column sums [kColsumSlices][NOUT + 3 NHID]: layers 4, 3, 2, 1
+  const float* lrow;          // loss rows
+  float* loss;                // may be NULL
+  float* grad;
+};
+
+__device__ inline void sum_rows(int64_t N, const float* __restrict__ x, float scale, float* out);
+
+__global__ void grad_colsum_kernel(const GradSums A) {
+  __shared__ float ws[8][32];
+  int bx = blockIdx.x;
+  if (bx == kColsumBlocks) {
+    if (blockIdx.y == 0 && A.loss) sum_rows(A.n, A.lrow, 1.f / (float)A.n, A.loss);
+    return;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int len = (A.n + kColsumSlices - 1) / kColsumSlices;
+  const int mb = blockIdx.y * len, me = min(A.n, mb + len);
+  float s = 0.f;
+  int col, N;
+  if (bx < kColsumOut) {
+    col = bx * 32 + lane;
+    N = NOUT;
+    if (col < N)
+      for (int m = mb + warp; m < me; m += 8) s += A.g4[(size_t)m * N + col];
+  } else {
+    bx -= kColsumOut;
+    const bf16* g = bx < kColsumHid ? A.g3 : (bx < 2 * kColsumHid ? A.g2 : A.g1);
+    col = bx % kColsumHid * 32 + lane;
+    N = NHID;
+    for (int m = mb + warp; m < me; m += 8) s += __bfloat162float(g[(size_t)m * N + col]);
+  }
+  ws[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && col < N) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += ws[w][lane];
+    const int off = (int)blockIdx.x < kColsumOut ? 0 : NOUT + bx / kColsumHid * NHID;
+    A.b[(size_t)blockIdx.y * (NOUT + 3 * NHID) + off + col] = t;
+  }
+}
+
+__global__ void grad_reduce_kernel(const GradSums A) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= NPARAMS) return;
+  const float* part;
+  size_t stride = NHID * NHID;
+  int nz = A.nz;
+  constexpr int nb = NOUT + 3 * NHID;
+  if (p < OFF_B1) part = A.w1 + p, stride = NHID * NFEAT;
+  else if (p < OFF_W2) part = A.b + NOUT + 2 * NHID + (p - OFF_B1), stride = nb, nz = kColsumSlices;
+  else if (p < OFF_B2) part = A.w2 + (p - OFF_W2);
+  else if (p < OFF_W3) part = A.b + NOUT + NHID + (p - OFF_B2), stride = nb, nz = kColsumSlices;
+  else if (p < OFF_B3) part = A.w3 + (p - OFF_W3);
+  else if (p < OFF_W4) part = A.b + NOUT + (p - OFF_B3), stride = nb, nz = kColsumSlices;
+  else if (p < OFF_B4) part = A.w4 + (p - OFF_W4), stride = NOUT * NHID;
+  else part = A.b + (p - OFF_B4), stride = nb, nz = kColsumSlices;
+  float s = 0.f;
+  for (int z = 0; z < nz; ++z) s += part[z * stride];
+  A.grad[p] = s;
+}
+
 // Weight entries (not biases) of the parameter vector, in the order of the BF16 copy.
 __device__ inline int weight_index(int p) {
   if (p < OFF_B1) return WOFF_1 + p;
@@ -611,7 +683,8 @@ __global__ void nll_kernel(int64_t N, int D, const float* __restrict__ out, cons
   if (lane == 0) loss_rows[n] = -t.lq;
 }
 
-__global__ void sum_kernel(int64_t N, const float* __restrict__ x, float scale, float* out) {
+// out = scale * sum of x, by one block of 256 threads.
+__device__ inline void sum_rows(int64_t N, const float* __restrict__ x, float scale, float* out) {
   __shared__ float sh[256];
   float s = 0.f;
   for (int64_t i = threadIdx.x; i < N; i += blockDim.x) s += x[i];
@@ -622,6 +695,9 @@ __global__ void sum_kernel(int64_t N, const float* __restrict__ x, float scale, 
     __syncthreads();
   }
   if (threadIdx.x == 0) *out = scale * sh[0];
+}
+__global__ void sum_kernel(int64_t N, const float* __restrict__ x, float scale, float* out) {
+  sum_rows(N, x, scale, out);
 }
 
 // ------------------------------------------------------------------ features, targets
@@ -1133,20 +1209,19 @@ __global__ void to_bf16_kernel(int64_t n, const float* __restrict__ in, bf16* ou
 }
 
 // The four layers as tcgen05 GEMMs with fused epilogues (BF16 hidden activations, FP32 outputs).
-static cudaError_t forward_tc(cudaStream_t s, const float* params, const bf16* W, int64_t N, const float* feat,
-                              float* out, bf16* f16, bf16* h1, bf16* h2, bf16* h3, int* err) {
+// t1..t3 (may be NULL): also the hidden activations transposed, [256][ldt].
+static cudaError_t forward_tc(cudaStream_t s, const float* params, const bf16* W, int64_t N, float* out,
+                              const bf16* f16, bf16* h1, bf16* h2, bf16* h3, int* err, bf16* t1 = nullptr,
+                              bf16* t2 = nullptr, bf16* t3 = nullptr, int ldt = 0) {
   const int n = (int)N;
-  to_bf16_kernel<<<(unsigned)((N * NFEAT + 255) / 256), 256, 0, s>>>(N * NFEAT, feat, f16);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = umma_gemm(s, n, NHID, NFEAT, f16, NFEAT, W + WOFF_1, NFEAT, h1, NHID, EPI_RELU_BF16, params + OFF_B1, nullptr,
-                  0, 1, err);
+  cudaError_t e = umma_gemm(s, n, NHID, NFEAT, f16, NFEAT, W + WOFF_1, NFEAT, h1, NHID, EPI_RELU_BF16, params + OFF_B1,
+                            nullptr, 0, 1, err, t1, ldt);
   if (e == cudaSuccess)
     e = umma_gemm(s, n, NHID, NHID, h1, NHID, W + WOFF_2, NHID, h2, NHID, EPI_RELU_BF16, params + OFF_B2, nullptr, 0, 1,
-                  err);
+                  err, t2, ldt);
   if (e == cudaSuccess)
     e = umma_gemm(s, n, NHID, NHID, h2, NHID, W + WOFF_3, NHID, h3, NHID, EPI_RELU_BF16, params + OFF_B3, nullptr, 0, 1,
-                  err);
+                  err, t3, ldt);
   if (e == cudaSuccess)
     e = umma_gemm(s, n, NOUT, NHID, h3, NHID, W + WOFF_4, NHID, out, NOUT, EPI_F32_BIAS, params + OFF_B4, nullptr, 0, 1,
                   err);
@@ -1211,9 +1286,13 @@ static cudaError_t forward_scratch(cudaStream_t s, const float* params, const ui
   bf16* Wp = (bf16*)p;
   p += packed_bytes();
   const size_t hb = align256((size_t)N * NHID * sizeof(bf16));
-  if (use_tc(N, tc_err, kTcMinRowsForward))
-    return forward_tc(s, params, (const bf16*)wbf16, N, feat, out, (bf16*)(p + 3 * hb), (bf16*)p, (bf16*)(p + hb),
-                      (bf16*)(p + 2 * hb), tc_err);
+  if (use_tc(N, tc_err, kTcMinRowsForward)) {
+    bf16* f16 = (bf16*)(p + 3 * hb);
+    to_bf16_kernel<<<(unsigned)((N * NFEAT + 255) / 256), 256, 0, s>>>(N * NFEAT, feat, f16);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return forward_tc(s, params, (const bf16*)wbf16, N, out, f16, (bf16*)p, (bf16*)(p + hb), (bf16*)(p + 2 * hb), tc_err);
+  }
   if (pack) {
     const cudaError_t e = pack_weights(s, (const bf16*)wbf16, Wp);
     if (e != cudaSuccess) return e;
@@ -1231,36 +1310,24 @@ cudaError_t learned_forward(cudaStream_t s, const float* params, const uint16_t*
 // rows, and the split partial products of the weight gradients.
 static int64_t pad8(int64_t n) { return (n + 7) / 8 * 8; }
 
+// The tensor-core path's: BF16 features, one more input gradient, the transposed operands of the
+// weight products (features, h1..h3; output gradients of layers 1..4), transposed weights, the products'
+// slices and the column sums'.
+static size_t grad_tc_scratch(int64_t N) {
+  const size_t np = (size_t)pad8(N);
+  return align256((size_t)N * NFEAT * sizeof(bf16)) + align256((size_t)N * NHID * sizeof(bf16)) +
+         align256(NFEAT * np * sizeof(bf16)) + 6 * align256(NHID * np * sizeof(bf16)) +
+         align256(NOUT * np * sizeof(bf16)) + align256((size_t)NHID * NOUT * sizeof(bf16)) +
+         2 * align256((size_t)NHID * NHID * sizeof(bf16)) +
+         align256((size_t)kWgradSplit * NWEIGHTS * sizeof(float)) +
+         align256((size_t)kColsumSlices * (NOUT + 3 * NHID) * sizeof(float));
+}
+
 size_t learned_grad_scratch(int64_t N) {
   return 5 * align256((size_t)N * NHID * sizeof(bf16)) + 2 * align256((size_t)N * NOUT * sizeof(float)) +
          align256((size_t)N * NOUT * sizeof(bf16)) + align256((size_t)N * sizeof(float)) +
          align256((size_t)kWgradSplit * NOUT * NHID * sizeof(float)) + packed_bytes() +
-         // the tensor-core path: operands transposed for the weight gradients, a transposed weight
-         // matrix and the BF16 features
-         align256((size_t)NOUT * pad8(N) * sizeof(bf16)) + align256((size_t)NHID * pad8(N) * sizeof(bf16)) +
-         align256((size_t)NHID * NOUT * sizeof(bf16)) + align256((size_t)N * NFEAT * sizeof(bf16));
-}
-
-// Weight gradient C[M][N] = sum_n A[n][M] B[n][N] on tcgen05: both factors transposed to K-major
-// ([M][n] and [N][n]), the batch split into FP32 partial products summed in slice order.
-static cudaError_t wgrad_tc(cudaStream_t s, int M, int N, int n, const void* A, int lda, bool a_f32, const void* B,
-                            int ldb, bool b_f32, float* C, float* part, bf16* TA, bf16* TB, int* err) {
-  const int np = (int)pad8(n);
-  cudaError_t e = transpose_to_bf16(s, n, M, A, lda, a_f32, TA, np);
-  if (e == cudaSuccess) e = transpose_to_bf16(s, n, N, B, ldb, b_f32, TB, np);
-  if (e == cudaSuccess) e = umma_gemm(s, M, N, n, TA, np, TB, np, part, N, EPI_F32, nullptr, nullptr, 0, kWgradSplit, err);
-  if (e != cudaSuccess) return e;
-  const int nz = umma_split_count(n, kWgradSplit);
-  splitk_reduce_kernel<<<(M * N + 255) / 256, 256, 0, s>>>(M * N, nz, part, C);
-  return cudaGetLastError();
-}
-
-// Input gradient dX[n][N] = (dY[n][K] . W[K][N]) masked by H > 0, on tcgen05 with W transposed.
-static cudaError_t dgrad_tc(cudaStream_t s, int n, int N, int K, const bf16* dY, const bf16* W, const bf16* H, bf16* dX,
-                            bf16* WT, int* err) {
-  cudaError_t e = transpose_to_bf16(s, K, N, W, N, false, WT, K);
-  if (e == cudaSuccess) e = umma_gemm(s, n, N, K, dY, K, WT, K, dX, N, EPI_MASK_BF16, nullptr, H, N, 1, err);
-  return e;
+         (N >= kTcMinRowsGrad ? grad_tc_scratch(N) : 0);
 }
 
 cudaError_t learned_grad(cudaStream_t s, const float* params, const uint16_t* wbf16, int64_t N, const float* feat,
@@ -1283,33 +1350,55 @@ cudaError_t learned_grad(cudaStream_t s, const float* params, const uint16_t* wb
   bf16* Wp = (bf16*)((char*)part + align256((size_t)kWgradSplit * NOUT * NHID * sizeof(float)));
   const int n = (int)N;
   if (use_tc(N, tc_err, kTcMinRowsGrad)) {
+    // Thirteen launches, each a few microseconds of latency at 4096 rows: the hidden activations and the
+    // input gradients leave their products transposed as well, and the four layers' weight
+    // products, column sums and slice sums share a launch each.  A gradient and an Adam step at 4096
+    // rows: 139 us, 244 with 46 launches (a transpose per operand, four of each closing sum).
+    const int np = (int)pad8(N);
     char* q = (char*)Wp + packed_bytes();
-    bf16* TA = (bf16*)q;
-    q += align256((size_t)NOUT * pad8(N) * sizeof(bf16));
-    bf16* TB = (bf16*)q;
-    q += align256((size_t)NHID * pad8(N) * sizeof(bf16));
-    bf16* WT = (bf16*)q;
-    q += align256((size_t)NHID * NOUT * sizeof(bf16));
-    bf16* f16 = (bf16*)q;
-    cudaError_t e = forward_tc(s, params, W, N, feat, out, f16, h1, h2, h3, tc_err);
+    auto take = [&](size_t elems) {
+      bf16* r = (bf16*)q;
+      q += align256(elems * sizeof(bf16));
+      return r;
+    };
+    bf16 *f16 = take((size_t)N * NFEAT), *dC = take((size_t)N * NHID), *Tf = take((size_t)NFEAT * np);
+    bf16 *Th1 = take((size_t)NHID * np), *Th2 = take((size_t)NHID * np), *Th3 = take((size_t)NHID * np);
+    bf16 *Td1 = take((size_t)NHID * np), *Td2 = take((size_t)NHID * np), *Td3 = take((size_t)NHID * np);
+    bf16 *Td4 = take((size_t)NOUT * np), *WT4 = take((size_t)NHID * NOUT), *WT3 = take((size_t)NHID * NHID),
+         *WT2 = take((size_t)NHID * NHID);
+    float* w4 = (float*)q;
+    float *w3 = w4 + (size_t)kWgradSplit * NOUT * NHID, *w2 = w3 + (size_t)kWgradSplit * NHID * NHID,
+          *w1 = w2 + (size_t)kWgradSplit * NHID * NHID;
+    q += align256((size_t)kWgradSplit * NWEIGHTS * sizeof(float));
+    const CopyTask prep[5] = {{feat, n, NFEAT, NFEAT, true, false, f16, NFEAT},
+                              {feat, n, NFEAT, NFEAT, true, true, Tf, np},
+                              {W + WOFF_4, NOUT, NHID, NHID, false, true, WT4, NOUT},
+                              {W + WOFF_3, NHID, NHID, NHID, false, true, WT3, NHID},
+                              {W + WOFF_2, NHID, NHID, NHID, false, true, WT2, NHID}};
+    cudaError_t e = copy_group(s, 5, prep);
+    if (e == cudaSuccess) e = forward_tc(s, params, W, N, out, f16, h1, h2, h3, tc_err, Th1, Th2, Th3, np);
     if (e != cudaSuccess) return e;
     nll_kernel<<<(unsigned)((N + 3) / 4), 128, 0, s>>>(N, D, out, delta, dout, dout16, lrow);
-    if (loss) sum_kernel<<<1, 256, 0, s>>>(N, lrow, 1.f / (float)N, loss);
-    e = wgrad_tc(s, NOUT, NHID, n, dout16, NOUT, false, h3, NHID, false, grad + OFF_W4, part, TA, TB, tc_err);
-    if (e == cudaSuccess) e = colsum<float>(s, n, NOUT, dout, grad + OFF_B4, part);
-    if (e == cudaSuccess) e = dgrad_tc(s, n, NHID, NOUT, dout16, W + WOFF_4, h3, dA, WT, tc_err);
-    if (e == cudaSuccess) e = wgrad_tc(s, NHID, NHID, n, dA, NHID, false, h2, NHID, false, grad + OFF_W3, part, TA, TB,
-                                       tc_err);
-    if (e == cudaSuccess) e = colsum<bf16>(s, n, NHID, dA, grad + OFF_B3, part);
-    if (e == cudaSuccess) e = dgrad_tc(s, n, NHID, NHID, dA, W + WOFF_3, h2, dB, WT, tc_err);
-    if (e == cudaSuccess) e = wgrad_tc(s, NHID, NHID, n, dB, NHID, false, h1, NHID, false, grad + OFF_W2, part, TA, TB,
-                                       tc_err);
-    if (e == cudaSuccess) e = colsum<bf16>(s, n, NHID, dB, grad + OFF_B2, part);
-    if (e == cudaSuccess) e = dgrad_tc(s, n, NHID, NHID, dB, W + WOFF_2, h1, dA, WT, tc_err);
-    if (e == cudaSuccess) e = wgrad_tc(s, NHID, NFEAT, n, dA, NHID, false, feat, NFEAT, true, grad + OFF_W1, part, TA,
-                                       TB, tc_err);
-    if (e == cudaSuccess) e = colsum<bf16>(s, n, NHID, dA, grad + OFF_B1, part);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const CopyTask post{dout16, n, NOUT, NOUT, false, true, Td4, np};
+    e = copy_group(s, 1, &post);
+    // input gradients dX[n][N] = (dY[n][K] . W[K][N]) masked by H > 0
+    auto dgrad = [&](int K, const bf16* dY, const bf16* WT, const bf16* H, bf16* dX, bf16* TX) {
+      return umma_gemm(s, n, NHID, K, dY, K, WT, K, dX, NHID, EPI_MASK_BF16, nullptr, H, NHID, 1, tc_err, TX, np);
+    };
+    if (e == cudaSuccess) e = dgrad(NOUT, dout16, WT4, h3, dA, Td3);
+    if (e == cudaSuccess) e = dgrad(NHID, dA, WT3, h2, dB, Td2);
+    if (e == cudaSuccess) e = dgrad(NHID, dB, WT2, h1, dC, Td1);
+    // weight gradients dY^T X, the batch split into FP32 partial products summed in slice order
+    const UmmaProduct prod[4] = {{NOUT, NHID, Td4, np, Th3, np, w4},
+                                 {NHID, NHID, Td3, np, Th2, np, w3},
+                                 {NHID, NHID, Td2, np, Th1, np, w2},
+                                 {NHID, NFEAT, Td1, np, Tf, np, w1}};
+    if (e == cudaSuccess) e = umma_group(s, 4, prod, n, kWgradSplit, tc_err);
+    if (e != cudaSuccess) return e;
+    const GradSums S{n, umma_split_count(n, kWgradSplit), dout, dA, dB, dC, w4, w3, w2, w1, (float*)q, lrow, loss, grad};
+    grad_colsum_kernel<<<dim3(kColsumBlocks + 1, kColsumSlices), 256, 0, s>>>(S);
+    grad_reduce_kernel<<<(NPARAMS + 255) / 256, 256, 0, s>>>(S);
+    return cudaGetLastError();
   }
   cudaError_t e = pack_weights(s, W, Wp);
   if (e == cudaSuccess) e = forward_run(s, params, W, Wp, N, feat, out, h1, h2, h3, true);

@@ -118,6 +118,8 @@ struct UmmaArgs {
   int k_len;         // K per blockIdx.z slice (a multiple of kUBK)
   size_t c_zstride;  // FP32 partial tiles: element offset between slices
   int* err;
+  bf16* CT;          // BF16 epilogues: also the transposed result [N][ldt], or NULL
+  int ldt;
 };
 
 template <int BN>
@@ -125,9 +127,10 @@ constexpr size_t umma_smem() {
   return 1024 + (size_t)kStages * (kUM + BN) * kUBK * 2 + 256;
 }
 
+// Tile (bx, by) of slice bz.
 template <int BN, int EPI>
-__global__ void __launch_bounds__(128, 1)
-    umma_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, const UmmaArgs P) {
+__device__ __forceinline__ void umma_tile(const CUtensorMap& tA, const CUtensorMap& tB, const UmmaArgs& P, int bx, int by,
+                                          int bz) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
@@ -137,8 +140,8 @@ __global__ void __launch_bounds__(128, 1)
   uint64_t* done = empty + kStages;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kUM, n0 = blockIdx.x * BN;
-  const int kb = blockIdx.z * P.k_len;
+  const int m0 = by * kUM, n0 = bx * BN;
+  const int kb = bz * P.k_len;
   const int ke = min(P.K, kb + P.k_len);
   const int nk = ke > kb ? (ke - kb + kUBK - 1) / kUBK : 0;
   if (threadIdx.x == 0) {
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(128, 1)
   }
   fence_after();
   const int row = m0 + 32 * warp + lane;
-  float* Cf = (float*)P.C + (size_t)blockIdx.z * P.c_zstride;
+  float* Cf = (float*)P.C + (size_t)bz * P.c_zstride;
   bf16* Cb = (bf16*)P.C;
   // vector epilogue: 16-byte aligned rows of C (and of the mask and the bias where they are read)
   const int esz = (EPI == 0 || EPI == 1) ? 4 : 2;
@@ -254,6 +257,10 @@ __global__ void __launch_bounds__(128, 1)
         uint4* dst = (uint4*)(Cb + (size_t)row * P.ldc + col0);
         dst[0] = out[0];
         dst[1] = out[1];
+        if (P.CT) {  // a warp's 32 rows are consecutive in each column
+#pragma unroll
+          for (int j = 0; j < 16; ++j) P.CT[(size_t)(col0 + j) * P.ldt + row] = oh[j];
+        }
       }
       continue;
     }
@@ -265,11 +272,11 @@ __global__ void __launch_bounds__(128, 1)
       if (EPI == 1 || EPI == 2) x += P.bias[col];
       if (EPI == 0 || EPI == 1) {
         Cf[(size_t)row * P.ldc + col] = x;
-      } else if (EPI == 2) {
-        Cb[(size_t)row * P.ldc + col] = __float2bfloat16(x > 0.f ? x : 0.f);
       } else {
-        const float h = __bfloat162float(P.mask[(size_t)row * P.ldm + col]);
-        Cb[(size_t)row * P.ldc + col] = __float2bfloat16(h > 0.f ? x : 0.f);
+        const float h = EPI == 2 ? x : __bfloat162float(P.mask[(size_t)row * P.ldm + col]);
+        const bf16 r = __float2bfloat16(h > 0.f ? x : 0.f);
+        Cb[(size_t)row * P.ldc + col] = r;
+        if (P.CT) P.CT[(size_t)col * P.ldt + row] = r;
       }
     }
   }
@@ -285,24 +292,55 @@ __global__ void __launch_bounds__(128, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((uint32_t)BN) : "memory");
 }
 
-// Out[c][r] = In[r][c] for BF16 (or FP32 converted to BF16) matrices, through a 32 x 33 shared tile.
-template <typename T>
-__global__ void transpose_kernel(int rows, int cols, const T* __restrict__ in, int ld_in, bf16* out, int ld_out) {
-  __shared__ float t[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+template <int BN, int EPI>
+__global__ void __launch_bounds__(128, 1)
+    umma_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, const UmmaArgs P) {
+  umma_tile<BN, EPI>(tA, tB, P, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// Several split products of one reduction length in one launch: blockIdx.x runs over the tiles of all
+// of them, blockIdx.z over the slices.
+constexpr int kGroupBN = 64;
+struct UmmaGroup {
+  CUtensorMap a[kUmmaGroupMax], b[kUmmaGroupMax];
+  UmmaArgs P[kUmmaGroupMax];
+  int first[kUmmaGroupMax + 1];  // first tile of each product
+};
+__global__ void __launch_bounds__(128, 1) umma_group_kernel(const __grid_constant__ UmmaGroup G) {
+  int g = 0;
+  while ((int)blockIdx.x >= G.first[g + 1]) ++g;
+  const int t = (int)blockIdx.x - G.first[g], nt = (G.P[g].N + kGroupBN - 1) / kGroupBN;
+  umma_tile<kGroupBN, 0>(G.a[g], G.b[g], G.P[g], t % nt, t / nt, blockIdx.z);
+}
+
+// BF16 copies of several matrices (BF16 or FP32) in one launch, transposed (Out[c][r] = In[r][c],
+// through a 32 x 33 shared tile) or not.
+struct CopyGroup {
+  CopyTask t[kCopyGroupMax];
+  int first[kCopyGroupMax + 1];  // first 32 x 32 tile of each task
+};
+__global__ void copy_group_kernel(const __grid_constant__ CopyGroup G) {
+  __shared__ float s[32][33];
+  int g = 0;
+  while ((int)blockIdx.x >= G.first[g + 1]) ++g;
+  const CopyTask& T = G.t[g];
+  const int b = (int)blockIdx.x - G.first[g], ct = (T.cols + 31) / 32;
+  const int c0 = b % ct * 32, r0 = b / ct * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const int r = r0 + i, c = c0 + threadIdx.x;
     float v = 0.f;
-    if (r < rows && c < cols) {
-      if constexpr (sizeof(T) == 4) v = (float)in[(size_t)r * ld_in + c];
-      else v = __bfloat162float(in[(size_t)r * ld_in + c]);
+    if (r < T.rows && c < T.cols) {
+      const size_t at = (size_t)r * T.ld_in + c;
+      v = T.f32 ? ((const float*)T.in)[at] : __bfloat162float(((const bf16*)T.in)[at]);
+      if (!T.transpose) ((bf16*)T.out)[(size_t)r * T.ld_out + c] = __float2bfloat16(v);
     }
-    t[i][threadIdx.x] = v;
+    s[i][threadIdx.x] = v;
   }
+  if (!T.transpose) return;
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const int c = c0 + i, r = r0 + threadIdx.x;
-    if (c < cols && r < ld_out) out[(size_t)c * ld_out + r] = __float2bfloat16(r < rows ? t[threadIdx.x][i] : 0.f);
+    if (c < T.cols && r < T.rows) ((bf16*)T.out)[(size_t)c * T.ld_out + r] = __float2bfloat16(s[threadIdx.x][i]);
   }
 }
 
@@ -374,7 +412,8 @@ bool umma_supported(int device) {
 }
 
 cudaError_t umma_gemm(cudaStream_t s, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,
-                      int ldc, int epi, const float* bias, const void* mask, int ldm, int n_split, int* err) {
+                      int ldc, int epi, const float* bias, const void* mask, int ldm, int n_split, int* err, void* CT,
+                      int ldt) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   // the operands' TMA rules: 16-byte aligned bases and row strides
   if (K <= 0 || lda % 8 || ldb % 8 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || !err) return cudaErrorInvalidValue;
@@ -392,7 +431,7 @@ cudaError_t umma_gemm(cudaStream_t s, int M, int N, int K, const void* A, int ld
   n_split = n_split < 1 ? 1 : n_split;
   int k_len = ((K + n_split - 1) / n_split + kUBK - 1) / kUBK * kUBK;
   const int nz = (K + k_len - 1) / k_len;
-  UmmaArgs P{M, N, K, C, ldc, bias, (const bf16*)mask, ldm, k_len, (size_t)M * ldc, err};
+  UmmaArgs P{M, N, K, C, ldc, bias, (const bf16*)mask, ldm, k_len, (size_t)M * ldc, err, (bf16*)CT, ldt};
   switch (epi) {
     case 0: return launch_epi<0>(s, bn, ma, mb, P, nz);
     case 1: return launch_epi<1>(s, bn, ma, mb, P, nz);
@@ -407,14 +446,37 @@ int umma_split_count(int K, int n_split) {
   return (K + k_len - 1) / k_len;
 }
 
-cudaError_t transpose_to_bf16(cudaStream_t s, int rows, int cols, const void* in, int ld_in, bool in_f32, void* out,
-                              int ld_out) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((ld_out + 31) / 32)), block(32, 8);
-  if (in_f32)
-    transpose_kernel<float><<<grid, block, 0, s>>>(rows, cols, (const float*)in, ld_in, (bf16*)out, ld_out);
-  else
-    transpose_kernel<bf16><<<grid, block, 0, s>>>(rows, cols, (const bf16*)in, ld_in, (bf16*)out, ld_out);
+cudaError_t umma_group(cudaStream_t s, int n, const UmmaProduct* p, int K, int n_split, int* err) {
+  if (n < 1 || n > kUmmaGroupMax || K <= 0 || !err) return cudaErrorInvalidValue;
+  const int k_len = ((K + n_split - 1) / n_split + kUBK - 1) / kUBK * kUBK;
+  UmmaGroup G;
+  G.first[0] = 0;
+  for (int i = 0; i < kUmmaGroupMax; ++i) {
+    const UmmaProduct& q = p[i < n ? i : 0];
+    if (q.lda % 8 || q.ldb % 8 || ((uintptr_t)q.A & 15) || ((uintptr_t)q.B & 15)) return cudaErrorInvalidValue;
+    if (!make_map(&G.a[i], q.A, q.M, K, q.lda, kUM) || !make_map(&G.b[i], q.B, q.N, K, q.ldb, kGroupBN))
+      return cudaErrorInvalidValue;
+    G.P[i] = UmmaArgs{q.M, q.N, K, q.C, q.N, nullptr, nullptr, 0, k_len, (size_t)q.M * q.N, err, nullptr, 0};
+    const int tiles = (q.M + kUM - 1) / kUM * ((q.N + kGroupBN - 1) / kGroupBN);
+    G.first[i + 1] = G.first[i] + (i < n ? tiles : 0);
+  }
+  cudaError_t e =
+      cudaFuncSetAttribute(umma_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem<kGroupBN>());
+  if (e != cudaSuccess) return e;
+  umma_group_kernel<<<dim3((unsigned)G.first[kUmmaGroupMax], 1, (unsigned)((K + k_len - 1) / k_len)), 128,
+                      umma_smem<kGroupBN>(), s>>>(G);
+  return cudaGetLastError();
+}
+
+cudaError_t copy_group(cudaStream_t s, int n, const CopyTask* t) {
+  if (n < 1 || n > kCopyGroupMax) return cudaErrorInvalidValue;
+  CopyGroup G;
+  G.first[0] = 0;
+  for (int i = 0; i < kCopyGroupMax; ++i) {
+    G.t[i] = t[i < n ? i : 0];
+    G.first[i + 1] = G.first[i] + (i < n ? (G.t[i].rows + 31) / 32 * ((G.t[i].cols + 31) / 32) : 0);
+  }
+  copy_group_kernel<<<(unsigned)G.first[kCopyGroupMax], dim3(32, 8), 0, s>>>(G);
   return cudaGetLastError();
 }
 
