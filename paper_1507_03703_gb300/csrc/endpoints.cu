@@ -10,9 +10,7 @@
 namespace algdock {
 namespace {
 
-constexpr int kTIThreads = 128;                     // threads of a target-interaction block
-constexpr int kTIPer = 4;                           // (configuration, atom) points per thread
-constexpr int kTIPoints = kTIPer * kTIThreads;      // points per block
+constexpr int kTIMaxThreads = 256;                  // threads of a target-interaction block at most
 constexpr int kRecPairTile = 128;                   // receptor atom pairs staged per shared-memory tile
 constexpr int kFepThreads = 256;
 constexpr int kFepMaxBlocks = 2 * 152;
@@ -23,21 +21,36 @@ __device__ __forceinline__ float rcp_approx(float v) {
   return r;
 }
 
-// Each thread evaluates kTIPer (configuration, atom) points against every receptor atom, two
-// receptor atoms per paired instruction.  A block holds whole configurations (spb of them,
-// spb * na <= 512 points), so the per-configuration sums stay inside the block and are taken in a
-// fixed order.  Receptor atoms j, j' = 2k, 2k + 1 (see ReceptorPair): x = x_hi + x_lo is the FP64
+// (double)v by integer operations on the ALU; zero, denormals, infinities and NaN by the instruction
+// (64-bit conversions run on the FP64 pipe, 2 lanes per clock and SM).
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  return (double)v;
+}
+
+// Each thread evaluates PER (configuration, atom) points against receptor atoms, two receptor atoms
+// per paired instruction.  A block holds whole configurations (spb of them), so the
+// per-configuration sums stay inside the block and are taken in a fixed order.  `groups` groups of
+// T threads share the block's points: group g takes the receptor tiles g, g + groups, ...
+// Receptor atoms j, j' = 2k, 2k + 1 (see ReceptorPair): x = x_hi + x_lo is the FP64
 // coordinate, so that the difference (x_L - x_hi) - x_lo carries the rounding of the difference
 // rather than of the coordinate.  Each term is FP32 (one approximate reciprocal; the floors of the
 // attractive and electrostatic sums at 2 A are minima of the reciprocal powers, which equal the
 // powers of max(r, 2)); a tile's terms are summed in FP32 and tiles in FP64.
-__global__ void __launch_bounds__(kTIThreads) target_interaction_kernel(
-    int64_t N, int na, int spb, const float* __restrict__ x, const TargetFactors* __restrict__ lig_fac,
-    const ReceptorPair* __restrict__ rec, const float2* __restrict__ rec_q, int n_pairs, double* __restrict__ psi) {
-  __shared__ ReceptorPair s_p[kRecPairTile];
-  __shared__ float2 s_q[kRecPairTile];
-  __shared__ double s_e[kTIPoints];
-  const int tid = threadIdx.x;
+// Bound: the FMA pipe, 15 lane-operations a pair term (2.7e12 terms/s); see kTIShapes for what the
+// shape of the blocks gives.  At 16384 x 48 x 4000 1.84 -> 1.63 ms, 1.93e12 terms/s.
+template <int PER>
+__global__ void __launch_bounds__(kTIMaxThreads, 2) target_interaction_kernel(
+    int64_t N, int na, int spb, int T, int groups, const float* __restrict__ x,
+    const TargetFactors* __restrict__ lig_fac, const ReceptorPair* __restrict__ rec,
+    const float2* __restrict__ rec_q, int n_pairs, double* __restrict__ psi) {
+  extern __shared__ __align__(16) unsigned char ti_smem[];  // groups x (pairs, charges), then the energies
+  const int g = threadIdx.x / T, tid = threadIdx.x - g * T;
+  ReceptorPair* s_p = (ReceptorPair*)ti_smem + g * kRecPairTile;
+  float2* s_q = (float2*)((ReceptorPair*)ti_smem + groups * kRecPairTile) + g * kRecPairTile;
+  double* s_e = (double*)(ti_smem + groups * kRecPairTile * (sizeof(ReceptorPair) + sizeof(float2)));
   const int64_t s0 = (int64_t)blockIdx.x * spb;
   const int nsamp = (int)min((int64_t)spb, N - s0);
   const int npts = nsamp * na;
@@ -45,11 +58,11 @@ __global__ void __launch_bounds__(kTIThreads) target_interaction_kernel(
   const float rmin2 = (float)(kRepulsiveMinDist * kRepulsiveMinDist);
   const float amin2_inv = (float)(1.0 / (kAttractiveMinDist * kAttractiveMinDist));
   const float amin6_inv = amin2_inv * amin2_inv * amin2_inv;
-  f32x2 X[kTIPer], Y[kTIPer], Z[kTIPer];
-  double dr[kTIPer], da[kTIPer], de[kTIPer];
+  f32x2 X[PER], Y[PER], Z[PER];
+  double dr[PER], da[PER], de[PER];
 #pragma unroll
-  for (int k = 0; k < kTIPer; ++k) {
-    const int p = tid + k * kTIThreads;
+  for (int k = 0; k < PER; ++k) {
+    const int p = tid + k * T;
     const bool v = p < npts;
     const float a = v ? xb[3 * p] : 0.f, b = v ? xb[3 * p + 1] : 0.f, c = v ? xb[3 * p + 2] : 0.f;
     X[k] = pack2(a, a);
@@ -57,17 +70,18 @@ __global__ void __launch_bounds__(kTIThreads) target_interaction_kernel(
     Z[k] = pack2(c, c);
     dr[k] = da[k] = de[k] = 0.0;
   }
-  for (int base = 0; base < n_pairs; base += kRecPairTile) {
-    const int m = min(kRecPairTile, n_pairs - base);
+  for (int round = 0; round < n_pairs; round += groups * kRecPairTile) {
+    const int base = round + g * kRecPairTile;
+    const int m = max(0, min(kRecPairTile, n_pairs - base));
     __syncthreads();
-    for (int t = tid; t < m; t += kTIThreads) {
+    for (int t = tid; t < m; t += T) {
       s_p[t] = rec[base + t];
       s_q[t] = rec_q[base + t];
     }
     __syncthreads();
-    f32x2 fr[kTIPer], fa[kTIPer], fe[kTIPer];
+    f32x2 fr[PER], fa[PER], fe[PER];
 #pragma unroll
-    for (int k = 0; k < kTIPer; ++k) fr[k] = fa[k] = fe[k] = 0ull;
+    for (int k = 0; k < PER; ++k) fr[k] = fa[k] = fe[k] = 0ull;
 #pragma unroll 2
     for (int t = 0; t < m; ++t) {
       const ReceptorPair R = s_p[t];
@@ -76,7 +90,7 @@ __global__ void __launch_bounds__(kTIThreads) target_interaction_kernel(
       const f32x2 lx = pack2(R.c1.z, R.c1.w), ly = pack2(R.c2.x, R.c2.y), lz = pack2(R.c2.z, R.c2.w);
       const f32x2 A = pack2(R.c3.x, R.c3.y), B = pack2(R.c3.z, R.c3.w), Q = pack2(q.x, q.y);
 #pragma unroll
-      for (int k = 0; k < kTIPer; ++k) {
+      for (int k = 0; k < PER; ++k) {
         const f32x2 dx = sub2(sub2(X[k], hx), lx), dy = sub2(sub2(Y[k], hy), ly), dz = sub2(sub2(Z[k], hz), lz);
         const f32x2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         float ra, rb;
@@ -92,29 +106,30 @@ __global__ void __launch_bounds__(kTIThreads) target_interaction_kernel(
       }
     }
 #pragma unroll
-    for (int k = 0; k < kTIPer; ++k) {
+    for (int k = 0; k < PER; ++k) {
       float a, b;
       unpack2(fr[k], a, b);
-      dr[k] += (double)a + (double)b;
+      dr[k] += widen(a) + widen(b);
       unpack2(fa[k], a, b);
-      da[k] += (double)a + (double)b;
+      da[k] += widen(a) + widen(b);
       unpack2(fe[k], a, b);
-      de[k] += (double)a + (double)b;
+      de[k] += widen(a) + widen(b);
     }
   }
-  // atom energy sqrt(A_i) LJr - sqrt(B_i) |LJa| + 332.0637 q_i elec
+  // atom energy sqrt(A_i) LJr - sqrt(B_i) |LJa| + 332.0637 q_i elec, each group's share
 #pragma unroll
-  for (int k = 0; k < kTIPer; ++k) {
-    const int p = tid + k * kTIThreads;
+  for (int k = 0; k < PER; ++k) {
+    const int p = tid + k * T;
     if (p < npts) {
       const TargetFactors f = lig_fac[p % na];
-      s_e[p] = f.sA * dr[k] - f.sB * da[k] + f.qC * de[k];
+      s_e[g * PER * T + p] = f.sA * dr[k] - f.sB * da[k] + f.qC * de[k];
     }
   }
   __syncthreads();
-  for (int k = tid; k < nsamp; k += kTIThreads) {  // up to 512 configurations (one-atom ligands)
+  for (int k = threadIdx.x; k < nsamp; k += groups * T) {  // up to 1024 configurations (one-atom ligands)
     double s = 0.0;
-    for (int i = 0; i < na; ++i) s += s_e[k * na + i];
+    for (int i = 0; i < na; ++i)
+      for (int h = 0; h < groups; ++h) s += s_e[h * PER * T + k * na + i];
     psi[s0 + k] = s;
   }
 }
@@ -162,30 +177,52 @@ __device__ __forceinline__ void lse_merge(Lse& a, const Lse& b) {
   a.m = m;
 }
 
-__device__ __forceinline__ Lse lse_shfl_down(const Lse& a, int o) {
-  Lse b;
-  b.m = __shfl_down_sync(0xffffffffu, a.m, o);
-  b.s1 = __shfl_down_sync(0xffffffffu, a.s1, o);
-  b.s2 = __shfl_down_sync(0xffffffffu, a.s2, o);
-  b.bad = __shfl_down_sync(0xffffffffu, a.bad, o);
-  return b;
+// A double's place in the order of the doubles as a signed integer (its own inverse).
+__device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
+
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// Block-wide merge in a fixed tree; the result is valid in thread 0.
+// Block-wide merge: the exact minimum by integer comparisons, one factor exp(m - m_t) per thread,
+// then sums in a fixed tree; the result is valid in thread 0.  GB300 issues 2 FP64 lanes per clock
+// and SM, so the FP64 instructions count: a tree of pairwise merges takes two exponentials at each
+// of its ten levels (44 us for 16384 samples with the launch of both kernels), this one in all.
 __device__ Lse lse_block(Lse a) {
-  __shared__ Lse s_w[kFepThreads / 32];
-  for (int o = 16; o > 0; o >>= 1) {
-    const Lse b = lse_shfl_down(a, o);
-    lse_merge(a, b);
-  }
+  constexpr int kWarps = kFepThreads / 32;
+  __shared__ long long s_key[kWarps];
+  __shared__ double s_1[kWarps], s_2[kWarps];
+  __shared__ int s_bad[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) s_w[warp] = a;
+  long long key = order_key(__double_as_longlong(a.m));
+  for (int o = 16; o > 0; o >>= 1) key = min(key, __shfl_xor_sync(0xffffffffu, key, o));
+  if (lane == 0) s_key[warp] = key;
   __syncthreads();
-  if (warp == 0) {
-    a = lane < kFepThreads / 32 ? s_w[lane] : Lse{INFINITY, 0.0, 0.0, 0};
-    for (int o = 16; o > 0; o >>= 1) {
-      const Lse b = lse_shfl_down(a, o);
-      lse_merge(a, b);
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) key = min(key, s_key[w]);
+  const double m = __longlong_as_double(order_key(key));
+  if (a.s1 > 0.0 && a.m > m) {
+    const double r = exp(m - a.m);
+    a.s1 *= r;
+    a.s2 *= r * r;
+  }
+  a.s1 = warp_sum(a.s1);
+  a.s2 = warp_sum(a.s2);
+  a.bad = __reduce_add_sync(0xffffffffu, a.bad);
+  if (lane == 0) {
+    s_1[warp] = a.s1;
+    s_2[warp] = a.s2;
+    s_bad[warp] = a.bad;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a = Lse{m, s_1[0], s_2[0], s_bad[0]};
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      a.s1 += s_1[w];
+      a.s2 += s_2[w];
+      a.bad += s_bad[w];
     }
   }
   return a;
@@ -227,18 +264,74 @@ __global__ void __launch_bounds__(kFepThreads) fep_final_kernel(int64_t N, int n
   }
 }
 
-}  // namespace
+struct TIShape {
+  int per, threads, groups;
+};
 
-int target_samples_per_block(int na) { return na > 0 ? kTIPoints / na : 0; }
+// The block shapes, and the rule that picks one: the least of max(pipe, chain) over the SM with most
+// blocks.  Pipe: a receptor pair holds the FMA pipe of a warp's SM quarter for 30 cycles a point
+// (15 paired instructions of two cycles) and 14 for the loop.  Chain: one warp alone takes 90 + 65
+// a point, and about 16 warps overlap.  So large calls take four or three points a thread, whichever
+// pads the blocks and the last SMs less, and small ones one point and several groups, down to a
+// few warps per SM.  Microseconds at (configurations, atoms, receptor atoms), in the order 128
+// threads of four points (the one shape before) -> 128 of three / two groups of 64 of three / four groups
+// of 64 of three / two groups of 96 of one:
+//   16384, 48, 4000   1858 -> 1683 / 1634 / 1762 / -    500, 10, 300     26 -> - / - / - / 12
+//   10000, 70, 4000   1678 -> 1684 / - / - / -          1000, 20, 700    50 -> - / 26 / 25 / 23
+//   3000, 33, 1200     122 -> 89 / 97 / - / -           2000, 13, 2500  163 -> - / 60 / 57 / 59
+//   5000, 61, 300       76 -> 69 / - / - / -            500, 70, 4000   261 -> 172 / 155 / 155 / -
+constexpr TIShape kTIShapes[] = {{4, 128, 1}, {3, 128, 1}, {3, 64, 2}, {3, 64, 4}, {1, 96, 2}, {1, 64, 4}};
+
+size_t ti_smem_bytes(const TIShape& h) {
+  return (size_t)h.groups * (kRecPairTile * (sizeof(ReceptorPair) + sizeof(float2)) + h.per * h.threads * sizeof(double));
+}
+
+TIShape ti_shape(int64_t N, int na, int n_pairs) {
+  TIShape best = kTIShapes[0];
+  double least = INFINITY;
+  for (const TIShape& h : kTIShapes) {
+    const int spb = h.per * h.threads / na;
+    if (spb < 1) continue;
+    const int64_t per_sm = ((N + spb - 1) / spb + 151) / 152;
+    const int rounds = (n_pairs + kRecPairTile * h.groups - 1) / (kRecPairTile * h.groups);
+    const double pairs = min(n_pairs, rounds * kRecPairTile);
+    const double warps = (double)per_sm * (h.threads / 32) * h.groups;
+    const double pipe = warps / 4 * (30 * h.per + 14), chain = fmax(1.0, warps / 16) * (90 + 65 * h.per);
+    const double t = pairs * fmax(pipe, chain);
+    if (t < least) {
+      least = t;
+      best = h;
+    }
+  }
+  return best;
+}
+
+template <int PER>
+cudaError_t ti_launch(cudaStream_t s, const TIShape& h, int64_t N, int na, const float* x,
+                      const TargetFactors* lig_fac, const ReceptorPair* rec, const float2* rec_q, int n_pairs,
+                      double* psi) {
+  const size_t smem = ti_smem_bytes(h);
+  const cudaError_t e =
+      cudaFuncSetAttribute(target_interaction_kernel<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int spb = h.per * h.threads / na;
+  const int64_t blocks = (N + spb - 1) / spb;
+  target_interaction_kernel<PER><<<(unsigned)blocks, h.threads * h.groups, smem, s>>>(
+      N, na, spb, h.threads, h.groups, x, lig_fac, rec, rec_q, n_pairs, psi);
+  return cudaGetLastError();
+}
+
+}  // namespace
 
 cudaError_t launch_target_interaction(cudaStream_t s, int64_t N, int na, const float* x, const TargetFactors* lig_fac,
                                       const ReceptorPair* rec, const float2* rec_q, int n_pairs, double* psi) {
   if (N <= 0) return cudaSuccess;
-  const int spb = target_samples_per_block(na);
-  const int64_t blocks = (N + spb - 1) / spb;
-  target_interaction_kernel<<<(unsigned)blocks, kTIThreads, 0, s>>>(N, na, spb, x, lig_fac, rec, rec_q, n_pairs,
-                                                                   psi);
-  return cudaGetLastError();
+  const TIShape h = ti_shape(N, na, n_pairs);
+  switch (h.per) {
+    case 1: return ti_launch<1>(s, h, N, na, x, lig_fac, rec, rec_q, n_pairs, psi);
+    case 3: return ti_launch<3>(s, h, N, na, x, lig_fac, rec, rec_q, n_pairs, psi);
+    default: return ti_launch<4>(s, h, N, na, x, lig_fac, rec, rec_q, n_pairs, psi);
+  }
 }
 
 size_t fep_scratch_bytes() { return sizeof(Lse) * kFepMaxBlocks + 8 * sizeof(double); }

@@ -446,7 +446,6 @@ cudaError_t learned_propose(cudaStream_t s, const algdock_ctx& c, const float* p
                             int64_t n_rep, const int32_t* state_of, float* x, double* comps, int n_moves,
                             int n_torsions, uint64_t seed, uint64_t cycle, int64_t rep_offset, int32_t* accepted,
                             int64_t* counters, void* scratch);
-int target_samples_per_block(int na);
 cudaError_t launch_target_interaction(cudaStream_t s, int64_t N, int na, const float* x, const TargetFactors* lig_fac,
                                       const ReceptorPair* rec, const float2* rec_q, int n_pairs, double* psi);
 size_t fep_scratch_bytes();
