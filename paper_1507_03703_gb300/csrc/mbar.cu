@@ -44,14 +44,58 @@ struct MbarState {
 struct Lse {
   double m, s;
 };
-__device__ inline void lse_add(Lse& a, double x, int mode) {
+__device__ inline void lse_add(Lse& a, double x) {
   if (x == -INFINITY) return;
   if (x <= a.m) {
-    a.s += mode ? (double)__expf((float)(x - a.m)) : exp(x - a.m);
+    a.s += exp(x - a.m);
   } else {
-    a.s = a.s * (mode ? (double)__expf((float)(a.m - x)) : exp(a.m - x)) + 1.0;
+    a.s = a.s * exp(a.m - x) + 1.0;
     a.m = x;
   }
+}
+
+// (float)v and (double)v with the instructions' results, by integer operations where value and result
+// are normal numbers (or, widening, zero): conversions between 32 and 64 bits run on the FP64 pipe,
+// 2 lanes per clock and SM.
+__device__ __forceinline__ float narrow(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t t = (hi & 0x7fffffffu) - 0x38000000u;
+  if (t - 0x00100000u >= 0x0fd00000u) return (float)v;
+  uint32_t b = __funnelshift_l(lo, t, 3);
+  b += (lo << 3) > 0x80000000u - (b & 1u);  // to nearest, ties to even
+  return __uint_as_float(b | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (b != 0 && m - 0x00800000u >= 0x7f000000u) return (double)v;
+  return __hiloint2double(b ? (int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)) : 0, (int)(b << 29));
+}
+
+// Precision mode 1, FP32 exponentials of FP64 arguments.  The FP64 pipe bounds it, so an element takes
+// three operations there: x itself, its distance from the maximum (whose sign decides, as it is exact)
+// and one multiply-add, s + e below the maximum and s e + 1 above it.  No branch: along a ladder the
+// maximum rises at half of the states.  m starts at kLowest in place of -inf (an argument of -inf
+// then adds nothing).
+// K = 256, N = 1.0e6: 8.8 -> 4.3 ms an iteration, the same bits.
+constexpr double kLowest = -1.7976931348623157e308;
+__device__ __forceinline__ void lse_add_f32exp(Lse& a, double x) {
+  const double d = x - a.m;
+  const int hi = __double2hiint(d);
+  const bool above = hi >= 0 && (hi | __double2loint(d)) != 0;
+  const double e = widen(__expf(-fabsf(narrow(d))));
+  a.s = fma(a.s, above ? e : 1.0, above ? 1.0 : e);
+  a.m = above ? x : a.m;
+}
+template <int MODE>
+__device__ __forceinline__ void lse_add_mode(Lse& a, double x) {
+  if (MODE) lse_add_f32exp(a, x);
+  else lse_add(a, x);
+}
+template <int MODE>
+__device__ __forceinline__ Lse lse_none() { return Lse{MODE ? kLowest : -INFINITY, 0.0}; }
+template <int MODE>
+__device__ __forceinline__ void lse_end(Lse& a) {
+  if (MODE && a.m == kLowest && a.s == 0.0) a.m = -INFINITY;
 }
 __device__ inline Lse lse_merge(Lse a, Lse b) {
   if (b.m == -INFINITY) return a;
@@ -60,36 +104,46 @@ __device__ inline Lse lse_merge(Lse a, Lse b) {
   return Lse{b.m, b.s + a.s * exp(a.m - b.m)};
 }
 
+constexpr int kDenTile = 256;  // states whose ln N_k + f_k a block holds at a time
+template <int MODE>
 __global__ void log_denominators(int K, int64_t N, const double* __restrict__ u, const double* __restrict__ logNk,
-                                 const double* __restrict__ f, double* logD, const MbarState* st, int mode) {
+                                 const double* __restrict__ f, double* logD, const MbarState* st) {
   if (st->converged) return;
+  __shared__ double s_g[kDenTile];
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  Lse a{-INFINITY, 0.0};
+  const double* col = u + min(n, N - 1);
+  Lse a = lse_none<MODE>();
   // eight independent loads in flight, then the updates in the same order as one at a time
   constexpr int kAhead = 8;
-  const double* col = u + n;
-  int k = 0;
-  for (; k + kAhead <= K; k += kAhead) {
-    double v[kAhead];
+  for (int k0 = 0; k0 < K; k0 += kDenTile) {
+    const int kn = min(kDenTile, K - k0);
+    __syncthreads();
+    for (int k = threadIdx.x; k < kn; k += blockDim.x) s_g[k] = logNk[k0 + k] + f[k0 + k];
+    __syncthreads();
+    int k = 0;
+    for (; k + kAhead <= kn; k += kAhead) {
+      double v[kAhead];
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) v[j] = __ldg(col + (int64_t)(k + j) * N);
+      for (int j = 0; j < kAhead; ++j) v[j] = __ldg(col + (int64_t)(k0 + k + j) * N);
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) lse_add(a, logNk[k + j] + f[k + j] - v[j], mode);
+      for (int j = 0; j < kAhead; ++j) lse_add_mode<MODE>(a, s_g[k + j] - v[j]);
+    }
+    for (; k < kn; ++k) lse_add_mode<MODE>(a, s_g[k] - __ldg(col + (int64_t)(k0 + k) * N));
   }
-  for (; k < K; ++k) lse_add(a, logNk[k] + f[k] - __ldg(col + (int64_t)k * N), mode);
-  logD[n] = a.m + log(a.s);
+  lse_end<MODE>(a);
+  if (n < N) logD[n] = a.m + log(a.s);
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(kPartialThreads) state_partials(int64_t N, int64_t chunk_len,
                                                                   const double* __restrict__ u,
                                                                   const double* __restrict__ logD, double2* part,
-                                                                  int n_chunks, const MbarState* st, int mode) {
+                                                                  int n_chunks, const MbarState* st) {
   if (st->converged) return;
   const int i = blockIdx.y, chunk = blockIdx.x;
   const int64_t begin = (int64_t)chunk * chunk_len;
   const int64_t end = min(N, begin + chunk_len);
-  Lse a{-INFINITY, 0.0};
+  Lse a = lse_none<MODE>();
   const double* ui = u + (int64_t)i * N;
   constexpr int kAhead = 8;
   const int64_t stride = blockDim.x;
@@ -102,9 +156,10 @@ __global__ void __launch_bounds__(kPartialThreads) state_partials(int64_t N, int
       d[j] = __ldg(logD + n + j * stride);
     }
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) lse_add(a, -v[j] - d[j], mode);
+    for (int j = 0; j < kAhead; ++j) lse_add_mode<MODE>(a, -v[j] - d[j]);
   }
-  for (; n < end; n += stride) lse_add(a, -ui[n] - logD[n], mode);
+  for (; n < end; n += stride) lse_add_mode<MODE>(a, -ui[n] - logD[n]);
+  lse_end<MODE>(a);
   __shared__ double sm[kPartialThreads], ss[kPartialThreads];
   sm[threadIdx.x] = a.m;
   ss[threadIdx.x] = a.s;
@@ -545,6 +600,20 @@ int weight_blocks(int K, int64_t N) {
   return (int)std::min<int64_t>(tiles, 152 * (K <= 128 ? 3 : 2));
 }
 
+// The two passes of a log-sum-exp iteration in FP64 or (mode 1) with FP32 exponentials.
+void launch_passes(cudaStream_t s, int K, int64_t N, int64_t chunk_len, int n_chunks, const double* u,
+                   const double* logNk, const double* f, double* logD, double2* part, const MbarState* st, int mode) {
+  const unsigned blocks = (unsigned)((N + 255) / 256);
+  const dim3 grid((unsigned)n_chunks, (unsigned)K);
+  if (mode) {
+    log_denominators<1><<<blocks, 256, 0, s>>>(K, N, u, logNk, f, logD, st);
+    state_partials<1><<<grid, kPartialThreads, 0, s>>>(N, chunk_len, u, logD, part, n_chunks, st);
+  } else {
+    log_denominators<0><<<blocks, 256, 0, s>>>(K, N, u, logNk, f, logD, st);
+    state_partials<0><<<grid, kPartialThreads, 0, s>>>(N, chunk_len, u, logD, part, n_chunks, st);
+  }
+}
+
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -602,10 +671,7 @@ cudaError_t mbar_local_pairs(cudaStream_t s, void* scratch, int K, int64_t N, co
   init_state<<<1, 256, 0, s>>>(K, Nk, logNk, f, st);
   e = cudaMemcpyAsync(f, f_host, sizeof(double) * K, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  const int threads = 256;
-  log_denominators<<<(unsigned)((N + threads - 1) / threads), threads, 0, s>>>(K, N, u_kn, logNk, f, logD, st, mode);
-  state_partials<<<dim3((unsigned)n_chunks, (unsigned)K), kPartialThreads, 0, s>>>(N, chunk_len, u_kn, logD, part,
-                                                                                    (int)n_chunks, st, mode);
+  launch_passes(s, K, N, chunk_len, (int)n_chunks, u_kn, logNk, f, logD, part, st, mode);
   merge_chunk_pairs<<<(unsigned)((K * 32 + 255) / 256), 256, 0, s>>>(K, (int)n_chunks, part, pairs);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(pairs_host, pairs, sizeof(double2) * K, cudaMemcpyDeviceToHost, s);
@@ -653,8 +719,7 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
       state_partials_f32<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, w32, (const float*)logD, part, (int)n_chunks,
                                                             st);
     } else {
-      log_denominators<<<blocks_n, threads, 0, s>>>(K, N, u_kn, logNk, f, logD, st, mode);
-      state_partials<<<grid_p, kPartialThreads, 0, s>>>(N, chunk_len, u_kn, logD, part, (int)n_chunks, st, mode);
+      launch_passes(s, K, N, chunk_len, (int)n_chunks, u_kn, logNk, f, logD, part, st, mode);
     }
     const unsigned merge_blocks = (unsigned)((K * 32 + 255) / 256);
     if (mode == 2)
