@@ -398,7 +398,7 @@ __global__ void init_state(int K, const int64_t* Nk, double* logNk, double* f, M
 // (the shifts c_n cancel, and so does a factor common to all a_k).  Two FP64 multiply-adds per
 // element and iteration remain, which is what bounds it: GB300 issues 2 FP64 lanes per clock and
 // SM, so K = 128, N = 102400 cannot take less than 42 us an iteration (its 105 MB of weights take
-// 15 us from HBM).  Measured: a solve of 43 iterations at that size 88.5 -> 3.94 ms (two log-sum-exp
+// 15 us from HBM).  Measured: a solve of 43 iterations at that size 88.5 -> 3.85 ms (4.00 with one tile a block; two log-sum-exp
 // passes with an FP64 exponential per element take 1455 us an iteration), and 25.9 -> 1.58 ms an
 // iteration, the forming of the weights included, at K = 256, N = 1e6.
 //
@@ -442,18 +442,19 @@ __global__ void __launch_bounds__(256) build_weights(int K, int64_t N, const dou
 // The sums of one iteration.  A block takes tiles blockIdx.x, + gridDim.x, ...: the tile goes to
 // shared memory once and serves both passes, D'_n (each warp its states, then one warp adds the
 // warps' parts) and the state sums, which stay in registers (lane = sample) over all the block's
-// tiles.  Several blocks per SM, so that one loads while another computes.  The reduction of the 32
+// tiles.  Several blocks per SM, so that one loads while another computes; with STAGES = 2 (where two
+// tiles a block leave room for three blocks) the next tile also loads during this one's passes.  The reduction of the 32
 // accumulators over the lanes halves their number at each step (31 FP64 additions instead of 160:
 // at 2 lanes per clock these count).  part[k][block].
-template <int NW>
+template <int NW, int STAGES>
 __global__ void __launch_bounds__(32 * NW) weight_pass(int K, int64_t N, const double* __restrict__ W,
                                                        const double* __restrict__ a, double* __restrict__ part,
                                                        const MbarState* st) {
   if (st->converged || st->trip) return;
-  extern __shared__ __align__(16) double s_w[];  // [K][32], then a [K]
+  extern __shared__ __align__(16) double s_w[];  // STAGES tiles [K][32], then a [K]
   __shared__ double s_part[NW][kWTile];
   __shared__ double s_r[kWTile];
-  double* s_a = s_w + K * kWTile;
+  double* s_a = s_w + STAGES * K * kWTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = (K + NW - 1) / NW;  // <= kWStates
   const int k0 = warp * per, kn = max(0, min(per, K - k0));
@@ -462,14 +463,22 @@ __global__ void __launch_bounds__(32 * NW) weight_pass(int K, int64_t N, const d
 #pragma unroll
   for (int j = 0; j < kWStates; ++j) acc[j] = 0.0;
   const int64_t tiles = (N + kWTile - 1) / kWTile;
-  const double* mine = s_w + k0 * kWTile + lane;
   const double* my_a = s_a + k0;
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const char* src = (const char*)(W + t * K * kWTile);
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_w);
-    for (int i = threadIdx.x; i < K * kWTile / 2; i += 32 * NW)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 16 * i) : "memory");
-    asm volatile("cp.async.wait_all;" ::: "memory");
+  auto load = [&](int64_t t, int stage) {
+    if (t < tiles) {
+      const char* src = (const char*)(W + t * K * kWTile);
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_w + stage * K * kWTile);
+      for (int i = threadIdx.x; i < K * kWTile / 2; i += 32 * NW)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 16 * i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (STAGES == 2) load(blockIdx.x, 0);
+  int stage = 0;
+  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, stage ^= STAGES - 1) {
+    const double* mine = s_w + (stage * K + k0) * kWTile + lane;
+    load(STAGES == 2 ? t + gridDim.x : t, stage ^ (STAGES - 1));
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
     __syncthreads();
     double d0 = 0.0, d1 = 0.0;
 #pragma unroll
@@ -492,6 +501,7 @@ __global__ void __launch_bounds__(32 * NW) weight_pass(int K, int64_t N, const d
       if (j < kn) acc[j] = fma(mine[j * kWTile], r, acc[j]);
     __syncthreads();  // the tile and s_r are free again
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   // lane l ends with the sum of accumulator l over all lanes
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -744,9 +754,9 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
     double* wpart = (double*)(q + align256(16 * (size_t)K));
     const int blocks = weight_blocks(K, N);
     double* W = (double*)((char*)wpart + align256((size_t)K * blocks * sizeof(double)));
-    const size_t smem = (size_t)K * (kWTile + 1) * sizeof(double);
     const bool wide = K > 128;
-    e = cudaFuncSetAttribute(wide ? weight_pass<8> : weight_pass<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = (size_t)K * ((wide ? 1 : 2) * kWTile + 1) * sizeof(double);
+    e = cudaFuncSetAttribute(wide ? weight_pass<8, 1> : weight_pass<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     if (e != cudaSuccess) { *err = e; return -1; }
     while (!done) {
@@ -755,8 +765,8 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
       build_weights<<<(unsigned)((N + kWTile - 1) / kWTile), 256, 0, s>>>(K, N, u_kn, g, W);
       for (bool trip = false; !done && !trip;) {
         for (int b = 0; b < batch && issued < max_iter; ++b, ++issued) {
-          if (wide) weight_pass<8><<<blocks, 256, smem, s>>>(K, N, W, a, wpart, st);
-          else weight_pass<4><<<blocks, 128, smem, s>>>(K, N, W, a, wpart, st);
+          if (wide) weight_pass<8, 1><<<blocks, 256, smem, s>>>(K, N, W, a, wpart, st);
+          else weight_pass<4, 2><<<blocks, 128, smem, s>>>(K, N, W, a, wpart, st);
           weight_update<<<(unsigned)((K + 3) / 4), 128, 0, s>>>(K, blocks, wpart, Nk, g, f, fnew, a, st, tol, max_iter);
         }
         e = poll();
