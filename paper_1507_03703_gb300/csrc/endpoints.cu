@@ -310,10 +310,7 @@ template <int PER>
 cudaError_t ti_launch(cudaStream_t s, const TIShape& h, int64_t N, int na, const float* x,
                       const TargetFactors* lig_fac, const ReceptorPair* rec, const float2* rec_q, int n_pairs,
                       double* psi) {
-  const size_t smem = ti_smem_bytes(h);
-  const cudaError_t e =
-      cudaFuncSetAttribute(target_interaction_kernel<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = ti_smem_bytes(h);  // 43,008 bytes at most: no opt-in
   const int spb = h.per * h.threads / na;
   const int64_t blocks = (N + spb - 1) / spb;
   target_interaction_kernel<PER><<<(unsigned)blocks, h.threads * h.groups, smem, s>>>(

@@ -764,8 +764,9 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
     double* W = (double*)((char*)wpart + align256((size_t)K * blocks * sizeof(double)));
     const bool wide = K > 128;
     const size_t smem = (size_t)K * ((wide ? 1 : 2) * kWTile + 1) * sizeof(double);
+    // the limit for the most states, whatever K: another thread's solve may set it between this and a launch
     e = cudaFuncSetAttribute(wide ? weight_pass<8, 1> : weight_pass<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+                             (int)((wide ? kWMaxStates * (kWTile + 1) : 128 * (2 * kWTile + 1)) * sizeof(double)));
     if (e != cudaSuccess) { *err = e; return -1; }
     while (!done) {
       const int applied = issued;  // iterations applied when the weights were last formed

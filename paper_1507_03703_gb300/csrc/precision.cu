@@ -415,7 +415,8 @@ cudaError_t launch_eval64(cudaStream_t s, const algdock_ctx& c, int64_t N, const
   const Eval64Args A{N, c.lig64, c.d_lig64, c.lig, c.d_blob, c.grid64, c.d_states, c.K, state_of, x, force, comps,
                      slots};
   auto k = force ? eval64_kernel<true> : eval64_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit itself, whatever the ligand: another thread's call may set it between this and the launch
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem64);
   if (e != cudaSuccess) return e;
   k<<<(unsigned)((N + warps - 1) / warps), warps * 32, smem, s>>>(A);
   return cudaGetLastError();
