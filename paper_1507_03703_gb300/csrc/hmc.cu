@@ -1636,6 +1636,10 @@ constexpr int kTableWarps = 16;  // replicas per block of the pair-table HMC ker
 // per team).  Up to 4 replicas per SM of 33-64 atoms take the kernel with 126 registers instead of 80
 // (32 replicas of 48 atoms: 166 us against 193); from there on the one with 24 warps per SM.
 constexpr int kTable1 = 5, kTable2 = 6, kTable2Few = 4, kType1 = 16, kType2 = 4, kType3 = 8;
+// Two warps a replica, with more replicas than two blocks of kTable2 hold per SM but no more than one of 16
+// does: one block of 16 takes them at once, where the two would need a second round for a few.  45 atoms, 1900 replicas, 50 steps: 547 -> 401 us (534
+// with one warp a replica).
+constexpr int kTable2Wave = 16;
 constexpr size_t kMaxBlockSmem = 227 * 1024;
 
 // Dynamic shared memory of an HMC block of `slots` replicas, and the most of at most `slots` that a
@@ -1684,6 +1688,9 @@ cudaError_t launch_hmc(cudaStream_t s, const algdock_ctx& c, int64_t n_rep, cons
   if (table && apl == 2 && n_rep <= (int64_t)kTable2Few * sms) {
     k = hmc_kernel<2, kTable2Few, true>;
     most = kTable2Few;
+  } else if (table && apl == 2 && n_rep > (int64_t)2 * kTable2 * sms && n_rep <= (int64_t)kTable2Wave * sms) {
+    k = hmc_kernel<2, kTable2Wave, true>;
+    most = kTable2Wave;
   } else if (table) {
     k = apl == 1 ? hmc_kernel<1, kTable1, true, false, 4> : hmc_kernel<2, kTable2, true, false, 2>;
     most = apl == 1 ? kTable1 : kTable2;
