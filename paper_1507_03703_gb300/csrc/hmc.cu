@@ -81,8 +81,9 @@ __device__ inline Lig bind_ligand(const uint32_t* s, const LigandLayout& L) {
 
 // The hardware's approximate reciprocal square root and quotient.  rsqrtf and __fdividef are the same
 // instructions wrapped in a scaling of denormal arguments (three more instructions each, a tenth of
-// the kernel's); the arguments here are squared distances and their products, which are zero or
-// normal, so the results are the same bits.
+// the kernel's), which these take for zero.  Their arguments are squared distances, denormal only below
+// 1.1e-19 A, and values with a floor; otherwise the results are the same bits.  Not so the product of a
+// torsion's two squared normals, each with a floor: that is 1e-40 where all four atoms lie on a line.
 __device__ __forceinline__ float rsqrt_fast(float v) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
@@ -296,7 +297,7 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
     const float inv_lb2 = rsqrt_fast(lb22);
     const float lb2 = lb22 * inv_lb2;
     const float n1s = fmaxf(dot(n1, n1), 1e-20f), n2s = fmaxf(dot(n2, n2), 1e-20f);
-    const float inv = rsqrt_fast(n1s * n2s);
+    const float inv = rsqrtf(n1s * n2s);       // finite also where both are at their floor
     const float cp = dot(n1, n2) * inv;        // cos phi
     const float sp = lb2 * dot(b1, n2) * inv;  // sin phi
     const float c2 = 2.f * cp * cp - 1.f, s2 = 2.f * sp * cp;
