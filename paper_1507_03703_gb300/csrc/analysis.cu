@@ -83,7 +83,7 @@ cudaError_t launch_equilibration(cudaStream_t st, int64_t T, int64_t S, const do
                                  double* g, int64_t* t0_best, double* neff_best) {
   const size_t smem = equilibration_smem(T);
   cudaError_t e = cudaFuncSetAttribute(tail_inefficiency_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+                                       (int)kMaxBlockSmem);
   if (e != cudaSuccess) return e;
   tail_inefficiency_kernel<<<dim3((unsigned)n_cand, (unsigned)S), 32, smem, st>>>(T, S, a, stride, n_cand, g);
   e = cudaGetLastError();

@@ -600,7 +600,7 @@ cudaError_t launch_exchange(cudaStream_t s, const algdock_ctx& c, int n_ladders,
                          : kg == 2 ? exchange_team_kernel<2>
                          : kg == 3 ? exchange_team_kernel<3>
                                    : exchange_team_kernel<4>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fast);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem);
     if (e != cudaSuccess) return e;
     fn<<<n_ladders, kFastThreads, fast, s>>>(A);
     return cudaGetLastError();
@@ -609,7 +609,7 @@ cudaError_t launch_exchange(cudaStream_t s, const algdock_ctx& c, int n_ladders,
     const size_t smem = (size_t)K * K * sizeof(double) + (size_t)K * (3 * sizeof(double) + sizeof(SlotE) + sizeof(int)) +
                         counters;
     cudaError_t e = cudaFuncSetAttribute(exchange_matrix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         (int)kMaxBlockSmem);
     if (e != cudaSuccess) return e;
     exchange_matrix_kernel<<<n_ladders, kExMaxWarps * 32, smem, s>>>(A);
     return cudaGetLastError();
@@ -623,7 +623,8 @@ cudaError_t launch_exchange(cudaStream_t s, const algdock_ctx& c, int n_ladders,
   while (warps > 1 && fixed + warps * per_warp > budget) --warps;
   if (fixed + warps * per_warp > budget) return cudaErrorInvalidValue;
   const size_t smem = fixed + warps * per_warp;
-  cudaError_t e = cudaFuncSetAttribute(exchange_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(exchange_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kMaxBlockSmem);
   if (e != cudaSuccess) return e;
   const int blocks = (n_ladders + warps - 1) / warps;
   exchange_direct_kernel<<<blocks, warps * 32, smem, s>>>(A);

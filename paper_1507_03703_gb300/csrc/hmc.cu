@@ -1641,7 +1641,6 @@ constexpr int kTable1 = 5, kTable2 = 6, kTable2Few = 4, kType1 = 16, kType2 = 4,
 // does: one block of 16 takes them at once, where the two would need a second round for a few.  45 atoms, 1900 replicas, 50 steps: 547 -> 401 us (534
 // with one warp a replica).
 constexpr int kTable2Wave = 16;
-constexpr size_t kMaxBlockSmem = 227 * 1024;
 
 // Dynamic shared memory of an HMC block of `slots` replicas, and the most of at most `slots` that a
 // limit holds (at least one).
@@ -1657,7 +1656,7 @@ template <typename Kernel, typename Args>
 cudaError_t launch_templated(Kernel k1, Kernel k2, Kernel k3, int apl, size_t smem, int64_t items, cudaStream_t s,
                              const Args& A, int wpb = kWarpsPerBlock) {
   Kernel k = apl == 1 ? k1 : (apl == 2 ? k2 : k3);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem);
   if (e != cudaSuccess) return e;
   const int64_t blocks = (items + wpb - 1) / wpb;
   k<<<(unsigned)blocks, wpb * 32, smem, s>>>(A);
@@ -1702,7 +1701,7 @@ cudaError_t launch_hmc(cudaStream_t s, const algdock_ctx& c, int64_t n_rep, cons
   }
   int slots = team_slots(c.lig, apl, most, table, kMaxBlockSmem), per_sm = 0;
   size_t smem = team_smem(c.lig, apl, slots, table);
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, slots * apl * 32, smem);
   if (e != cudaSuccess) return e;
@@ -1784,7 +1783,8 @@ cudaError_t batch_set_attributes(const algdock_ctx& c) {
     const BatchClass& B = c.batch_cls[k];
     if (B.n_items == 0) continue;
     cudaError_t e = cudaFuncSetAttribute(batch_kernel(kClassApl[k], B.wpb, B.table),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B.smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)batch_smem_limit(kClassApl[k], B.wpb, B.table));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1833,7 +1833,8 @@ cudaError_t launch_evaluate(cudaStream_t s, const algdock_ctx& c, int64_t N, con
   const int apl = atoms_per_lane(c.lig.na);
   void (*k)(const EnergyArgs) = apl == 1 ? energy_kernel<1> : (apl == 2 ? energy_kernel<2> : energy_kernel<3>);
   const size_t smem = 4 * ((size_t)staged_words(c.lig, false) + (size_t)kEnergyWarps * 8 * 32 * apl);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(kMaxBlockSmem - sizeof(double[kEnergyWarps * kEnergyPer][4])));
   int per_sm = 0, sms = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kEnergyWarps * 32, smem);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);

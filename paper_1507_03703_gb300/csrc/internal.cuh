@@ -32,6 +32,11 @@ constexpr double kRepulsiveMinDist = 0.01;         // A
 constexpr double kAttractiveMinDist = 2.0;         // A
 constexpr int kMaxAtoms = 96;                      // 3 atoms per lane of one warp
 constexpr int kMaxLadder = 1024;
+// Shared memory a block can opt in to on sm_103a (static and dynamic).  A kernel's own limit of dynamic
+// shared memory belongs to the kernel on its device, for all contexts and threads, so launches set it to
+// this (less the kernel's static shared memory) whatever the call needs: a limit that followed the call
+// could be lowered by another context between one's setting and its launch.
+constexpr size_t kMaxBlockSmem = 227 * 1024;
 constexpr size_t kMbarFlagBytes = 16;              // pinned words a context polls device flags in
 constexpr size_t kMbarKeepBytes = (size_t)4 << 30;  // MBAR scratch with stored weights kept between solves
 constexpr int kMbarMaxStates = 65535;             // MBAR's state_partials grid has one y-index per state

@@ -728,7 +728,7 @@ int mbar_run(cudaStream_t s, void* scratch, int K, int64_t N, const double* u_kn
     w32 = (float*)((char*)scratch + off);
     shift_columns<<<blocks_n, threads, 0, s>>>(K, N, u_kn, w32);
     e = cudaFuncSetAttribute(log_denominators_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(K * sizeof(float)));
+                             (int)kMaxBlockSmem);
     if (e != cudaSuccess) { *err = e; return -1; }
   }
   auto iterate = [&] {  // one log-sum-exp iteration
