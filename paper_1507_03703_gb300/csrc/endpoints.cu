@@ -177,9 +177,6 @@ __device__ __forceinline__ void lse_merge(Lse& a, const Lse& b) {
   a.m = m;
 }
 
-// A double's place in the order of the doubles as a signed integer (its own inverse).
-__device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
-
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;

@@ -73,6 +73,10 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   return r;
 }
 
+// A double's place in the order of the doubles as a signed integer (its own inverse), for minima and maxima
+// on the integer units.
+__device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
+
 enum : uint32_t { kPurposeMomentum = 1, kPurposeAccept = 2, kPurposeExchange = 3, kPurposeExternal = 5 };
 
 // ------------------------------------------------------------------ Philox4x32-10

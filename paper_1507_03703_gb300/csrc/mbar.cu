@@ -410,8 +410,8 @@ __global__ void init_state(int K, const int64_t* Nk, double* logNk, double* f, M
 // passes with an FP64 exponential per element take 1455 us an iteration), and 25.9 -> 1.58 ms an
 // iteration, the forming of the weights included, at K = 256, N = 1e6.
 //
-// Range.  c_n is the column's maximum (to 2^-20 relative), so the largest weight of a column is 1
-// and only weights below 1e-308 of it are lost.  While the spread of f - g stays within kMaxSpread,
+// Range.  c_n is the column's maximum, so the largest weight of a column is 1, D'_n is finite and only
+// weights below 1e-308 of the largest are lost.  While the spread of f - g stays within kMaxSpread,
 // D'_n >= N_k exp(-200) and the lost terms are below 1e-120 of any sum of at least kMinSum.  An
 // iteration outside these limits is not applied (trip): the host then runs one log-sum-exp
 // iteration from the same f, takes g = f and forms the weights again.  A ladder whose reduced
@@ -425,23 +425,21 @@ constexpr double kMinSum = 1e-150;     // of sum_n W_kn / D'_n
 // One block per tile: lane = sample, each warp every eighth state.
 __global__ void __launch_bounds__(256) build_weights(int K, int64_t N, const double* __restrict__ u,
                                                      const double* __restrict__ g, double* __restrict__ W) {
-  __shared__ int s_key[8][kWTile];
+  __shared__ long long s_key[8][kWTile];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t n = (int64_t)blockIdx.x * kWTile + lane;
   const bool in = n < N;
   const double* col = u + (in ? n : N - 1);
-  // the maximum from the high words alone: as signed integers, with the lower 31 bits of a
-  // negative one inverted, they order as the doubles do
-  int key = INT_MIN;
-  for (int k = warp; k < K; k += 8) {
-    const int hi = __double2hiint(g[k] - __ldg(col + (int64_t)k * N));
-    key = max(key, hi ^ ((hi >> 31) & 0x7fffffff));
-  }
+  // the exact maximum, by integer comparisons: a shift rounded to the high word would be off by up to
+  // 2^-20 of an offset common to the column, and the weights or D'_n could leave the range of a double
+  long long key = LLONG_MIN;
+  for (int k = warp; k < K; k += 8)
+    key = max(key, order_key(__double_as_longlong(g[k] - __ldg(col + (int64_t)k * N))));
   s_key[warp][lane] = key;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < 8; ++w) key = max(key, s_key[w][lane]);
-  const double c = __hiloint2double(key ^ ((key >> 31) & 0x7fffffff), 0);
+  const double c = __longlong_as_double(order_key(key));
   double* out = W + (int64_t)blockIdx.x * K * kWTile + lane;
   for (int k = warp; k < K; k += 8)
     out[(int64_t)k * kWTile] = in ? exp((g[k] - __ldg(col + (int64_t)k * N)) - c) : 0.0;
