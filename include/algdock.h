@@ -369,11 +369,11 @@ algdock_status algdock_reduced_energies(algdock_ctx* ctx, int64_t N, const float
  *   f_i <- -ln sum_n exp(-u_in) / sum_k N_k exp(f_k - u_kn)
  * until max_i |change| < tol or max_iter iterations.  u_kn [K][N] double (device), N_k [K] int64
  * (host).  precision_mode 0: FP64 throughout (with every N_k > 0 and K <= 256 the iteration runs on
- * stored weights, K*N*8 bytes of scratch where at most half of the free memory, kept with the context
- * up to 4 GiB); 1: exponentials in FP32 of FP64 arguments, sums in
- * FP64; 2: each sample's column shifted by its minimum (FP64, exact in the result) and stored as
- * FP32, then FP32 arguments, exponentials and Kahan-compensated sums, FP64 only where partial sums
- * meet (K <= 16384; extra scratch K*N*4 bytes).  K <= 65535 in every mode.  tol = 0, max_iter = 0
+ * stored weights, K*N*8 bytes of scratch where at most half of the free memory; the context keeps
+ * it up to 1 GiB and gives a larger one back before the call returns); 1: exponentials in FP32 of
+ * FP64 arguments, sums in FP64; 2: each sample's column shifted by its minimum (FP64, exact in the
+ * result) and stored as FP32, then FP32 arguments, exponentials and Kahan-compensated sums, FP64 only
+ * where partial sums meet (K <= 16384; extra scratch K*N*4 bytes).  K <= 65535 in every mode.  tol = 0, max_iter = 0
  * and precision_mode = -1 take the context's params (mbar_tol, mbar_max_iter, mbar_precision).
  * f_k [K] (host) and iters (host) receive the result.  Synchronises.  Returns
  * ALGDOCK_E_NOT_CONVERGED (with the last iterate in f_k) if max_iter is reached. */

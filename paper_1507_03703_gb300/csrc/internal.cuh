@@ -38,7 +38,10 @@ constexpr int kMaxLadder = 1024;
 // could be lowered by another context between one's setting and its launch.
 constexpr size_t kMaxBlockSmem = 227 * 1024;
 constexpr size_t kMbarFlagBytes = 16;              // pinned words a context polls device flags in
-constexpr size_t kMbarKeepBytes = (size_t)4 << 30;  // MBAR scratch with stored weights kept between solves
+// MBAR scratch with stored weights kept between solves: what mode 2 keeps at 256 states and 1e6 samples.  A
+// larger solve allocates it anew and gives it back, so that a context holds no more of the device than that
+// (1.2 GB: 1.0 ms of a solve's 30.9; 3.0 GB: 2.2 of 77.6).
+constexpr size_t kMbarKeepBytes = (size_t)1 << 30;
 constexpr int kMbarMaxStates = 65535;             // MBAR's state_partials grid has one y-index per state
 
 // Two FP32 values in one 64-bit register pair, for the paired FP32 instructions of sm_100-class
