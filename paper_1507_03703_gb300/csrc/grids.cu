@@ -15,7 +15,10 @@ namespace {
 constexpr int kBuildThreads = 128;
 constexpr int kBuildTile = 128;      // receptor atom pairs staged per shared-memory tile
 constexpr int kBuildNodes = 4;       // nodes per thread, spread along x
-constexpr float kBuildMaxR2 = 1e30f;  // keeps the reciprocal's refinement finite
+constexpr float kBuildMaxR2 = 8e37f;  // keeps the reciprocal normal and its refinement finite
+// Nodes beyond kBuildFar of the origin, whose square FP32 does not hold, and atoms beyond three times that are
+// taken to lie there: as far from all else, and hi + lo stays finite.
+constexpr double kBuildFar = 2e19;
 
 __device__ __forceinline__ float rcp_approx(float v) {
   float r;
@@ -69,7 +72,7 @@ __global__ void __launch_bounds__(kBuildThreads) grid_build_kernel(
   // thread (q, j, k) of nq x ny x nz: nodes q, q + nq, q + 2 nq, q + 3 nq of row (j, k)
   const int q = (int)(item % nq), j = (int)((item / nq) % ny), k = (int)(item / ((int64_t)nq * ny));
   auto split = [&](int i, f32x2& hi, f32x2& lo) {
-    const double p = h * i;
+    const double p = fmin(h * i, kBuildFar);
     const float ph = (float)(rint(p / quantum) * quantum);
     const float pl = (float)(p - (double)ph);
     hi = pack2(ph, ph);
@@ -242,8 +245,9 @@ cudaError_t launch_grid_build(cudaStream_t s, const algdock_grid_desc& d, int n_
   std::vector<ReceptorPair> h_rec(np, ReceptorPair{});
   std::vector<float2> h_q(np, make_float2(0.f, 0.f));
   // the quantum of the hi parts: 2^-23 of the range the lattice and 64 A around it span
-  const double range = d.spacing * std::max({d.n[0], d.n[1], d.n[2]}) + 64.0;
-  const double quantum = std::isfinite(range) ? ldexp(1.0, std::ilogb(range) + 1 - 23) : 1.0;
+  const int n_max = std::max({d.n[0], d.n[1], d.n[2]});
+  const double range = std::min(d.spacing * n_max + 64.0, kBuildFar);
+  const double quantum = ldexp(1.0, std::ilogb(range) + 1 - 23);
   for (int j = 0; j < n_rec; ++j) {
     const double two_r = 2.0 * rstar[j];
     const double r6 = two_r * two_r * two_r * two_r * two_r * two_r;
@@ -251,7 +255,7 @@ cudaError_t launch_grid_build(cudaStream_t s, const algdock_grid_desc& d, int n_
     const bool odd = j & 1;
     float hi[3], lo[3];
     for (int a = 0; a < 3; ++a) {
-      const double v = xyz[3 * (size_t)j + a] - d.origin[a];
+      const double v = std::min(std::max(xyz[3 * (size_t)j + a] - d.origin[a], -3.0 * kBuildFar), 3.0 * kBuildFar);
       hi[a] = (float)(rint(v / quantum) * quantum);
       lo[a] = (float)(v - (double)hi[a]);
     }
@@ -266,8 +270,10 @@ cudaError_t launch_grid_build(cudaStream_t s, const algdock_grid_desc& d, int n_
     (odd ? h_q[j / 2].y : h_q[j / 2].x) = (float)(q[j] / 4.0);
   }
   bool lo = false;  // whether some node coordinate is no multiple of the quantum
-  for (int i = 0; i < std::max({d.n[0], d.n[1], d.n[2]}) && !lo; ++i)
-    lo = !(rint(d.spacing * i / quantum) * quantum == d.spacing * i);
+  for (int i = 0; i < n_max && !lo; ++i) {
+    const double p = std::min(d.spacing * i, kBuildFar);
+    lo = !((double)(float)(rint(p / quantum) * quantum) == p);
+  }
   void* d_rec = nullptr;
   const size_t bytes = np * (sizeof(ReceptorPair) + sizeof(float2));
   cudaError_t e = cudaMallocAsync(&d_rec, bytes, s);
