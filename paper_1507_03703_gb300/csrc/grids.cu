@@ -14,7 +14,7 @@ namespace {
 
 constexpr int kBuildThreads = 128;
 constexpr int kBuildTile = 128;      // receptor atom pairs staged per shared-memory tile
-constexpr int kBuildNodes = 4;       // nodes per thread, spread along x
+constexpr int kBuildNodes = 4;       // nodes per thread, spread along z
 constexpr float kBuildMaxR2 = 8e37f;  // keeps the reciprocal normal and its refinement finite
 // Nodes beyond kBuildFar of the origin, whose square FP32 does not hold, and atoms beyond three times that are
 // taken to lie there: as far from all else, and hi + lo stays finite.
@@ -41,22 +41,25 @@ __device__ __forceinline__ double total2(f32x2 s, f32x2 e) {
 }
 
 // Direct sums, all in paired FP32 instructions (two receptor atoms each).  A thread takes four nodes
-// of one row, so the y and z differences are shared, and `slices` groups of a block's threads share
+// of one column, so the x and y differences are shared, and `slices` groups of a block's threads share
 // the receptor where the lattice alone would not fill the GPU.
 //
 // The differences are as exact as FP64 ones rounded to FP32: every coordinate (relative to the
 // lattice origin) is hi + lo, with hi a multiple of a power of two such that every hi within 64 A of
 // the lattice has at most 23 bits.  hi - hi is then exact, and one rounding remains, of the sum with
 // lo - lo (an error of dx counts twelve times in r^-12).  LO: the nodes have a lo part; lattices of
-// 0.25 or 0.5 A have none.  The reciprocal takes one Newton step, and the floors of the attractive
+// 0.25 or 0.5 A have none.  What dx lost in that rounding goes back into dx^2 (ex), and dz^2 comes last, as
+// in the plain sum: shared by four nodes, this costs 3.5 % and keeps the error below that of FP32 terms of
+// FP64 differences (without it, it was up to 2 % above in the attractive grid).  The reciprocal takes one Newton step, and the floors of the attractive
 // and electrostatic sums at 2 A are minima of the reciprocal powers.  The sums of thousands of terms
 // (of mixed sign in the electrostatic grid) carry their rounding errors along (acc2): four
 // instructions per channel, as good as FP64 sums of FP32 terms.
 //
-// FP32-pipe bound: 21 paired instructions per two terms, of two cycles each, 4.6 ms for the 129^3
-// lattice of a 4000-atom receptor.  Measured 7.1 ms, against 192 ms with FP64 differences and sums (6
-// FP64 operations and 6 conversions a term on a pipe of 2 lanes per clock) and IEEE divisions.  The
-// error against 64 bits is the same (3.1e-7 and 3.2e-7 in the 2-norm of the repulsive grid).
+// FP32-pipe bound: 22.5 paired instructions per two terms, of two cycles each, 4.8 ms for the 129^3
+// lattice of a 4000-atom receptor.  Measured 7.36 ms, against 192 ms with FP64 differences and sums (6
+// FP64 operations and 6 conversions a term on a pipe of 2 lanes per clock) and IEEE divisions.  Root mean
+// square of the error against 64 bits, over 36 lattices and receptors, in units of 2^-24 of a node's sum of
+// magnitudes, with those and here: repulsive 4.15, 3.87; attractive 0.960, 0.920; electrostatic 0.082, 0.076.
 template <bool LO>
 __global__ void __launch_bounds__(kBuildThreads) grid_build_kernel(
     int nx, int ny, int nz, int nq, int slices, double h, double quantum, int n_pairs,
@@ -67,24 +70,27 @@ __global__ void __launch_bounds__(kBuildThreads) grid_build_kernel(
   const int width = kBuildThreads / slices;  // threads of a slice
   const int slice = threadIdx.x / width, tid = threadIdx.x % width;
   const int64_t item = (int64_t)blockIdx.x * width + tid;
-  const int64_t n_items = (int64_t)nq * ny * nz;
+  const int64_t n_items = (int64_t)nx * ny * nq;
   const bool active = item < n_items;
-  // thread (q, j, k) of nq x ny x nz: nodes q, q + nq, q + 2 nq, q + 3 nq of row (j, k)
-  const int q = (int)(item % nq), j = (int)((item / nq) % ny), k = (int)(item / ((int64_t)nq * ny));
-  auto split = [&](int i, f32x2& hi, f32x2& lo) {
-    const double p = fmin(h * i, kBuildFar);
+  // thread (i, j, q) of nx x ny x nq: nodes q, q + nq, q + 2 nq, q + 3 nq of column (i, j)
+  const int i = (int)(item % nx), j = (int)((item / nx) % ny), q = (int)(item / ((int64_t)nx * ny));
+  auto split = [&](int node, f32x2& hi, f32x2& lo) {
+    const double p = fmin(h * node, kBuildFar);
     const float ph = (float)(rint(p / quantum) * quantum);
     const float pl = (float)(p - (double)ph);
     hi = pack2(ph, ph);
     lo = pack2(pl, pl);
   };
-  f32x2 X[kBuildNodes], Xl[kBuildNodes], Y, Yl, Z, Zl;
-#pragma unroll
-  for (int m = 0; m < kBuildNodes; ++m) split(q + m * nq, X[m], Xl[m]);
+  f32x2 X, Xl, Y, Yl, Z[kBuildNodes], Zl[kBuildNodes];
+  split(i, X, Xl);
   split(j, Y, Yl);
-  split(k, Z, Zl);
+#pragma unroll
+  for (int m = 0; m < kBuildNodes; ++m) split(q + m * nq, Z[m], Zl[m]);
   auto diff = [](f32x2 p, f32x2 pl, f32x2 a, f32x2 al) {
     return LO ? add2(sub2(p, a), sub2(pl, al)) : sub2(sub2(p, a), al);
+  };
+  auto diff_error = [](f32x2 d, f32x2 p, f32x2 pl, f32x2 a, f32x2 al) {  // exact less rounded difference
+    return LO ? add2(sub2(sub2(p, a), d), sub2(pl, al)) : sub2(sub2(sub2(p, a), d), al);
   };
   const float rmin2 = (float)(kRepulsiveMinDist * kRepulsiveMinDist);
   const float amin2_inv = (float)(1.0 / (kAttractiveMinDist * kAttractiveMinDist));
@@ -108,14 +114,15 @@ __global__ void __launch_bounds__(kBuildThreads) grid_build_kernel(
       const float2 c = s_q[t];
       const f32x2 A = pack2(R.c3.x, R.c3.y), B = pack2(R.c3.z, R.c3.w), Q = pack2(c.x, c.y);
       const f32x2 hx = pack2(R.c0.x, R.c0.y), lx = pack2(R.c1.z, R.c1.w);
+      const f32x2 dx = diff(X, Xl, hx, lx), ex = mul2(dx, diff_error(dx, X, Xl, hx, lx));
       const f32x2 dy = diff(Y, Yl, pack2(R.c0.z, R.c0.w), pack2(R.c2.x, R.c2.y));
-      const f32x2 dz = diff(Z, Zl, pack2(R.c1.x, R.c1.y), pack2(R.c2.z, R.c2.w));
-      const f32x2 yz = fma2(dy, dy, mul2(dz, dz));
+      const f32x2 hz = pack2(R.c1.x, R.c1.y), lz = pack2(R.c2.z, R.c2.w);
+      const f32x2 xy = fma2(dy, dy, fma2(dx, dx, add2(ex, ex)));
 #pragma unroll
       for (int m = 0; m < kBuildNodes; ++m) {
-        const f32x2 dx = diff(X[m], Xl[m], hx, lx);
+        const f32x2 dz = diff(Z[m], Zl[m], hz, lz);
         float ra, rb;
-        unpack2(fma2(dx, dx, yz), ra, rb);
+        unpack2(fma2(dz, dz, xy), ra, rb);
         ra = fminf(fmaxf(ra, rmin2), kBuildMaxR2);
         rb = fminf(fmaxf(rb, rmin2), kBuildMaxR2);
         const f32x2 i0 = pack2(rcp_approx(ra), rcp_approx(rb));
@@ -146,8 +153,8 @@ __global__ void __launch_bounds__(kBuildThreads) grid_build_kernel(
         e += s_sum[g * width + tid][2];
       }
     }
-    const int i = q + m * nq;
-    if (active && slice == 0 && i < nx) {
+    const int k = q + m * nq;
+    if (active && slice == 0 && k < nz) {
       const int64_t p = ((int64_t)k * ny + j) * nx + i;
       ljr[p] = (float)r;
       lja[p] = (float)(-a);
@@ -283,8 +290,8 @@ cudaError_t launch_grid_build(cudaStream_t s, const algdock_grid_desc& d, int n_
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_q, h_q.data(), np * sizeof(float2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host staging buffers are freed below
   if (e == cudaSuccess) {
-    const int nq = (d.n[0] + kBuildNodes - 1) / kBuildNodes;
-    const int64_t items = (int64_t)nq * d.n[1] * d.n[2];
+    const int nq = (d.n[2] + kBuildNodes - 1) / kBuildNodes;
+    const int64_t items = (int64_t)d.n[0] * d.n[1] * nq;
     // four threads share a node's receptor where one each would leave fewer than eight blocks per SM
     const int slices = items >= (int64_t)152 * 8 * kBuildThreads ? 1 : 4;
     const int64_t blocks = (items * slices + kBuildThreads - 1) / kBuildThreads;
