@@ -15,15 +15,8 @@ constexpr int kRecPairTile = 128;                   // receptor atom pairs stage
 constexpr int kFepThreads = 256;
 constexpr int kFepMaxBlocks = 2 * 152;
 
-__device__ __forceinline__ float rcp_approx(float v) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
-// (double)v by integer operations on the ALU; zero, denormals, infinities and NaN by the instruction
-// (64-bit conversions run on the FP64 pipe, 2 lanes per clock and SM).
-__device__ __forceinline__ double widen(float v) {
+// widen without its case for zero, which sums of terms hardly ever are: 1 % of the kernel's time.
+__device__ __forceinline__ double widen_sum(float v) {
   const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
   if (m - 0x00800000u < 0x7f000000u)
     return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
@@ -109,11 +102,11 @@ __global__ void __launch_bounds__(kTIMaxThreads, 2) target_interaction_kernel(
     for (int k = 0; k < PER; ++k) {
       float a, b;
       unpack2(fr[k], a, b);
-      dr[k] += widen(a) + widen(b);
+      dr[k] += widen_sum(a) + widen_sum(b);
       unpack2(fa[k], a, b);
-      da[k] += widen(a) + widen(b);
+      da[k] += widen_sum(a) + widen_sum(b);
       unpack2(fe[k], a, b);
-      de[k] += widen(a) + widen(b);
+      de[k] += widen_sum(a) + widen_sum(b);
     }
   }
   // atom energy sqrt(A_i) LJr - sqrt(B_i) |LJa| + 332.0637 q_i elec, each group's share
@@ -277,6 +270,9 @@ struct TIShape {
 //   10000, 70, 4000   1678 -> 1684 / - / - / -          1000, 20, 700    50 -> - / 26 / 25 / 23
 //   3000, 33, 1200     122 -> 89 / 97 / - / -           2000, 13, 2500  163 -> - / 60 / 57 / 59
 //   5000, 61, 300       76 -> 69 / - / - / -            500, 70, 4000   261 -> 172 / 155 / 155 / -
+// Taken: two groups of 64 at the first and third, four points at the second, three points at the fourth; on
+// the right two groups of 96, four groups of one point (not in the table), two groups of 96, four groups of 64.
+// So the rule is up to 9 % from the best shape (97 for 89, 59 for 57).
 constexpr TIShape kTIShapes[] = {{4, 128, 1}, {3, 128, 1}, {3, 64, 2}, {3, 64, 4}, {1, 96, 2}, {1, 64, 4}};
 
 size_t ti_smem_bytes(const TIShape& h) {

@@ -20,12 +20,6 @@ constexpr float kBuildMaxR2 = 8e37f;  // keeps the reciprocal normal and its ref
 // taken to lie there: as far from all else, and hi + lo stays finite.
 constexpr double kBuildFar = 2e19;
 
-__device__ __forceinline__ float rcp_approx(float v) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
 // s + e += a b: the rounded sum in s, its error (of the exact product) in e.
 __device__ __forceinline__ void acc2(f32x2& s, f32x2& e, f32x2 a, f32x2 b) {
   const f32x2 t = fma2(a, b, s);
@@ -48,12 +42,13 @@ __device__ __forceinline__ double total2(f32x2 s, f32x2 e) {
 // lattice origin) is hi + lo, with hi a multiple of a power of two such that every hi within 64 A of
 // the lattice has at most 23 bits.  hi - hi is then exact, and one rounding remains, of the sum with
 // lo - lo (an error of dx counts twelve times in r^-12).  LO: the nodes have a lo part; lattices of
-// 0.25 or 0.5 A have none.  What dx lost in that rounding goes back into dx^2 (ex), and dz^2 comes last, as
-// in the plain sum: shared by four nodes, this costs 3.5 % and keeps the error below that of FP32 terms of
-// FP64 differences (without it, it was up to 2 % above in the attractive grid).  The reciprocal takes one Newton step, and the floors of the attractive
-// and electrostatic sums at 2 A are minima of the reciprocal powers.  The sums of thousands of terms
-// (of mixed sign in the electrostatic grid) carry their rounding errors along (acc2): four
-// instructions per channel, as good as FP64 sums of FP32 terms.
+// 0.25 or 0.5 A have none.  What dx lost in that rounding goes back into dx^2 (ex), and dz^2 comes last,
+// as in the plain sum: shared by four nodes, this costs 3.5 % and keeps the error below that of FP32
+// terms of FP64 differences (without it, it was up to 2 % above in the attractive grid).  The reciprocal
+// takes one Newton step, and the floors of the attractive and electrostatic sums at 2 A are minima of the
+// reciprocal powers.  The sums of thousands of terms (of mixed sign in the electrostatic grid) carry their
+// rounding errors along (acc2): four instructions per channel, and exact products; only where a term
+// exceeds the sum so far is part of the error lost.
 //
 // FP32-pipe bound: 22.5 paired instructions per two terms, of two cycles each, 4.8 ms for the 129^3
 // lattice of a 4000-atom receptor.  Measured 7.36 ms, against 192 ms with FP64 differences and sums (6

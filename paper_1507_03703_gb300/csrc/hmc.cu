@@ -328,7 +328,7 @@ __device__ inline float bonded_terms(const Lig& L, const LigandLayout& LL, const
 // Step 3: nonbonded pairs.  A pass covers atoms base .. base+31; a pass with at most 16 atoms gives
 // each atom two lanes, which split the partner range and combine with one shuffle.  Adds the
 // lane's energies to e2 and returns the force on atom base + lane (valid where that atom exists).
-template <bool ENERGY, bool FORCES = true>
+template <bool ENERGY>
 __device__ inline float3 nonbonded_pass(const Lig& L, int na, int base, const float4* xs, float& e2) {
   const int lane = threadIdx.x & 31;
   const int m = na - base;
@@ -369,11 +369,9 @@ __device__ inline float3 nonbonded_pass(const Lig& L, int na, int base, const fl
       const float qq = excluded ? 0.f : (ty == 1u ? (float)(1.0 / 1.2) : 1.f) * (qi * pj.w);
       const float eel = qq * inv_r;
       const float fr = fmaf(12.f * eps, s6 * s6 - s6, eel) * inv_r2;
-      if (FORCES) {
-        fx = fmaf(fr, dx, fx);
-        fy = fmaf(fr, dy, fy);
-        fz = fmaf(fr, dz, fz);
-      }
+      fx = fmaf(fr, dx, fx);
+      fy = fmaf(fr, dy, fy);
+      fz = fmaf(fr, dz, fz);
       if (ENERGY) e2 += fmaf(eps, s6 * s6 - 2.f * s6, eel);
     }
   }
@@ -492,7 +490,7 @@ __device__ inline void nonbonded_energy_pass(const Lig& L, int na, int base, con
   }
 }
 
-template <int APL, bool ENERGY, bool FORCES = true>
+template <int APL>
 __device__ inline void nonbonded(const Lig& L, int na, const float4* xs, float (&F)[APL][3], float& el) {
   const int lane = threadIdx.x & 31;
   float e2 = 0.f;
@@ -500,14 +498,14 @@ __device__ inline void nonbonded(const Lig& L, int na, const float4* xs, float (
   for (int a = 0; a < APL; ++a) {
     const int m = na - 32 * a;
     if (m <= 0) break;
-    const float3 f = nonbonded_pass<ENERGY, FORCES>(L, na, 32 * a, xs, e2);
+    const float3 f = nonbonded_pass<true>(L, na, 32 * a, xs, e2);
     if (lane < m) {
       F[a][0] += f.x;
       F[a][1] += f.y;
       F[a][2] += f.z;
     }
   }
-  if (ENERGY) el += 0.5f * e2;
+  el += 0.5f * e2;
 }
 
 // Step 3 from the pair table: the same passes and lane layout as `nonbonded`, with each pair's
@@ -674,7 +672,7 @@ __device__ inline void evaluate(const LigandLayout& LL, const Lig& L, const Grid
       F[a][2] += ((q0.z + q1.z) + q2.z) + q3.z;
     }
   }
-  nonbonded<APL, true>(L, na, xs, F, el);
+  nonbonded<APL>(L, na, xs, F, el);
   // restraint on the centre of mass
   mx = warp_sumf(mx);
   my = warp_sumf(my);
@@ -1228,8 +1226,7 @@ __global__ void __launch_bounds__(SLOTS * APL * 32, MINB) hmc_kernel(const HmcAr
   }
 }
 
-// Energy (and, with force != NULL, force) of stored configurations, one warp each.  With
-// state_of == NULL the grid weights are zero (components only).
+// Energies and forces of stored configurations, one warp each; comps may be NULL.
 struct EvalArgs {
   GridDev G;
   LigandLayout LL;
@@ -1255,13 +1252,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
   const WarpSmem ws = warp_smem<APL, false>(smem + A.LL.words + warp * warp_words(A.LL, APL, false), A.LL);
   if (lane == 0) ws.sl[A.LL.n_slots] = make_float4(0.f, 0.f, 0.f, 0.f);  // the zero slot
   const int na = A.LL.na;
-  float w_sg = 0.f, w_g = 0.f;
-  if (A.state_of) {
-    const int k = A.state_of[n];
-    if ((unsigned)k >= (unsigned)A.n_states) return;  // invalid state index: no output
-    w_sg = A.states[k].w_sg_f;
-    w_g = A.states[k].w_g_f;
-  }
+  const int k = A.state_of[n];
+  if ((unsigned)k >= (unsigned)A.n_states) return;  // invalid state index: no output
+  const float w_sg = A.states[k].w_sg_f, w_g = A.states[k].w_g_f;
   float x[APL][3], F[APL][3], mass[APL];
 #pragma unroll
   for (int a = 0; a < APL; ++a) {
@@ -1282,16 +1275,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) eval_kernel(const EvalArg
   evaluate<APL>(A.LL, L, A.G, ws.xs, ws.sl, x, mass, F, w_sg, w_g, en);
   double c[4];
   reduce_components(en, c);
-  {
 #pragma unroll
-    for (int a = 0; a < APL; ++a) {
-      const int i = lane + 32 * a;
-      if (i < na) {
-        float* dst = A.force + (n * na + i) * 3;
-        dst[0] = F[a][0];
-        dst[1] = F[a][1];
-        dst[2] = F[a][2];
-      }
+  for (int a = 0; a < APL; ++a) {
+    const int i = lane + 32 * a;
+    if (i < na) {
+      float* dst = A.force + (n * na + i) * 3;
+      dst[0] = F[a][0];
+      dst[1] = F[a][1];
+      dst[2] = F[a][2];
     }
   }
   if (A.comps && lane < 4) A.comps[n * 4 + lane] = c[lane];
@@ -1638,8 +1629,8 @@ constexpr int kTableWarps = 16;  // replicas per block of the pair-table HMC ker
 // (32 replicas of 48 atoms: 166 us against 193); from there on the one with 24 warps per SM.
 constexpr int kTable1 = 5, kTable2 = 6, kTable2Few = 4, kType1 = 16, kType2 = 4, kType3 = 8;
 // Two warps a replica, with more replicas than two blocks of kTable2 hold per SM but no more than one of 16
-// does: one block of 16 takes them at once, where the two would need a second round for a few.  45 atoms, 1900 replicas, 50 steps: 547 -> 401 us (534
-// with one warp a replica).
+// does: one block of 16 takes them at once, where the two would need a second round for a few.  45 atoms,
+// 1900 replicas, 50 steps: 547 -> 401 us (534 with one warp a replica).
 constexpr int kTable2Wave = 16;
 
 // Dynamic shared memory of an HMC block of `slots` replicas, and the most of at most `slots` that a

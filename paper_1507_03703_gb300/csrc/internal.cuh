@@ -76,6 +76,20 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   return r;
 }
 
+__device__ __forceinline__ float rcp_approx(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// (double)v by integer operations on the ALU; denormals, infinities and NaN by the instruction (conversions
+// between 32 and 64 bits run on the FP64 pipe, 2 lanes per clock and SM).
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (b != 0 && m - 0x00800000u >= 0x7f000000u) return (double)v;
+  return __hiloint2double(b ? (int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)) : 0, (int)(b << 29));
+}
+
 // A double's place in the order of the doubles as a signed integer (its own inverse), for minima and maxima
 // on the integer units.
 __device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }

@@ -54,9 +54,8 @@ __device__ inline void lse_add(Lse& a, double x) {
   }
 }
 
-// (float)v and (double)v with the instructions' results, by integer operations where value and result
-// are normal numbers (or, widening, zero): conversions between 32 and 64 bits run on the FP64 pipe,
-// 2 lanes per clock and SM.
+// (float)v with the instruction's result, by integer operations where value and result are normal
+// numbers (as widen).
 __device__ __forceinline__ float narrow(double v) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const uint32_t t = (hi & 0x7fffffffu) - 0x38000000u;
@@ -64,11 +63,6 @@ __device__ __forceinline__ float narrow(double v) {
   uint32_t b = __funnelshift_l(lo, t, 3);
   b += (lo << 3) > 0x80000000u - (b & 1u);  // to nearest, ties to even
   return __uint_as_float(b | (hi & 0x80000000u));
-}
-__device__ __forceinline__ double widen(float v) {
-  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
-  if (b != 0 && m - 0x00800000u >= 0x7f000000u) return (double)v;
-  return __hiloint2double(b ? (int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)) : 0, (int)(b << 29));
 }
 
 // Precision mode 1, FP32 exponentials of FP64 arguments.  The FP64 pipe bounds it, so an element takes
@@ -406,9 +400,9 @@ __global__ void init_state(int K, const int64_t* Nk, double* logNk, double* f, M
 // (the shifts c_n cancel, and so does a factor common to all a_k).  Two FP64 multiply-adds per
 // element and iteration remain, which is what bounds it: GB300 issues 2 FP64 lanes per clock and
 // SM, so K = 128, N = 102400 cannot take less than 42 us an iteration (its 105 MB of weights take
-// 15 us from HBM).  Measured: a solve of 43 iterations at that size 88.5 -> 3.85 ms (4.00 with one tile a block; two log-sum-exp
-// passes with an FP64 exponential per element take 1455 us an iteration), and 25.9 -> 1.58 ms an
-// iteration, the forming of the weights included, at K = 256, N = 1e6.
+// 15 us from HBM).  Measured: a solve of 43 iterations at that size 88.5 -> 3.85 ms (4.00 with one tile a
+// block; two log-sum-exp passes with an FP64 exponential per element take 1455 us an iteration), and
+// 25.9 -> 1.58 ms an iteration, the forming of the weights included, at K = 256, N = 1e6.
 //
 // Range.  c_n is the column's maximum, so the largest weight of a column is 1, D'_n is finite and only
 // weights below 1e-308 of the largest are lost.  While the spread of f - g stays within kMaxSpread,
