@@ -752,9 +752,11 @@ algdock_status build_ligand(algdock_ctx* c, const algdock_ligand* L, const algdo
       const int i = p % na, j = (i + 1 + p / na) % na;
       const int ty = ptype[(size_t)j * na + i];
       const double s_lj = ty == 1 ? 0.5 : 1.0, s_el = ty == 1 ? 1.0 / 1.2 : 1.0;
-      const double R = L->rstar[i] + L->rstar[j];
+      // (R*_i + R*_j)^2 rounded once; R + e is the exact sum
+      const double ri = L->rstar[i], rj = L->rstar[j], R = ri + rj, t = R - ri;
+      const double e = (ri - (R - t)) + (rj - t);
       double* q = &d[G.off_pair + p];
-      q[0] = ty == 2 ? -1.0 : R * R;
+      q[0] = ty == 2 ? -1.0 : fma(R, R, 2.0 * R * e);
       q[n_pairs] = ty == 2 ? 0.0 : 12.0 * s_lj * sqrt(L->eps[i]) * sqrt(L->eps[j]);
       q[2 * n_pairs] = ty == 2 ? 0.0 : s_el * kCoulomb * L->charge[i] * L->charge[j];
     }

@@ -15,8 +15,11 @@
 //      one d at a time);
 //   3. per atom: the five interpolated channels, edge differences along x, then y, then z.
 // Reciprocal square roots take the place of square roots and divisions (the pair loop's from an
-// FP32 seed by one third-order step), torsions the multiple-angle polynomials of cos(phi), sin(phi).
-// 8192 configurations of 48 atoms take 1.25 ms with the FP64 pipe 86 % busy.  With one thread per
+// FP32 seed by one third-order step), torsions the multiple-angle polynomials of cos(phi), sin(phi).  Where a
+// rounding would count many times (a bond's length, R^2/r^2) one more step takes it out: the forces of bonds
+// and of pairs are as close to extended precision as with square roots and divisions (1.5e-15 and 6.5e-16
+// relative), their energies closer.
+// 8192 configurations of 48 atoms take 1.22 ms.  With one thread per
 // configuration (64 blocks, square roots, divisions, atan2, sincos, and forces added in global
 // memory) they took 5.67 ms.  Two configurations per block or four make no difference at that size;
 // two leave more blocks to a small one.
@@ -45,12 +48,21 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-// 1 / sqrt(v) from an FP32 seed y (error e = 1 - v y^2 about 2^-22) by the third-order step
-// y (1 + e/2 + 3 e^2/8), whose error 5 e^3/16 is below FP64 rounding.
-__device__ inline double rsqrt_step(double v) {
-  const double y = (double)rsqrtf((float)v);
-  const double e = fma(-(v * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
+// 1 / sqrt(v) and 1 / v from an FP32 seed y (error e = 1 - v y^2 about 2^-22, y^2 exact): y (1 + e/2 + 3 e^2/8)
+// and y^2 (1 + e + e^2), whose errors 5 e^3/16 and e^3 are below FP64 rounding.  (The square of the root
+// would carry its rounding twice, and r^-12 that twelve times.)
+__device__ inline void reciprocals(double v, double& inv_root, double& inv) {
+  const double y = (double)rsqrtf((float)v), y2 = y * y;
+  const double e = fma(-v, y2, 1.0);
+  inv_root = fma(y * e, fma(0.375, e, 0.5), y);
+  inv = fma(y2, fma(e, e, e), y2);
+}
+
+// sqrt(v) from y = 1 / sqrt(v) by a Newton step: within 0.51 ulp, where v y is within 1.5 (a bond's stretch is a
+// few hundredths of its length).
+__device__ inline double sqrt_step(double v, double y) {
+  const double r = v * y;
+  return v > 0.0 ? fma(0.5 * y, fma(-r, r, v), r) : v;
 }
 
 // A warp's shared memory: positions [3][na], forces [3][na], bonded slots [3][n_slots + 1] (the last
@@ -184,7 +196,7 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
     const int i = (int)b[0], j = (int)b[1];
     const V3 d = W.pos(i) - W.pos(j);
     const double r2 = dot3(d, d), inv_r = rsqrt(r2);
-    const double dr = (r2 > 0.0 ? r2 * inv_r : r2) - b[3];
+    const double dr = sqrt_step(r2, inv_r) - b[3];
     e_lig += b[2] * dr * dr;
     if (FORCES) {
       const V3 f = (-2.0 * b[2] * dr * inv_r) * d;
@@ -273,33 +285,38 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
       const int p = p0 + lane;
       const bool on = lane < width && p < n_pairs;
       int i = 0, j = 0;
-      V3 f{0.0, 0.0, 0.0};
+      V3 dx{0.0, 0.0, 0.0};
+      double fr = 0.0;  // -dE/dr / r
       if (on) {
         const int d = p / na;
         i = p - d * na;
         j = i + d + 1;
         j = j >= na ? j - na : j;
         const double R2 = __ldg(T + p), eps12 = __ldg(T + n_pairs + p), qq = __ldg(T + 2 * n_pairs + p);
-        const V3 dx = W.pos(i) - W.pos(j);
-        double y = rsqrt_step(dot3(dx, dx));
-        y = __double2hiint(R2) < 0 ? 0.0 : y;
-        const double y2 = y * y, s2 = R2 * y2, s6 = s2 * s2 * s2;
-        const double A12 = eps12 * s6, eel = qq * y;
+        dx = W.pos(i) - W.pos(j);
+        const double r2 = dot3(dx, dx);
+        double y, y2;
+        reciprocals(r2, y, y2);
+        if (__double2hiint(R2) < 0) y = y2 = 0.0;
+        // R^2 / r^2 rounded once, by the remainder of the product with the rounded reciprocal
+        double s2 = R2 * y2;
+        s2 = fma(fma(-s2, r2, R2), y2, s2);
+        const double s6 = s2 * s2 * s2, A12 = eps12 * s6, eel = qq * y;
         e12 = fma(A12, s6 - 2.0, e12);
         e_el += eel;
-        if (FORCES) f = (fma(A12, s6 - 1.0, eel) * y2) * dx;  // -dE/dr / r times the difference
+        if (FORCES) fr = fma(A12, s6 - 1.0, eel) * y2;
       }
       if (FORCES) {
         if (on) {
-          W.f[i] += f.x;
-          W.f[na + i] += f.y;
-          W.f[2 * na + i] += f.z;
+          W.f[i] = fma(fr, dx.x, W.f[i]);
+          W.f[na + i] = fma(fr, dx.y, W.f[na + i]);
+          W.f[2 * na + i] = fma(fr, dx.z, W.f[2 * na + i]);
         }
         __syncwarp();
         if (on) {
-          W.f[j] -= f.x;
-          W.f[na + j] -= f.y;
-          W.f[2 * na + j] -= f.z;
+          W.f[j] = fma(-fr, dx.x, W.f[j]);
+          W.f[na + j] = fma(-fr, dx.y, W.f[na + j]);
+          W.f[2 * na + j] = fma(-fr, dx.z, W.f[2 * na + j]);
         }
         __syncwarp();
       }
