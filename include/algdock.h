@@ -178,7 +178,7 @@ algdock_status algdock_grids_load(algdock_ctx* ctx, const algdock_grid_desc* des
  * The FP64 arm of the precision study (no counterpart in the paper): the same energy function
  * as algdock_energy_force with every operation in FP64, on FP64 lattices and the ligand's FP64
  * parameters (kept by algdock_ligand_load).  One warp per configuration, bound by the GPU's FP64
- * rate (2 lanes per clock and SM): about 16 times the FP32 path's time. */
+ * rate (2 lanes per clock and SM): about 18 times the FP32 path's time. */
 
 /* FP64 lattices from raw grids (host or device double [nz][ny][nx]), derived as algdock_grids_load
  * does (4th root of the capped repulsive grid, tanh-capped soft grids) but kept in FP64.  They

@@ -23,8 +23,8 @@
 // and third pass, its long chain of stages and 38 instructions a pair without the pair table set the
 // pace.  Teams keep 24 warps per SM in two blocks, run stages 2 to 4 beside each other and spread a
 // few replicas over all SMs.  Measured (trials of 50 steps, bit-identical): 48 atoms, 8192 replicas
-// 1852 -> 1592 us; 83 atoms, 1152 replicas 1100 -> 673 us; 60 atoms (no pair table), 4096 replicas
-// 1924 -> 1332 us; 27 atoms, 8192 replicas 1025 -> 825 us; 16 replicas of 20 atoms, 20 steps, 96 -> 62 us.
+// 1852 -> 1596 us; 83 atoms, 1152 replicas 1100 -> 674 us; 60 atoms (no pair table), 4096 replicas
+// 1924 -> 1334 us; 27 atoms, 8192 replicas 1025 -> 826 us; 16 replicas of 20 atoms, 20 steps, 96 -> 62 us.
 // Every force is accumulated by one lane in a fixed order (no atomics), so results are
 // deterministic.
 #include <math.h>
@@ -1153,7 +1153,7 @@ __device__ __forceinline__ void hmc_trial(const HmcArgs& A, const LigandLayout& 
 
 // A team of APL warps per replica, one atom per lane; a block holds the ligand's tables and up to
 // SLOTS replicas (blockDim.x / (32 APL) of them, fewer where their shared memory does not fit).
-// MINB blocks per SM.  At 48 atoms two blocks of 6 replicas take 1592 us, one of 12 1685, of 10 1770, of
+// MINB blocks per SM.  At 48 atoms two blocks of 6 replicas take 1596 us, one of 12 1685, of 10 1770, of
 // 8 1769, of 16 (64 registers) 1810: more warps wait on the shared-memory pipe (70 % busy) instead.
 // TABLE: the pair table is staged with the blob.
 // BATCH: the block's ligand and replicas come from its work item (a run of consecutive replicas of

@@ -453,7 +453,7 @@ struct CopyTask {
 };
 cudaError_t copy_group(cudaStream_t s, int n, const CopyTask* t);
 // Rows from which the learned network's gradient and forward pass run on tcgen05 (with tc_err set):
-// measured against the mma.sync kernels on one GB300, the gradient takes 139 us at 4096 rows (with an
+// measured against the mma.sync kernels on one GB300, the gradient takes 142 us at 4096 rows (with an
 // Adam step) against about 255 and 1075 at 65536 against 2350 (before its launches were grouped); the
 // forward ties at 8192 and wins from 16384 (1.6x at 65536).  The two paths round differently, so the
 // lines stay where they were set.

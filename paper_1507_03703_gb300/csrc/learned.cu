@@ -1353,7 +1353,7 @@ cudaError_t learned_grad(cudaStream_t s, const float* params, const uint16_t* wb
     // Thirteen launches, each a few microseconds of latency at 4096 rows: the hidden activations and the
     // input gradients leave their products transposed as well, and the four layers' weight
     // products, column sums and slice sums share a launch each.  A gradient and an Adam step at 4096
-    // rows: 139 us, 244 with 46 launches (a transpose per operand, four of each closing sum).
+    // rows: 142 us, 246 with 46 launches (a transpose per operand, four of each closing sum).
     const int np = (int)pad8(N);
     char* q = (char*)Wp + packed_bytes();
     auto take = [&](size_t elems) {
