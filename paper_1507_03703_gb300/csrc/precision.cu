@@ -19,7 +19,7 @@
 // rounding would count many times (a bond's length, R^2/r^2) one more step takes it out: the forces of bonds
 // and of pairs are as close to extended precision as with square roots and divisions (1.5e-15 and 6.5e-16
 // relative), their energies closer.
-// 8192 configurations of 48 atoms take 1.22 ms.  With one thread per
+// 8192 configurations of 48 atoms take 1.23 ms.  With one thread per
 // configuration (64 blocks, square roots, divisions, atan2, sincos, and forces added in global
 // memory) they took 5.67 ms.  Two configurations per block or four make no difference at that size;
 // two leave more blocks to a small one.
@@ -59,10 +59,30 @@ __device__ inline void reciprocals(double v, double& inv_root, double& inv) {
 }
 
 // sqrt(v) from y = 1 / sqrt(v) by a Newton step: within 0.51 ulp, where v y is within 1.5 (a bond's stretch is a
-// few hundredths of its length).
+// few hundredths of its length).  Zero and infinity are their own roots.
 __device__ inline double sqrt_step(double v, double y) {
   const double r = v * y;
-  return v > 0.0 ? fma(0.5 * y, fma(-r, r, v), r) : v;
+  return v > 0.0 && y > 0.0 ? fma(0.5 * y, fma(-r, r, v), r) : v;
+}
+
+// (c, s) / |(c, s)| where the sum of squares is zero, overflows or is not a number: (1, 0) for (0, 0), and the
+// limit of the direction where a part is infinite, as the angle atan2(s, c) has it.
+__device__ __noinline__ void direction(double& c, double& s) {
+  double m = fmax(fabs(c), fabs(s));
+  if (isinf(m)) {
+    c = isinf(c) ? copysign(1.0, c) : 0.0 * c;
+    s = isinf(s) ? copysign(1.0, s) : 0.0 * s;
+    m = 1.0;
+  }
+  if (m > 0.0) {
+    c /= m;
+    s /= m;
+    m = rsqrt(c * c + s * s);
+    c *= m;
+    s *= m;
+  } else if (c == 0.0) {
+    c = 1.0;
+  }
 }
 
 // A warp's shared memory: positions [3][na], forces [3][na], bonded slots [3][n_slots + 1] (the last
@@ -232,11 +252,16 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
     const V3 pj = W.pos(j), pk = W.pos(k);
     const V3 b1 = pj - W.pos(i), b2 = pk - pj, b3 = W.pos(l) - pk;
     const V3 n1 = cross3(b1, b2), n2 = cross3(b2, b3);
-    const double lb22 = dot3(b2, b2), inv_lb2 = rsqrt(lb22), lb2 = lb22 > 0.0 ? lb22 * inv_lb2 : lb22;
+    const double lb22 = dot3(b2, b2), inv_lb2 = rsqrt(lb22), lb2 = sqrt_step(lb22, inv_lb2);
     // (cos phi, sin phi) is (n1.n2, |b2| b1.n2) normalised; collinear bonds have phi = 0
     const double cx = dot3(n1, n2), sx = lb2 * dot3(b1, n2);
     const double h2 = cx * cx + sx * sx, inv_h = rsqrt(h2);
-    const double c1 = h2 > 0.0 ? cx * inv_h : 1.0, s1 = h2 > 0.0 ? sx * inv_h : 0.0;
+    double c1 = cx * inv_h, s1 = sx * inv_h;
+    if (!(h2 > 0.0 && inv_h > 0.0)) {
+      c1 = cx;
+      s1 = sx;
+      direction(c1, s1);
+    }
     const double c2 = 2.0 * c1 * c1 - 1.0, s2 = 2.0 * s1 * c1;
     const double c3 = c1 * (2.0 * c2 - 1.0), s3 = s1 * (2.0 * c2 + 1.0);
     const double *V = q + 4, *cg = q + 7, *sg = q + 10;
@@ -287,6 +312,7 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
       int i = 0, j = 0;
       V3 dx{0.0, 0.0, 0.0};
       double fr = 0.0;  // -dE/dr / r
+      bool pair = false;
       if (on) {
         const int d = p / na;
         i = p - d * na;
@@ -294,10 +320,12 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
         j = j >= na ? j - na : j;
         const double R2 = __ldg(T + p), eps12 = __ldg(T + n_pairs + p), qq = __ldg(T + 2 * n_pairs + p);
         dx = W.pos(i) - W.pos(j);
-        const double r2 = dot3(dx, dx);
-        double y, y2;
+        double r2 = dot3(dx, dx), y, y2;
+        pair = __double2hiint(R2) >= 0;
+        const bool none = !pair || __double2hiint(r2) == 0x7ff00000;  // excluded, or infinitely far apart
+        r2 = none ? 1.0 : r2;
         reciprocals(r2, y, y2);
-        if (__double2hiint(R2) < 0) y = y2 = 0.0;
+        if (none) y = y2 = 0.0;
         // R^2 / r^2 rounded once, by the remainder of the product with the rounded reciprocal
         double s2 = R2 * y2;
         s2 = fma(fma(-s2, r2, R2), y2, s2);
@@ -307,13 +335,13 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
         if (FORCES) fr = fma(A12, s6 - 1.0, eel) * y2;
       }
       if (FORCES) {
-        if (on) {
+        if (pair) {
           W.f[i] = fma(fr, dx.x, W.f[i]);
           W.f[na + i] = fma(fr, dx.y, W.f[na + i]);
           W.f[2 * na + i] = fma(fr, dx.z, W.f[2 * na + i]);
         }
         __syncwarp();
-        if (on) {
+        if (pair) {
           W.f[j] = fma(-fr, dx.x, W.f[j]);
           W.f[na + j] = fma(-fr, dx.y, W.f[na + j]);
           W.f[2 * na + j] = fma(-fr, dx.z, W.f[2 * na + j]);
@@ -379,7 +407,8 @@ __global__ void __launch_bounds__(kWarps64 * 32) eval64_kernel(const Eval64Args 
     psi_sg += v;
     if (FORCES) {
       const V3 f = (-w_g) * dg + (-w_sg) * dsg;
-      V3 s = V3{W.f[i], W.f[na + i], W.f[2 * na + i]} + (c_rest * m) * dc;
+      V3 s = V3{W.f[i], W.f[na + i], W.f[2 * na + i]};
+      if (c_rest != 0.0) s = s + (c_rest * m) * dc;
       if (A.slots) {
         const uint2 p = __ldg((const uint2*)(A.blob + A.LL.off_gp) + i);
         s = s + (W.slot(p.x & 0xffffu) + W.slot(p.x >> 16) + W.slot(p.y & 0xffffu) + W.slot(p.y >> 16));
